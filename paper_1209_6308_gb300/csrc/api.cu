@@ -180,7 +180,7 @@ tc_status init_graph(tc_graph* g, uint32_t n, const tc_options* opt) {
     Opts check;
     TC_TRY(resolve_opts(opt, nullptr, &check));
     g->s.opts = merge_opts(opt, nullptr);
-    TC_TRY(g->s.ctr.alloc_persistent(sizeof(uint32_t) * 4));
+    TC_TRY(g->s.ctr.alloc_persistent(sizeof(uint32_t) * 8));
     TC_TRY(g->s.acc.alloc_persistent(sizeof(unsigned long long) * 16));
     TC_CUDA(cudaMallocHost(&g->s.h_counts, sizeof(unsigned long long) * 16));
     return TC_OK;
@@ -447,7 +447,7 @@ tc_status tc_census_shard(tc_graph* g, void* stream, const tc_options* opt, uint
     const uint32_t i0 = b[2 * rank], i1 = b[2 * rank + 2];
     const uint32_t v0 = b[2 * rank + 1], v1 = b[2 * rank + 3];
     TC_CUDA(cudaMemsetAsync(d_out16, 0, sizeof(uint64_t) * 16, st));
-    return census_enqueue_range(g->s, o, p->items.as<Item>() + i0, i1 - i0, p->warp_begin + v0, p->warp_begin + v1, st,
+    return census_enqueue_range(g->s, o, *p, i0, i1 - i0, p->warp_begin + v0, p->warp_begin + v1, st,
                                 reinterpret_cast<unsigned long long*>(d_out16));
 }
 

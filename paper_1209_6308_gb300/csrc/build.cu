@@ -137,16 +137,17 @@ __global__ void k_up(const uint64_t* off, const uint32_t* adj, uint32_t n, uint3
 
 // stats[3] sum deg^2, stats[4] sum over upper pairs of deg(v), stats[5] max degree,
 // stats[7] vertices with deg > 0, stats[10] sum of up (up - 1) / 2 (the entries the triangle form
-// walks: for every upper pair (b, c), the neighbours of c below b)
+// walks: for every upper pair (b, c), the neighbours of c below b), stats[11] vertices with deg > kHubDeg
 __global__ void k_graph_sums(const uint64_t* off, const uint32_t* adj, const uint32_t* up, uint32_t n,
                              unsigned long long* stats) {
     unsigned long long d2 = 0, dv = 0, tw = 0;
-    uint32_t mx = 0, act = 0;
+    uint32_t mx = 0, act = 0, hub = 0;
     for (uint64_t x = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; x < n; x += (uint64_t)gridDim.x * blockDim.x) {
         uint64_t d = off[x + 1] - off[x];
         d2 += d * d;
         mx = max(mx, (uint32_t)d);
         act += (d > 0);
+        hub += (d > kHubDeg);
         // x is the v of every pair (u, x) with u < x: the first up[x] neighbours
         dv += (unsigned long long)up[x] * d;
         tw += (unsigned long long)up[x] * (up[x] ? up[x] - 1ull : 0ull) / 2ull;
@@ -157,9 +158,11 @@ __global__ void k_graph_sums(const uint64_t* off, const uint32_t* adj, const uin
         tw += __shfl_xor_sync(0xffffffffu, tw, o);
         mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
         act += __shfl_xor_sync(0xffffffffu, act, o);
+        hub += __shfl_xor_sync(0xffffffffu, hub, o);
     }
     if ((threadIdx.x & 31) == 0) {
         if (act) atomicAdd(&stats[7], (unsigned long long)act);
+        if (hub) atomicAdd(&stats[11], (unsigned long long)hub);
         atomicAdd(&stats[3], d2);
         atomicAdd(&stats[4], dv);
         atomicAdd(&stats[10], tw);
@@ -436,7 +439,7 @@ tc_status finish_graph(GraphStore& g, uint64_t E, int B, uint64_t* ukey, uint32_
     kp = ek.as<uint64_t>();
     tp = etmp.as<uint64_t>();
     TC_TRY(radix_sort_u64(&kp, &tp, total, 2, 2 * B + 2, st));
-    TC_TRY(g.adj.alloc_persistent(sizeof(uint32_t) * (total ? total : 1)));
+    TC_TRY(g.adj.alloc_persistent(sizeof(uint32_t) * (total + 4)));   // read in aligned blocks of four
     if (total) {
         k_adj_from_entries<<<grid_for(total, kB, 1u << 16), kB, 0, st>>>(kp, total, B, g.adj.as<uint32_t>());
         TC_LAUNCH("k_adj_from_entries");
@@ -489,10 +492,11 @@ tc_status finish_graph(GraphStore& g, uint64_t E, int B, uint64_t* ukey, uint32_
             TC_LAUNCH("k_pair_rp_long");
         }
     }
-    unsigned long long hs[11];
+    unsigned long long hs[12];
     TC_CUDA(cudaMemcpyAsync(hs, stats.p, sizeof(hs), cudaMemcpyDeviceToHost, st));
     TC_CUDA(cudaStreamSynchronize(st));
     g.sum_tri_walk = hs[10];
+    g.n_hub = (uint32_t)hs[11];
     g.sum_walk = hs[8];
     g.sum_walk_map = hs[9];
     g.e_sym = E;
@@ -564,8 +568,8 @@ tc_status build_from_arcs(GraphStore& g, uint64_t m, const uint32_t* d_src, cons
     const int B = bits_for(n);
     if (m >= (1ull << 32)) return fail(TC_ERR_RANGE, "more than 2^32-1 arcs");
     DevBuf stats, keys, tmp;
-    TC_TRY(stats.alloc(sizeof(unsigned long long) * 11, st));
-    TC_CUDA(cudaMemsetAsync(stats.p, 0, sizeof(unsigned long long) * 11, st));
+    TC_TRY(stats.alloc(sizeof(unsigned long long) * 12, st));
+    TC_CUDA(cudaMemsetAsync(stats.p, 0, sizeof(unsigned long long) * 12, st));
     TC_TRY(keys.alloc(sizeof(uint64_t) * (m ? m : 1), st));
     TC_TRY(tmp.alloc(sizeof(uint64_t) * (m ? m : 1), st));
     if (m) {
@@ -596,8 +600,8 @@ tc_status build_from_sorted_arcs(GraphStore& g, const uint64_t* d_keys, uint64_t
     const int B = bits_for(g.n);
     if (m >= (1ull << 32)) return fail(TC_ERR_RANGE, "more than 2^32-1 arcs");
     DevBuf stats, ukey, udir;
-    TC_TRY(stats.alloc(sizeof(unsigned long long) * 11, st));
-    TC_CUDA(cudaMemsetAsync(stats.p, 0, sizeof(unsigned long long) * 11, st));
+    TC_TRY(stats.alloc(sizeof(unsigned long long) * 12, st));
+    TC_CUDA(cudaMemsetAsync(stats.p, 0, sizeof(unsigned long long) * 12, st));
     uint32_t E = 0;
     TC_TRY(pairs_from_sorted(d_keys, m, ukey, udir, E, st));
     TC_TRY(graph_from_pairs(g, B, E, ukey, udir, stats, st));
@@ -616,8 +620,8 @@ tc_status build_from_csr(GraphStore& g, const uint64_t* d_off, const uint32_t* d
     if (total_h & 1) return fail(TC_ERR_ARG, "CSR is not symmetric (odd number of entries)");
     if (total_h >= (1ull << 32)) return fail(TC_ERR_RANGE, "more than 2^32-1 CSR entries");
     DevBuf stats;
-    TC_TRY(stats.alloc(sizeof(unsigned long long) * 11, st));
-    TC_CUDA(cudaMemsetAsync(stats.p, 0, sizeof(unsigned long long) * 11, st));
+    TC_TRY(stats.alloc(sizeof(unsigned long long) * 12, st));
+    TC_CUDA(cudaMemsetAsync(stats.p, 0, sizeof(unsigned long long) * 12, st));
     const unsigned gridN = grid_for(n, kB, 1u << 16);
     k_check_csr<<<gridN, kB, 0, st>>>(d_off, d_adj, n, total_h, stats.as<unsigned long long>());
     TC_LAUNCH("k_check_csr");

@@ -996,6 +996,21 @@ tc_status prepare_device(cudaStream_t st, int algo, size_t smem) {
 
 }  // namespace
 
+namespace {
+// split[t] = the first item (they ascend by u) with u >= (t ? u1 : u0)
+__global__ void k_item_splits(const Item* __restrict__ items, uint32_t n, uint32_t u0, uint32_t u1, uint32_t* split) {
+    if (threadIdx.x > 1) return;
+    const uint32_t u = threadIdx.x ? u1 : u0;
+    uint32_t lo = 0, hi = n;
+    while (lo < hi) {
+        const uint32_t mid = (lo + hi) >> 1;
+        if (items[mid].u < u) lo = mid + 1;
+        else hi = mid;
+    }
+    split[threadIdx.x] = lo;
+}
+}  // namespace
+
 tc_status get_plan(GraphStore& g, const Opts& o, cudaStream_t st, Plan** out) {
     for (auto& p : g.plans)
         if (p.valid && p.key == o) { *out = &p; return TC_OK; }
@@ -1069,6 +1084,15 @@ tc_status get_plan(GraphStore& g, const Opts& o, cudaStream_t st, Plan** out) {
         if (p.n_items) {
             k_plan_items<true><<<tgrid, 256, 0, st>>>(gd, pa, pos.as<uint32_t>(), nullptr, p.items.as<Item>());
             TC_LAUNCH("k_plan_items (emit)");
+            p.split[0] = p.split[1] = 0;
+            if (o.algo == TC_ALGO_TRIANGLE && walk16_takes(g)) {
+                DevBuf sp;
+                TC_TRY(sp.alloc(sizeof(p.split), st));
+                k_item_splits<<<1, 32, 0, st>>>(p.items.as<Item>(), p.n_items, std::min(kTableFrom, g.n_hub), g.n_hub,
+                                                sp.as<uint32_t>());
+                TC_LAUNCH("k_item_splits");
+                TC_CUDA(cudaMemcpyAsync(p.split, sp.p, sizeof(p.split), cudaMemcpyDeviceToHost, st));
+            }
         }
         TC_CUDA(cudaStreamSynchronize(st));
     }
@@ -1221,16 +1245,16 @@ tc_status plan_shards(GraphStore& g, const Opts& o, Plan& p, uint32_t world, cud
 
 tc_status census_enqueue(GraphStore& g, const Opts& o, const Plan& p, cudaStream_t st, unsigned long long* d_out16,
                          unsigned long long* d_vcost, unsigned long long* d_phase) {
-    return census_enqueue_range(g, o, p.items.as<Item>(), p.n_items, p.warp_begin, p.warp_end, st, d_out16, d_vcost,
+    return census_enqueue_range(g, o, p, 0u, p.n_items, p.warp_begin, p.warp_end, st, d_out16, d_vcost,
                                 d_phase);
 }
 
-tc_status census_enqueue_range(GraphStore& g, const Opts& o, const Item* items, uint32_t n_items, uint32_t warp_begin,
-                               uint32_t warp_end, cudaStream_t st, unsigned long long* d_out16,
+tc_status census_enqueue_range(GraphStore& g, const Opts& o, const Plan& p, uint32_t item0, uint32_t n_items,
+                               uint32_t warp_begin, uint32_t warp_end, cudaStream_t st, unsigned long long* d_out16,
                                unsigned long long* d_vcost, unsigned long long* d_phase) {
     if (g.e_sym == 0) return TC_OK;
     if (o.algo == TC_ALGO_TRIANGLE)
-        return triangle_census_enqueue(g, o, items, n_items, warp_begin, warp_end, st, d_out16, d_vcost, d_phase);
+        return triangle_census_enqueue(g, o, p, item0, n_items, warp_begin, warp_end, st, d_out16, d_vcost, d_phase);
     const bool vt = g.vs.p != nullptr;
     const bool map = census_map(g, o);
     const size_t smem = census_smem(o.algo, o.chunk, map);
@@ -1238,7 +1262,7 @@ tc_status census_enqueue_range(GraphStore& g, const Opts& o, const Item* items, 
     TC_CUDA(cudaMemsetAsync(g.ctr.p, 0, sizeof(uint32_t) * 4, st));
     Params P;
     P.g = g.dev();
-    P.items = items;
+    P.items = p.items.as<Item>() + item0;
     P.n_items = n_items;
     P.warp_begin = warp_begin;
     P.warp_end = warp_end;

@@ -48,6 +48,9 @@ struct Plan {
     DevBuf items;
     uint32_t n_items = 0;
     uint32_t warp_begin = 0, warp_end = 0;
+    // items before split[0] are of vertices below kTableFrom, before split[1] of vertices with degree
+    // above kHubDeg (triangle form: walk16.cu)
+    uint32_t split[2] = {0, 0};
     // shards of the plan's work for shard_world ranks (plan_shards): rank r runs items
     // [shard_bounds[2r], shard_bounds[2r+2]) and warp-tier vertices warp_begin +
     // [shard_bounds[2r+1], shard_bounds[2r+3]); 0 = not computed
@@ -60,9 +63,11 @@ struct GraphStore {
     uint64_t arcs = 0, e_sym = 0, mutual = 0, loops = 0, dups = 0, sum_d2 = 0, sum_dv_upper = 0, sum_walk = 0;
     uint64_t sum_walk_map = 0;   // walked entries with ids below kMapIdsSuffix
     uint64_t sum_tri_walk = 0;   // sum of up (up - 1) / 2: the entries the triangle form walks
+    uint32_t n_hub = 0;          // vertices with deg > kHubDeg: ids [0, n_hub)
     DevBuf off, adj, up, new_of_old;
     DevBuf ub, rp, vs, us;   // per upper pair tables (see GraphDev)
-    DevBuf ctr;        // census work counters (uint32 x 4)
+    DevBuf rec, blk16;   // 16-bit lower lists (see GraphDev): rec holds rec, rec2 and n16 of the active vertices
+    DevBuf ctr;        // census work counters (uint32 x 8)
     DevBuf acc;        // census accumulators (uint64 x 16)
     DevBuf cost;       // optional per-vertex predicted cost (float x n) for the learned schedule
     DevBuf tri;        // triangle form: bulk sums and triangle tricode histogram (uint64 x 96)
@@ -84,6 +89,10 @@ struct GraphStore {
         d.rp = rp.as<uint32_t>();
         d.vs = vs.as<uint2>();
         d.us = us.as<uint2>();
+        d.rec = rec.as<uint4>();
+        d.blk16 = blk16.as<uint4>();
+        d.rec2 = rec.p ? d.rec + n_active : nullptr;
+        d.n16 = rec.p ? reinterpret_cast<const uint32_t*>(d.rec + 3ull * n_active) : nullptr;
         return d;
     }
 };
@@ -134,14 +143,14 @@ void census_fit_chunk(const GraphStore& g, Opts& o);
 // d_phase (optional, [3 * CTAs] uint64) the globaltimer at start, end of items, end per CTA.
 tc_status census_enqueue(GraphStore& g, const Opts& o, const Plan& p, cudaStream_t st, unsigned long long* d_out16,
                          unsigned long long* d_vcost = nullptr, unsigned long long* d_phase = nullptr);
-// The same census over a part of a plan: items[0, n_items) and warp-tier vertices
+// The same census over a part of a plan: items [item0, item0 + n_items) and warp-tier vertices
 // [warp_begin, warp_end) (a shard; census_enqueue runs the whole plan).
-tc_status census_enqueue_range(GraphStore& g, const Opts& o, const Item* items, uint32_t n_items, uint32_t warp_begin,
-                               uint32_t warp_end, cudaStream_t st, unsigned long long* d_out16,
+tc_status census_enqueue_range(GraphStore& g, const Opts& o, const Plan& p, uint32_t item0, uint32_t n_items,
+                               uint32_t warp_begin, uint32_t warp_end, cudaStream_t st, unsigned long long* d_out16,
                                unsigned long long* d_vcost = nullptr, unsigned long long* d_phase = nullptr);
 // TC_ALGO_TRIANGLE (triangles.cu): the bulk pair sums and the triangle tricode histogram over
 // the given items and warp-tier range, and the fold into d_out16[1..15].
-tc_status triangle_census_enqueue(GraphStore& g, const Opts& o, const Item* items, uint32_t n_items,
+tc_status triangle_census_enqueue(GraphStore& g, const Opts& o, const Plan& p, uint32_t item0, uint32_t n_items,
                                   uint32_t warp_begin, uint32_t warp_end, cudaStream_t st, unsigned long long* d_out16,
                                   unsigned long long* d_vcost, unsigned long long* d_phase = nullptr);
 // Batched triangle form: k graphs (d_graphs), items tagged with the graph (pad), warp-tier
@@ -159,11 +168,17 @@ tc_status triangle_census_wave(const WaveReq* d_reqs, uint32_t n_reqs, uint32_t 
 tc_status triangle_collect(unsigned long long* const* scratch, uint32_t n, unsigned long long* d_dst, cudaStream_t st);
 // The triangle walk alone: histogram of the 64 tricodes (old == nullptr) or of the 64 states in
 // the caller's id order (old = original id per vertex, d_perm_state = [9][64] state of a
-// tricode per rank pattern) of every triangle, added into d_hist64; ctr: 4 zeroed uint32.
+// tricode per rank pattern) of every triangle, added into d_hist64; ctr: 4 zeroed uint32.  split (old
+// == nullptr only): run the three launches of walk16.cu instead, which take the items before split[0],
+// before split[1] and the others; ctr then holds 4 more zeroed uint32.
 tc_status triangles_launch(const GraphDev& gd, const Opts& o, const Item* items, uint32_t n_items, uint32_t warp_begin,
                            uint32_t warp_end, uint32_t* ctr, const uint32_t* old, const uint8_t* d_perm_state,
                            unsigned long long* d_hist64, unsigned long long* d_vcost, cudaStream_t st,
-                           unsigned long long* d_phase = nullptr);
+                           unsigned long long* d_phase = nullptr, const uint32_t* split = nullptr);
+// Whether the triangle walk of a single-graph census of g takes the launches of walk16.cu.
+bool walk16_takes(const GraphStore& g);
+// Make g's 16-bit lower lists (synchronises st).
+tc_status lists16_build(GraphStore& g, cudaStream_t st);
 // Cut p's work into `world` contiguous shards of about equal work (cached in p for that world);
 // synchronises st when it computes them.
 tc_status plan_shards(GraphStore& g, const Opts& o, Plan& p, uint32_t world, cudaStream_t st);

@@ -66,7 +66,26 @@ struct GraphDev {
     const uint32_t* rp;     // [E]
     const uint2* vs;        // [E]
     const uint2* us;        // [E]
+    // The triangle form's 16-bit lower lists (null until a census of walk16.cu made them): the neighbours of x with ids below both x and
+    // kIds16, split by window of kWin16 ids and, in a window, by direction class (1, 2, 3 seen
+    // from x).  Each of the 12 segments holds ids within its window, ascending, in 16-byte blocks
+    // of eight, the last block padded with kPad16; the segments' blocks follow each other.
+    // rec[x] = (first block, the lengths of window 0's class 1 and 2 as 16-bit halves, the class-1
+    // and class-2 entries of all of N[x]); rec2[2x], rec2[2x + 1] (x >= kWin16 only) = the 16-bit
+    // lengths of the segments from window 0's class 3 on.  n16[x] = entries in all segments.
+    const uint4* rec;       // [n_active], set where n16 is not 0
+    const uint4* rec2;      // [2 n_active]
+    const uint4* blk16;
+    const uint32_t* n16;    // [n_active]
 };
+constexpr uint32_t kWin16 = 1u << 15, kIds16 = 4u * kWin16, kPad16 = kWin16;
+
+// walk16.cu gives the items of vertices of at most kHubDeg neighbours a warp, the others a CTA; those
+// from id kTableFrom on are walked as stored instead of from the 16-bit lists.  A warp's hash holds
+// 2 kHubDeg slots; scale 20 / 24 with 128, 256 and 512: 1.74 / 58.8, 1.65 / 55.0 and 2.45 / 54.9 ms.
+// Past kTableFrom a pair's prefix of a few dozen entries spreads over 12 segments; scale 26 with
+// 2^15, 2^16, 2^17, 2^18 and 2^19: 369, 318, 279, 282 and 295 ms.
+constexpr uint32_t kHubDeg = 256, kTableFrom = 1u << 17;
 
 // One CTA work item of the census: vertex u and its pairs (u, N[u][j]) for j in [j0, j1)
 // (all with N[u][j] > u).  N[u] is staged in shared memory one chunk at a time.

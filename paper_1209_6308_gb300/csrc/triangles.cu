@@ -28,239 +28,18 @@
 // shared-memory hash, and its warps walk the lists L(c) of 32 pairs at a time as one
 // flattened range, so short and long lists share the lanes.  The other vertices run one warp
 // each, with L(b) in the warp's own hash.
+#include <algorithm>
 #include <atomic>
 #include <cstring>
 
 #include "graph.cuh"
+#include "triangles.cuh"
 
 namespace tc {
+
+tc_status walk16_launch(const TriParams& P, const uint32_t split[2], uint32_t grid, uint32_t* ctr, cudaStream_t st);   // walk16.cu
+
 namespace {
-
-constexpr int kThreads = 256;
-constexpr int kWarps = kThreads / 32;
-// Prefixes of at least kLongPrefix entries are walked one pair at a time by the whole warp
-// (walk_pairs<..., LONGW = true>), kLongRounds loads of 32 entries in flight per lane; shorter
-// ones share flattened ranges.
-// (Swept at scales 20 and 26: thresholds 64-512, 2-8 rounds.)
-constexpr uint32_t kLongPrefix = 128;
-constexpr int kLongRounds = 8;
-constexpr uint32_t kWarpSlots = 256;     // per-warp hash slots: |L(b)| <= warp_max_deg <= 128
-constexpr uint32_t kFlushElems = 1u << 30;
-
-__device__ __forceinline__ unsigned long long tri_clock_ns() {
-    unsigned long long t;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-    return t;
-}
-
-__device__ __forceinline__ uint32_t tri_hash(uint32_t x, int hb) { return (x * 2654435761u) >> (32 - hb); }
-
-// Tricode of the triangle (a, b, c) from the direction bits of three stored entries: a in N[b]
-// (seen from b: 1 b->a, 2 a->b), c in N[b] (1 b->c, 2 c->b) and a in N[c] (1 c->a, 2 a->c).
-// Tricode bits: 1 b->a, 2 a->b, 4 b->c, 8 c->b, 16 a->c, 32 c->a.  The walk keeps the second
-// term pre-shifted per pair (bc_bits = (dir(b,c)) << 2) and maps the third through a four-entry
-// byte table: dir(c,a) 1 -> 32, 2 -> 16, 3 -> 48.
-__device__ __forceinline__ uint32_t tri_code(uint32_t dir_ba, uint32_t bc_bits, uint32_t e_ca) {
-    return dir_ba | bc_bits | __byte_perm(0x30102000u, 0u, e_ca & 3u);
-}
-
-struct TriParams {
-    GraphDev g;
-    const Item* items;
-    uint32_t n_items;
-    uint32_t warp_begin, warp_end;
-    uint32_t wshift;              // warp tier: 2^wshift consecutive vertices per grab
-    uint32_t chunk;               // entries of L(b) staged per pass of a CTA item (hash: 2 x chunk slots)
-    uint32_t* ctr;                // [0] next item, [1] next warp-tier vertex
-    const uint32_t* old;          // OLD: the caller's id of each vertex
-    const uint8_t* perm_state;    // OLD: [9][64] state of a tricode under the rank pattern 3 ra + rb
-    unsigned long long* hist;     // 64 bins (triangle tricodes, or states with OLD); batched: graph g's at
-                                  // hist + kBatchStride g
-    unsigned long long* vcost;    // optional [n]: SM cycles per CTA-tier vertex b
-    unsigned long long* phase;    // optional [3 * gridDim]: globaltimer at start, end of items, end
-    // batched launch: item.pad is the graph index, warp-tier blocks are (u0, u1, graph)
-    const GraphDev* graphs;
-    const uint4* wblocks;
-    uint32_t n_wblocks;
-    // serving wave: n_items / n_wblocks are the wave's totals over its request slices
-    const WaveReq* reqs;
-    uint32_t n_reqs;
-};
-
-// batched triangle form: per graph 96 uint64 of scratch, the 21 bulk sums at [0, 21) and the 64
-// triangle tricodes at [32, 96); a serving wave's requests have the same scratch at WaveReq.out
-constexpr uint32_t kBatchStride = 96;
-
-// launch modes: one graph; a batch of graphs (items tagged with the graph, blocks (u0, u1, g));
-// a serving wave (slices of several requests, descriptors in global memory)
-enum { kTriSingle = 0, kTriBatch = 1, kTriWave = 2 };
-
-// index r of the last request whose prefix is <= i (prefixes ascend from 0)
-template <typename F>
-__device__ __forceinline__ uint32_t find_req(uint32_t count, uint32_t i, F pre) {
-    uint32_t lo = 0, hi = count;
-    while (hi - lo > 1) {
-        const uint32_t mid = (lo + hi) >> 1;
-        if (pre(mid) <= i) lo = mid; else hi = mid;
-    }
-    return lo;
-}
-
-// Walk, for the pairs (b, c = N[b][j]), j in [j0, j1), 32 pairs per batch, the entries of N[c]
-// below b (rp = b's position in N[c], from the pair tables; pb + j indexes the pair) and count
-// each a found in the staged L(b).  MAP: L(b) is a direct map of two direction bits per id (every
-// a < b is in its range); else a hash.  One warp: a batch's pairs with long prefixes are walked
-// one after another by all lanes, and the lanes share the flattened (pair, position) range of
-// the others.  Returns the entries walked (warp-uniform).
-template <bool OLD, bool MAP, bool LONGW>
-__device__ __forceinline__ uint32_t walk_pairs(const TriParams& P, const GraphDev& G, uint64_t bbase, uint64_t pb,
-                                               uint32_t j0, uint32_t j1, const uint32_t* sH, const uint32_t* sO,
-                                               int hb, uint32_t hmask, uint32_t ob, const uint8_t* sPerm,
-                                               uint32_t* myHist, int lane) {
-    const uint64_t* __restrict__ off = G.off;
-    const uint32_t* __restrict__ adj = G.adj;
-    const uint32_t* __restrict__ rp = G.rp;
-    const uint32_t le_mask = (2u << lane) - 1u;
-    uint32_t walked = 0;
-    // one walked entry e_ca = a in N[c] of the pair whose b-c tricode bits are bcb (and whose c has
-    // the caller id oc2): look a up in L(b), count the triangle's tricode (or state) if found
-    auto count = [&](uint32_t e_ca, uint32_t bcb, uint32_t oc2) {
-        if (!e_ca) return;
-        const uint32_t a = e_ca >> 2;
-        uint32_t dir, oa = 0;
-        if (MAP) {   // word a / 16, bits 2 (a mod 16), read straight from the entry
-            dir = (sH[e_ca >> 6] >> ((e_ca >> 1) & 30u)) & 3u;
-            if (OLD && dir) oa = P.old[a];
-        } else {
-            uint32_t h = tri_hash(a, hb);
-            uint32_t e = sH[h];
-            while (e != 0u && (e >> 2) != a) {
-                h = (h + 1u) & hmask;
-                e = sH[h];
-            }
-            dir = e & 3u;
-            if (OLD && e) oa = sO[h];
-        }
-        if (dir != 0u) {
-            uint32_t t = tri_code(dir, bcb, e_ca);
-            if (OLD) {
-                const uint32_t ra = (oa > ob) + (oa > oc2), rb = (ob > oa) + (ob > oc2);
-                t = sPerm[(3u * ra + rb) * 64u + t];
-            }
-            atomicAdd(&myHist[t], 1u);
-        }
-    };
-    for (uint32_t jb = j0; jb < j1; jb += 32) {
-        const uint32_t j = jb + lane;
-        const bool ok = j < j1;
-        uint32_t e_bc = ok ? adj[bbase + j] : 0u;
-        const uint32_t c = e_bc >> 2;
-        uint64_t cb = ok ? off[c] : 0ull;
-        uint32_t len = ok ? rp[pb + j] : 0u;
-        uint32_t oc = (OLD && ok) ? P.old[c] : 0u;
-        if (LONGW) {
-            // pairs with long prefixes, one at a time over the whole warp: consecutive entries,
-            // no search for the pair that holds an entry
-            uint32_t lm = __ballot_sync(0xffffffffu, len >= kLongPrefix);
-            while (lm) {
-                const int q = __ffs(lm) - 1;
-                lm &= lm - 1u;
-                const uint64_t B = __shfl_sync(0xffffffffu, cb, q);
-                const uint32_t L = __shfl_sync(0xffffffffu, len, q);
-                const uint32_t bcb = (__shfl_sync(0xffffffffu, e_bc, q) & 3u) << 2;
-                const uint32_t oq = OLD ? __shfl_sync(0xffffffffu, oc, q) : 0u;
-                walked += L;
-                for (uint32_t i = lane; i < L; i += 32u * kLongRounds) {
-                    uint32_t x[kLongRounds];
-#pragma unroll
-                    for (int r = 0; r < kLongRounds; ++r)
-                        x[r] = i + 32u * r < L ? __ldg(adj + (B + i + 32u * r)) : 0u;
-#pragma unroll
-                    for (int r = 0; r < kLongRounds; ++r) count(x[r], bcb, oq);
-                }
-            }
-            if (len >= kLongPrefix) len = 0u;
-        }
-        // compact the pairs with a non-empty L(c) into lanes 0 .. cnt-1
-        const uint32_t nz = __ballot_sync(0xffffffffu, len != 0u);
-        if (!nz) continue;
-        const uint32_t cnt = __popc(nz);
-        const uint32_t src = __fns(nz, 0, lane + 1) & 31u;
-        e_bc = __shfl_sync(0xffffffffu, e_bc, src);
-        cb = __shfl_sync(0xffffffffu, cb, src);
-        len = __shfl_sync(0xffffffffu, len, src);
-        if (OLD) oc = __shfl_sync(0xffffffffu, oc, src);
-        if ((uint32_t)lane >= cnt) len = 0u;
-        uint32_t incl = len;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= o) incl += y;
-        }
-        const uint32_t excl = incl - len;
-        const uint32_t total = __shfl_sync(0xffffffffu, incl, 31);
-        walked += total;
-        // entry i of the flattened range lies at adj[cbx + i] for the pair that holds it (modular
-        // arithmetic: i >= excl), and its tricode's b-c bits are bcb
-        const uint64_t cbx = cb - excl;
-        const uint32_t bcb = (e_bc & 3u) << 2;
-        int seg_prev = -1;
-        // two rounds of 32 entries per iteration, so each lane has two loads in flight
-        for (uint32_t base = 0; base < total; base += 64) {
-            // the pairs whose range starts in a round mark their start; lane i's pair is the
-            // last one started at or before the round's entry i
-            const bool stA = (uint32_t)lane < cnt && excl >= base && excl < base + 32u;
-            const bool stB = (uint32_t)lane < cnt && excl >= base + 32u && excl < base + 64u;
-            const uint32_t MA = __reduce_or_sync(0xffffffffu, stA ? (1u << (excl - base)) : 0u);
-            const uint32_t MB = __reduce_or_sync(0xffffffffu, stB ? (1u << (excl - base - 32u)) : 0u);
-            // (lane 31's count covers the whole round: the last pair of a round needs no shuffle)
-            const int segA = seg_prev + __popc(MA & le_mask);
-            const int lastA = seg_prev + __popc(MA);
-            const int segB = lastA + __popc(MB & le_mask);
-            seg_prev = lastA + __popc(MB);
-            const uint32_t sa = (uint32_t)segA & 31u, sb = (uint32_t)segB & 31u;
-            const uint64_t BA = __shfl_sync(0xffffffffu, cbx, sa), BB = __shfl_sync(0xffffffffu, cbx, sb);
-            const uint32_t EA = __shfl_sync(0xffffffffu, bcb, sa), EB = __shfl_sync(0xffffffffu, bcb, sb);
-            uint32_t OA = 0, OB = 0;
-            if (OLD) {
-                OA = __shfl_sync(0xffffffffu, oc, sa);
-                OB = __shfl_sync(0xffffffffu, oc, sb);
-            }
-            const uint32_t iA = base + lane, iB = base + 32u + lane;
-            const uint32_t xA = iA < total ? __ldg(adj + (BA + iA)) : 0u;
-            const uint32_t xB = iB < total ? __ldg(adj + (BB + iB)) : 0u;
-            count(xA, EA, OA);
-            count(xB, EB, OB);
-        }
-    }
-    return walked;
-}
-
-// A warp's next pairs of the CTA's item: guided sizes, 32 pairs while many remain, then fewer
-// (down to 4) as the item runs out, so that the warps reach the item's end barrier together.
-__device__ __forceinline__ void grab_pairs(uint32_t* s_next, uint32_t j1, int lane, uint32_t& jb, uint32_t& g) {
-    jb = 0;
-    g = 32;
-    if (lane == 0) {
-        const uint32_t cur = *(volatile uint32_t*)s_next;
-        const uint32_t rem = cur < j1 ? j1 - cur : 0u;
-        g = max(4u, min(32u, rem / (2u * kWarps)));
-        jb = atomicAdd(s_next, g);
-    }
-    jb = __shfl_sync(0xffffffffu, jb, 0);
-    g = __shfl_sync(0xffffffffu, g, 0);
-}
-
-// Add a warp's 64 bins to the graph's histogram and clear them (one warp).
-__device__ __forceinline__ void flush_warp_hist(uint32_t* myHist, unsigned long long* hist, int lane) {
-    __syncwarp();
-    for (int t = lane; t < 64; t += 32) {
-        const uint32_t v = myHist[t];
-        if (v) atomicAdd(&hist[t], (unsigned long long)v);
-        myHist[t] = 0u;
-    }
-    __syncwarp();
-}
 
 template <bool OLD, int MODE>
 __global__ void __launch_bounds__(kThreads, 8) k_triangles(TriParams P) {
@@ -742,10 +521,8 @@ tc_status fold_table(Table64* T) {
 tc_status triangles_launch(const GraphDev& gd, const Opts& o, const Item* items, uint32_t n_items, uint32_t warp_begin,
                            uint32_t warp_end, uint32_t* ctr, const uint32_t* old, const uint8_t* d_perm_state,
                            unsigned long long* d_hist64, unsigned long long* d_vcost, cudaStream_t st,
-                           unsigned long long* d_phase) {
+                           unsigned long long* d_phase, const uint32_t* split) {
     const bool is_old = old != nullptr;
-    const size_t smem = tri_smem(o.chunk, is_old);
-    TC_TRY(tri_prepare(is_old ? 1 : 0, smem));
     TriParams P;
     std::memset(&P, 0, sizeof(P));
     P.g = gd;
@@ -762,13 +539,16 @@ tc_status triangles_launch(const GraphDev& gd, const Opts& o, const Item* items,
     P.vcost = d_vcost;
     P.phase = d_phase;
     const unsigned grid = (unsigned)census_grid(o);
+    if (split && !is_old) return walk16_launch(P, split, grid, ctr + 4, st);
+    const size_t smem = tri_smem(o.chunk, is_old);
+    TC_TRY(tri_prepare(is_old ? 1 : 0, smem));
     if (is_old) k_triangles<true, kTriSingle><<<grid, kThreads, smem, st>>>(P);
     else k_triangles<false, kTriSingle><<<grid, kThreads, smem, st>>>(P);
     TC_LAUNCH("k_triangles");
     return TC_OK;
 }
 
-tc_status triangle_census_enqueue(GraphStore& g, const Opts& o, const Item* items, uint32_t n_items,
+tc_status triangle_census_enqueue(GraphStore& g, const Opts& o, const Plan& p, uint32_t item0, uint32_t n_items,
                                   uint32_t warp_begin, uint32_t warp_end, cudaStream_t st, unsigned long long* d_out16,
                                   unsigned long long* d_vcost, unsigned long long* d_phase) {
     if (g.e_sym == 0) return TC_OK;
@@ -777,7 +557,13 @@ tc_status triangle_census_enqueue(GraphStore& g, const Opts& o, const Item* item
     unsigned long long* raw = g.tri.as<unsigned long long>();   // [0, 21) bulk sums, [32, 96) triangle tricodes
     unsigned long long* hist = raw + 32;
     TC_CUDA(cudaMemsetAsync(raw, 0, sizeof(unsigned long long) * kBatchStride, st));
-    TC_CUDA(cudaMemsetAsync(g.ctr.p, 0, sizeof(uint32_t) * 4, st));
+    TC_CUDA(cudaMemsetAsync(g.ctr.p, 0, sizeof(uint32_t) * 8, st));
+    const Item* items = p.items.as<Item>() + item0;
+    // the range's part of each of the plan's splits
+    const uint32_t split[2] = {std::min(std::max(p.split[0], item0) - item0, n_items),
+                               std::min(std::max(p.split[1], item0) - item0, n_items)};
+    const bool walk16 = walk16_takes(g);
+    if (walk16 && !g.blk16.p) TC_TRY(lists16_build(g, st));
     const GraphDev gd = g.dev();
     const uint64_t units = (uint64_t)n_items + (warp_end - warp_begin + 31u) / 32u;
     if (units) {
@@ -794,7 +580,7 @@ tc_status triangle_census_enqueue(GraphStore& g, const Opts& o, const Item* item
         TC_LAUNCH("k_pair_bulk");
     }
     TC_TRY(triangles_launch(gd, o, items, n_items, warp_begin, warp_end, g.ctr.as<uint32_t>(), nullptr, nullptr, hist,
-                            d_vcost, st, d_phase));
+                            d_vcost, st, d_phase, walk16 ? split : nullptr));
     Table64 T;
     TC_TRY(fold_table(&T));
     k_tri_fold<<<1, 64, 0, st>>>(raw, hist, T, d_out16);
