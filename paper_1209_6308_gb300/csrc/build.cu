@@ -419,7 +419,7 @@ tc_status finish_graph(GraphStore& g, uint64_t E, int B, uint64_t* ukey, uint32_
     TC_LAUNCH("k_relabel_keys");
     uint64_t* kp = rk.as<uint64_t>();
     uint64_t* tp = rtmp.as<uint64_t>();
-    TC_TRY(radix_sort_u64(&kp, &tp, n, 0, 2 * B, st));
+    TC_TRY(radix_sort_u64(&kp, &tp, n, B, 2 * B, st));   // stable: ties stay in id order
     k_perm<<<gridN, kB, 0, st>>>(kp, n, B, deg, g.new_of_old.as<uint32_t>(), ndeg.as<uint32_t>());
     TC_LAUNCH("k_perm");
     rk.release();

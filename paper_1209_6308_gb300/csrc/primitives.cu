@@ -1,12 +1,18 @@
 // primitives.cu - device scans and a stable LSD radix sort, used by the graph builder
 // (symmetrise, dedupe, relabel and sort steps of the Sec. 6 compact structure).
 //
-// Scan: reduce-then-scan over tiles of 4096 values (256 threads x 16 per thread), the tile
-// sums scanned by one CTA, then a downsweep.
-// Radix sort: 8-bit digits.  Per pass: a tile histogram (digit-major counts), an exclusive
-// scan of the counts, and a scatter that ranks each key stably inside its tile with a
-// warp multi-split (eight ballots give the lanes sharing a digit), stages the tile in
-// shared memory in digit order, then writes contiguous runs per digit.
+// Both read their input once per pass: a tile learns what comes before it from its predecessors
+// ("decoupled look-back", Merrill and Garland 2016).  A tile publishes its own sum at once and, when
+// it knows it, the sum of everything up to its end; a tile looks back over its predecessors' sums
+// until it meets such an inclusive one.  Tiles are handed out by an atomic ticket, so every
+// predecessor is already running and the look-back ends; after kPatience looks at one word a tile
+// stops waiting and sums its predecessors' input itself.
+// Scan: tiles of 4096 values, one kernel.
+// Radix sort: 8-bit digits; one kernel counts every digit of every pass, then one kernel per pass
+// ranks a tile's keys stably (per warp: the lanes sharing a digit, by eight ballots, against the
+// warp's running counts), looks back per digit, stages the tile in shared memory in digit order
+// and writes contiguous runs per digit ("onesweep", Adinets and Merrill 2022).  16 bytes per key and
+// pass where a histogram, a scan and a scatter per pass moved 24 in five kernels.
 #include <algorithm>
 
 #include "tc_internal.cuh"
@@ -17,9 +23,24 @@ namespace {
 constexpr int kScanThreads = 256;
 constexpr int kScanPer = 16;
 constexpr int kScanTile = kScanThreads * kScanPer;
-constexpr int kSortThreads = 256;
-constexpr int kSortRounds = 16;
-constexpr int kSortTile = kSortThreads * kSortRounds;
+constexpr int kSortThreads = 512;
+constexpr int kSortWarps = kSortThreads / 32;
+constexpr int kSortPer = 16;
+constexpr int kSortTile = kSortThreads * kSortPer;
+constexpr int kPasses = 8;                      // of 8 bits
+constexpr uint32_t kPatience = 1u << 16;
+
+// A tile's published sums: the value, and in the top bits which one it is.
+constexpr unsigned long long kOwn = 1ull << 62, kUpTo = 2ull << 62, kValue = kOwn - 1ull;
+
+__device__ __forceinline__ unsigned long long peek(const unsigned long long* p) {
+    unsigned long long v;
+    asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ void post(unsigned long long* p, unsigned long long v) {
+    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" :: "l"(p), "l"(v) : "memory");
+}
 
 template <typename T>
 __device__ __forceinline__ T warp_incl_scan(T v) {
@@ -55,56 +76,71 @@ __device__ __forceinline__ T block_excl_scan(T v, T* total) {
     return res;
 }
 
+// state[0]: the ticket; state[1 + t]: tile t's sums (all zero before the launch).  total may be null.
 template <typename Tout>
-__global__ void __launch_bounds__(kScanThreads) k_scan_reduce(const uint32_t* in, uint64_t n, Tout* tile_sums) {
-    uint64_t base = (uint64_t)blockIdx.x * kScanTile;
-    Tout s = 0;
+__global__ void __launch_bounds__(kScanThreads) k_scan(const uint32_t* __restrict__ in, uint64_t n, Tout* __restrict__ out,
+                                                       Tout* total, unsigned long long* state) {
+    __shared__ uint32_t tile_in[kScanTile];
+    __shared__ unsigned long long s_before;
+    __shared__ uint32_t s_tile;
+    const int tid = threadIdx.x, lane = tid & 31;
+    if (tid == 0) s_tile = (uint32_t)atomicAdd(state, 1ull);
+    __syncthreads();
+    const uint32_t tile = s_tile;
+    const uint64_t base = (uint64_t)tile * kScanTile;
 #pragma unroll
     for (int r = 0; r < kScanPer; ++r) {
-        uint64_t i = base + (uint64_t)r * kScanThreads + threadIdx.x;
-        if (i < n) s += in[i];
-    }
-    Tout tot;
-    block_excl_scan<Tout>(s, &tot);
-    if (threadIdx.x == 0) tile_sums[blockIdx.x] = tot;
-}
-
-// One CTA scans `cnt` tile sums in place (exclusive); writes the grand total to *total.
-template <typename Tout>
-__global__ void __launch_bounds__(1024) k_scan_tiles(Tout* sums, uint64_t cnt, Tout* total) {
-    Tout carry = 0;
-    for (uint64_t base = 0; base < cnt; base += 1024) {
-        uint64_t i = base + threadIdx.x;
-        Tout v = i < cnt ? sums[i] : Tout(0);
-        Tout tot;
-        Tout ex = block_excl_scan<Tout>(v, &tot);
-        if (i < cnt) sums[i] = ex + carry;
-        carry += tot;
-    }
-    if (threadIdx.x == 0 && total) *total = carry;
-}
-
-template <typename Tout>
-__global__ void __launch_bounds__(kScanThreads) k_scan_down(const uint32_t* in, uint64_t n, const Tout* tile_off, Tout* out) {
-    __shared__ uint32_t tile[kScanTile];
-    uint64_t base = (uint64_t)blockIdx.x * kScanTile;
-#pragma unroll
-    for (int r = 0; r < kScanPer; ++r) {
-        uint64_t i = base + (uint64_t)r * kScanThreads + threadIdx.x;
-        tile[r * kScanThreads + threadIdx.x] = i < n ? in[i] : 0u;
+        const uint64_t i = base + (uint64_t)r * kScanThreads + tid;
+        tile_in[r * kScanThreads + tid] = i < n ? in[i] : 0u;
     }
     __syncthreads();
     // thread t owns the 16 consecutive values [16t, 16t+16) of the tile
-    Tout loc[kScanPer];
-    Tout s = 0;
-#pragma unroll
-    for (int k = 0; k < kScanPer; ++k) { loc[k] = s; s += tile[threadIdx.x * kScanPer + k]; }
-    Tout tot;
-    Tout ex = block_excl_scan<Tout>(s, &tot) + tile_off[blockIdx.x];
+    unsigned long long loc[kScanPer], s = 0;
 #pragma unroll
     for (int k = 0; k < kScanPer; ++k) {
-        uint64_t i = base + (uint64_t)threadIdx.x * kScanPer + k;
-        if (i < n) out[i] = ex + loc[k];
+        loc[k] = s;
+        s += tile_in[tid * kScanPer + k];
+    }
+    unsigned long long own;
+    const unsigned long long ex = block_excl_scan<unsigned long long>(s, &own);
+    if (tid < 32) {
+        if (lane == 0) post(&state[1 + tile], (tile ? kOwn : kUpTo) | own);
+        unsigned long long before = 0;
+        bool gave_up = false;
+        // 32 predecessors at a time, the nearest in lane 0
+        for (int64_t t = (int64_t)tile - 1; t >= 0 && !gave_up; t -= 32) {
+            unsigned long long v = kUpTo;   // before the first tile: nothing
+            if (t - lane >= 0) {
+                uint32_t looks = 0;
+                while ((v = peek(&state[1 + t - lane])) < kOwn && ++looks < kPatience) {}
+            }
+            gave_up = __any_sync(0xffffffffu, v < kOwn);
+            const uint32_t done = __ballot_sync(0xffffffffu, v >= kUpTo);
+            const int last = done ? __ffs(done) - 1 : 31;   // the nearest inclusive sum ends the look-back
+            unsigned long long part = lane <= last ? v & kValue : 0ull;
+            for (int o = 16; o; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
+            before += part;
+            if (done) break;
+        }
+        if (lane == 0) s_before = gave_up ? ~0ull : before;
+    }
+    __syncthreads();
+    if (s_before == ~0ull) {   // uniform: the predecessors' input itself
+        unsigned long long sum = 0, all;
+        for (uint64_t i = tid; i < base; i += kScanThreads) sum += in[i];
+        block_excl_scan<unsigned long long>(sum, &all);
+        if (tid == 0) s_before = all;
+        __syncthreads();
+    }
+    const unsigned long long before = s_before;
+    if (tid == 0) {
+        if (tile) post(&state[1 + tile], kUpTo | (before + own));
+        if (total && base + kScanTile >= n) *total = (Tout)(before + own);
+    }
+#pragma unroll
+    for (int k = 0; k < kScanPer; ++k) {
+        const uint64_t i = base + (uint64_t)tid * kScanPer + k;
+        if (i < n) out[i] = (Tout)(before + ex + loc[k]);
     }
 }
 
@@ -114,107 +150,164 @@ tc_status scan_impl(const uint32_t* in, Tout* out, uint64_t n, Tout* total, cuda
         if (total) TC_CUDA(cudaMemsetAsync(total, 0, sizeof(Tout), st));
         return TC_OK;
     }
-    uint64_t tiles = (n + kScanTile - 1) / kScanTile;
+    const uint64_t tiles = (n + kScanTile - 1) / kScanTile;
     if (tiles > 0x7fffffffull) return fail(TC_ERR_RANGE, "scan: too many elements");
-    DevBuf sums;
-    TC_TRY(sums.alloc(sizeof(Tout) * tiles, st));
-    k_scan_reduce<Tout><<<(unsigned)tiles, kScanThreads, 0, st>>>(in, n, sums.as<Tout>());
-    TC_LAUNCH("k_scan_reduce");
-    k_scan_tiles<Tout><<<1, 1024, 0, st>>>(sums.as<Tout>(), tiles, total);
-    TC_LAUNCH("k_scan_tiles");
-    k_scan_down<Tout><<<(unsigned)tiles, kScanThreads, 0, st>>>(in, n, sums.as<Tout>(), out);
-    TC_LAUNCH("k_scan_down");
+    DevBuf state;
+    TC_TRY(state.alloc(sizeof(unsigned long long) * (tiles + 1), st));
+    TC_CUDA(cudaMemsetAsync(state.p, 0, sizeof(unsigned long long) * (tiles + 1), st));
+    k_scan<Tout><<<(unsigned)tiles, kScanThreads, 0, st>>>(in, n, out, total, state.as<unsigned long long>());
+    TC_LAUNCH("k_scan");
     return TC_OK;
 }
 
 // ------------------------------------------------------------------ radix sort
-__global__ void __launch_bounds__(kSortThreads) k_radix_hist(const uint64_t* keys, uint64_t n, int shift,
-                                                             uint32_t* counts, uint32_t tiles) {
-    __shared__ uint32_t wh[kSortThreads / 32][256];
-    const int warp = threadIdx.x >> 5;
-    for (int d = threadIdx.x; d < (kSortThreads / 32) * 256; d += kSortThreads) (&wh[0][0])[d] = 0;
+// hist[256 p + d] += the keys whose digit p (bits lo + 8 p and up) is d, for every pass.
+__global__ void __launch_bounds__(kSortThreads) k_digit_counts(const uint64_t* __restrict__ keys, uint64_t n, int lo,
+                                                               int passes, uint32_t* hist) {
+    __shared__ uint32_t h[kPasses][256];
+    for (int k = threadIdx.x; k < passes * 256; k += kSortThreads) (&h[0][0])[k] = 0u;
     __syncthreads();
-    uint64_t base = (uint64_t)blockIdx.x * kSortTile;
-    // all of the thread's keys are loaded before any is counted, so the tile's loads are in
-    // flight together
-    uint32_t dg[kSortRounds];
+    const uint32_t lane = threadIdx.x & 31;
+    const uint64_t stride = (uint64_t)gridDim.x * kSortThreads;
+    constexpr int kAhead = 4;
+    for (uint64_t i0 = blockIdx.x * (uint64_t)kSortThreads + (threadIdx.x & ~31u); i0 < n; i0 += kAhead * stride) {
+        uint64_t key[kAhead];
 #pragma unroll
-    for (int r = 0; r < kSortRounds; ++r) {
-        uint64_t i = base + (uint64_t)r * kSortThreads + threadIdx.x;
-        dg[r] = i < n ? (uint32_t)(keys[i] >> shift) & 255u : 256u;
+        for (int r = 0; r < kAhead; ++r) {
+            const uint64_t i = i0 + r * stride + lane;
+            key[r] = i < n ? keys[i] : 0ull;
+        }
+#pragma unroll
+        for (int r = 0; r < kAhead; ++r) {
+            const uint64_t i = i0 + r * stride;
+            if (i >= n) break;
+            const bool ok = i + lane < n;
+            const uint32_t live = __ballot_sync(0xffffffffu, ok);
+            for (int p = 0; p < passes; ++p) {
+                const uint32_t d = (uint32_t)(key[r] >> (lo + 8 * p)) & 255u;
+                const uint32_t d0 = __shfl_sync(0xffffffffu, d, 0);
+                // sorted input has one digit in the whole warp: one add instead of 32 on one address
+                if (__all_sync(0xffffffffu, !ok || d == d0)) {
+                    if (lane == 0) atomicAdd(&h[p][d], (uint32_t)__popc(live));
+                } else if (ok) {
+                    atomicAdd(&h[p][d], 1u);
+                }
+            }
+        }
     }
-#pragma unroll
-    for (int r = 0; r < kSortRounds; ++r)
-        if (dg[r] < 256u) atomicAdd(&wh[warp][dg[r]], 1u);
     __syncthreads();
-    uint32_t s = 0;
-#pragma unroll
-    for (int w = 0; w < kSortThreads / 32; ++w) s += wh[w][threadIdx.x];
-    counts[(uint64_t)threadIdx.x * tiles + blockIdx.x] = s;
+    for (int k = threadIdx.x; k < passes * 256; k += kSortThreads)
+        if ((&h[0][0])[k]) atomicAdd(&hist[k], (&h[0][0])[k]);
 }
 
-__global__ void __launch_bounds__(kSortThreads, 3) k_radix_scatter(const uint64_t* in, uint64_t* out, uint64_t n, int shift,
-                                                                const uint32_t* counts, const uint32_t* offs,
-                                                                uint32_t tiles) {
-    __shared__ uint64_t s_keys[kSortTile];
-    __shared__ uint32_t s_start[256];
-    __shared__ uint32_t s_run[256];
-    __shared__ uint32_t s_wc[kSortThreads / 32][256];
+struct SortShared {
+    uint64_t keys[kSortTile];
+    uint32_t wh[kSortWarps][256];   // a warp's keys per digit; then its first place behind the earlier warps'
+    uint32_t start[256];            // first place of a digit in the tile
+    uint32_t to[256];               // first place of a digit of this tile in the output, less start
+    uint32_t tile, gave_up;
+};
+
+// One pass: out = in stably sorted by its digit at `shift`; hist = the digit's counts, ticket and
+// state (256 words per tile) as for k_scan but state words of other passes are left over: they
+// carry their pass in bits 32..39 of the value.
+__global__ void __launch_bounds__(kSortThreads, 2) k_radix_pass(const uint64_t* __restrict__ in, uint64_t* __restrict__ out,
+                                                                uint64_t n, int shift, const uint32_t* __restrict__ hist,
+                                                                uint32_t* ticket, unsigned long long* state, uint32_t pass) {
+    extern __shared__ __align__(16) unsigned char raw[];
+    SortShared& S = *reinterpret_cast<SortShared*>(raw);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const uint32_t lt_mask = (1u << lane) - 1u;
-    uint64_t base = (uint64_t)blockIdx.x * kSortTile;
-
-    uint32_t c = counts[(uint64_t)tid * tiles + blockIdx.x];
-    uint32_t tot;
-    s_start[tid] = block_excl_scan<uint32_t>(c, &tot);
-    s_run[tid] = 0;
-    __syncthreads();
-
-    // the thread's keys of all rounds, loaded together (coalesced, one tile in flight)
-    uint64_t kr[kSortRounds];
-#pragma unroll
-    for (int r = 0; r < kSortRounds; ++r) {
-        uint64_t i = base + (uint64_t)r * kSortThreads + tid;
-        kr[r] = i < n ? in[i] : 0ull;
+    if (tid == 0) {
+        S.tile = atomicAdd(ticket, 1u);
+        S.gave_up = 0u;
     }
+    for (int k = tid; k < kSortWarps * 256; k += kSortThreads) (&S.wh[0][0])[k] = 0u;
+    __syncthreads();
+    const uint32_t tile = S.tile;
+    const uint64_t base = (uint64_t)tile * kSortTile, wbase = base + (uint64_t)warp * (32 * kSortPer);
+    const uint32_t tile_n = n - base < (uint64_t)kSortTile ? (uint32_t)(n - base) : (uint32_t)kSortTile;
+    // keys past the end read as all ones: the last of the last digit, never written
+    uint64_t key[kSortPer];
 #pragma unroll
-    for (int r = 0; r < kSortRounds; ++r) {
-        uint64_t i = base + (uint64_t)r * kSortThreads + tid;
-        bool valid = i < n;
-        uint64_t k = kr[r];
-        uint32_t d = (uint32_t)(k >> shift) & 255u;
+    for (int r = 0; r < kSortPer; ++r) {
+        const uint64_t i = wbase + 32 * r + lane;
+        key[r] = i < n ? in[i] : ~0ull;
+    }
+    uint32_t rank[kSortPer / 2];   // 16 bits each: the key's place among its warp's keys of its digit
 #pragma unroll
-        for (int q = 0; q < 8; ++q) s_wc[warp][lane + 32 * q] = 0;
-        __syncwarp();
-        uint32_t peers = __ballot_sync(0xffffffffu, valid);
+    for (int r = 0; r < kSortPer; ++r) {
+        const uint32_t d = (uint32_t)(key[r] >> shift) & 255u;
+        uint32_t peers = 0xffffffffu;
 #pragma unroll
         for (int b = 0; b < 8; ++b) {
-            uint32_t bal = __ballot_sync(0xffffffffu, (d >> b) & 1u);
+            const uint32_t bal = __ballot_sync(0xffffffffu, (d >> b) & 1u);
             peers &= ((d >> b) & 1u) ? bal : ~bal;
         }
-        uint32_t rank = __popc(peers & lt_mask);
-        if (valid && rank == 0) s_wc[warp][d] = __popc(peers);
-        __syncthreads();
-        {
-            uint32_t run = s_run[tid];
-#pragma unroll
-            for (int w = 0; w < kSortThreads / 32; ++w) {
-                uint32_t cw = s_wc[w][tid];
-                s_wc[w][tid] = run;
-                run += cw;
-            }
-            s_run[tid] = run;
-        }
-        __syncthreads();
-        if (valid) s_keys[s_start[d] + s_wc[warp][d] + rank] = k;
-        __syncthreads();
+        const uint32_t before = S.wh[warp][d];
+        __syncwarp();
+        if ((peers & lt_mask) == 0u) S.wh[warp][d] = before + __popc(peers);
+        __syncwarp();
+        const uint32_t k = before + __popc(peers & lt_mask);
+        if (r & 1) rank[r / 2] |= k << 16;
+        else rank[r / 2] = k;
     }
-    uint64_t rem = n - base;
-    uint32_t tile_n = rem < (uint64_t)kSortTile ? (uint32_t)rem : (uint32_t)kSortTile;
+    __syncthreads();
+    const unsigned long long mark = (unsigned long long)(pass + 1u) << 32;
+    uint32_t count = 0, first = 0;
+    if (tid < 256) {
+#pragma unroll
+        for (int w = 0; w < kSortWarps; ++w) {
+            const uint32_t c = S.wh[w][tid];
+            S.wh[w][tid] = count;
+            count += c;
+        }
+    }
+    const uint32_t all = count;
+    if (tid == 255) count -= (uint32_t)kSortTile - tile_n;
+    if (tid < 256) post(&state[256ull * tile + tid], (tile ? kOwn : kUpTo) | mark | count);
+    uint32_t unused;
+    const uint32_t start = block_excl_scan<uint32_t>(all, &unused);
+    const uint32_t digit0 = block_excl_scan<uint32_t>(tid < 256 ? hist[tid] : 0u, &unused);
+    if (tid < 256) S.start[tid] = start;
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < kSortPer; ++r) {
+        const uint32_t d = (uint32_t)(key[r] >> shift) & 255u;
+        S.keys[S.start[d] + S.wh[warp][d] + ((rank[r / 2] >> (16 * (r & 1))) & 0xffffu)] = key[r];
+    }
+    if (tid < 256) {
+        bool waits = tile != 0u;
+        for (uint64_t t = tile; waits;) {
+            --t;
+            unsigned long long v;
+            uint32_t looks = 0;
+            while (((v = peek(&state[256ull * t + tid])) & (0xffull << 32)) != mark && ++looks < kPatience) {}
+            if (looks == kPatience) {
+                S.gave_up = 1u;
+                break;
+            }
+            first += (uint32_t)v;
+            waits = v < kUpTo;   // tile 0's sum is inclusive
+        }
+    }
+    __syncthreads();
+    if (S.gave_up) {   // uniform: count the predecessors' keys themselves
+        uint32_t* h = &S.wh[0][0];
+        if (tid < 256) h[tid] = 0u;
+        __syncthreads();
+        for (uint64_t i = tid; i < base; i += kSortThreads) atomicAdd(&h[(uint32_t)(in[i] >> shift) & 255u], 1u);
+        __syncthreads();
+        if (tid < 256) first = h[tid];
+    }
+    if (tid < 256) {
+        if (tile) post(&state[256ull * tile + tid], kUpTo | mark | (uint32_t)(first + count));
+        S.to[tid] = digit0 + first - start;
+    }
+    __syncthreads();
     for (uint32_t i = tid; i < tile_n; i += kSortThreads) {
-        uint64_t k = s_keys[i];
-        uint32_t d = (uint32_t)(k >> shift) & 255u;
-        out[(uint64_t)offs[(uint64_t)d * tiles + blockIdx.x] + (i - s_start[d])] = k;
+        const uint64_t k = S.keys[i];
+        out[(uint32_t)(S.to[(uint32_t)(k >> shift) & 255u] + i)] = k;
     }
 }
 
@@ -231,18 +324,24 @@ tc_status scan_u32_to_u64(const uint32_t* in, uint64_t* out, uint64_t n, cudaStr
 tc_status radix_sort_u64(uint64_t** keys, uint64_t** tmp, uint64_t n, int lo_bit, int hi_bit, cudaStream_t st) {
     if (n <= 1 || hi_bit <= lo_bit) return TC_OK;
     if (n >= (1ull << 32)) return fail(TC_ERR_RANGE, "radix sort: more than 2^32-1 keys");
-    uint64_t tiles64 = (n + kSortTile - 1) / kSortTile;
-    uint32_t tiles = (uint32_t)tiles64;
-    DevBuf counts, offs;
-    TC_TRY(counts.alloc(sizeof(uint32_t) * 256ull * tiles, st));
-    TC_TRY(offs.alloc(sizeof(uint32_t) * 256ull * tiles, st));
-    for (int sh = lo_bit; sh < hi_bit; sh += 8) {
-        k_radix_hist<<<tiles, kSortThreads, 0, st>>>(*keys, n, sh, counts.as<uint32_t>(), tiles);
-        TC_LAUNCH("k_radix_hist");
-        TC_TRY(scan_u32(counts.as<uint32_t>(), offs.as<uint32_t>(), 256ull * tiles, nullptr, st));
-        k_radix_scatter<<<tiles, kSortThreads, 0, st>>>(*keys, *tmp, n, sh, counts.as<uint32_t>(),
-                                                        offs.as<uint32_t>(), tiles);
-        TC_LAUNCH("k_radix_scatter");
+    const int passes = (hi_bit - lo_bit + 7) / 8;
+    if (passes > kPasses) return fail(TC_ERR_ARG, "radix sort: more than 64 bits");
+    const uint64_t tiles = (n + kSortTile - 1) / kSortTile;
+    // a count per digit and a ticket per pass, then the tiles' sums
+    const size_t counts = sizeof(uint32_t) * 257ull * kPasses;
+    DevBuf work;
+    TC_TRY(work.alloc(counts + sizeof(unsigned long long) * 256ull * tiles, st));
+    TC_CUDA(cudaMemsetAsync(work.p, 0, work.bytes, st));
+    uint32_t* hist = work.as<uint32_t>();
+    uint32_t* ticket = hist + 256 * kPasses;
+    unsigned long long* state = reinterpret_cast<unsigned long long*>(work.as<unsigned char>() + counts);
+    k_digit_counts<<<grid_for(n, kSortThreads * 4, 4u * (unsigned)sm_count()), kSortThreads, 0, st>>>(*keys, n, lo_bit, passes, hist);
+    TC_LAUNCH("k_digit_counts");
+    TC_CUDA(cudaFuncSetAttribute((const void*)k_radix_pass, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SortShared)));
+    for (int p = 0; p < passes; ++p) {
+        k_radix_pass<<<(unsigned)tiles, kSortThreads, sizeof(SortShared), st>>>(*keys, *tmp, n, lo_bit + 8 * p, hist + 256 * p,
+                                                                              ticket + p, state, (uint32_t)p);
+        TC_LAUNCH("k_radix_pass");
         std::swap(*keys, *tmp);
     }
     return TC_OK;
