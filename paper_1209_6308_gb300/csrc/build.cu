@@ -12,6 +12,7 @@
 #include <algorithm>
 
 #include "graph.cuh"
+#include "rows.cuh"
 #include "tc_internal.cuh"
 
 namespace tc {
@@ -137,17 +138,19 @@ __global__ void k_up(const uint64_t* off, const uint32_t* adj, uint32_t n, uint3
 
 // stats[3] sum deg^2, stats[4] sum over upper pairs of deg(v), stats[5] max degree,
 // stats[7] vertices with deg > 0, stats[10] sum of up (up - 1) / 2 (the entries the triangle form
-// walks: for every upper pair (b, c), the neighbours of c below b), stats[11] vertices with deg > kHubDeg
+// walks: for every upper pair (b, c), the neighbours of c below b), stats[11] vertices with deg > kHubDeg,
+// stats[12] vertices with deg > 32
 __global__ void k_graph_sums(const uint64_t* off, const uint32_t* adj, const uint32_t* up, uint32_t n,
                              unsigned long long* stats) {
     unsigned long long d2 = 0, dv = 0, tw = 0;
-    uint32_t mx = 0, act = 0, hub = 0;
+    uint32_t mx = 0, act = 0, hub = 0, wide = 0;
     for (uint64_t x = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; x < n; x += (uint64_t)gridDim.x * blockDim.x) {
         uint64_t d = off[x + 1] - off[x];
         d2 += d * d;
         mx = max(mx, (uint32_t)d);
         act += (d > 0);
         hub += (d > kHubDeg);
+        wide += (d > 32);
         // x is the v of every pair (u, x) with u < x: the first up[x] neighbours
         dv += (unsigned long long)up[x] * d;
         tw += (unsigned long long)up[x] * (up[x] ? up[x] - 1ull : 0ull) / 2ull;
@@ -159,10 +162,12 @@ __global__ void k_graph_sums(const uint64_t* off, const uint32_t* adj, const uin
         mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
         act += __shfl_xor_sync(0xffffffffu, act, o);
         hub += __shfl_xor_sync(0xffffffffu, hub, o);
+        wide += __shfl_xor_sync(0xffffffffu, wide, o);
     }
     if ((threadIdx.x & 31) == 0) {
         if (act) atomicAdd(&stats[7], (unsigned long long)act);
         if (hub) atomicAdd(&stats[11], (unsigned long long)hub);
+        if (wide) atomicAdd(&stats[12], (unsigned long long)wide);
         atomicAdd(&stats[3], d2);
         atomicAdd(&stats[4], dv);
         atomicAdd(&stats[10], tw);
@@ -173,42 +178,47 @@ __global__ void k_graph_sums(const uint64_t* off, const uint32_t* adj, const uin
 constexpr uint32_t kLongList = 4096;   // longer lists: k_pair_tables_long, a CTA per vertex
 constexpr int kLongThreads = 1024;
 
-// Per upper pair tables.  One warp per vertex v (lists of at most kLongList entries; longer ones
-// are k_pair_tables_long's) takes N[v] in 32-entry blocks from the end,
-// keeping running counts of the direction classes of the entries behind the block and adding,
-// per lane, the block's entries after its own by ballot: so the lane at position k knows the
-// counts of the entries after k.  At a lower neighbour u = N[v][k] (k < up[v]) those are the
-// third vertices w > u reached from v: the lane writes them to sfx[lb[v] + k] (lb[v] = the
-// lower entries of the vertices before v), where k_pair_rp picks them up for the upper pair
-// (u, v).  At an upper neighbour
-// (k >= up[v]) they are the third vertices w > N[v][k] reached from v, the u side of the pair
-// (v, N[v][k]): us = (class-1, class-2 counts).  wk[0] += the suffix lengths at lower
-// neighbours (the N[v] entries a census walks), wk[1] += those of them with ids below
-// kMapIdsSuffix: with c the entries of N[v] below it (a prefix), the walk past position k
-// meets max(0, c - k - 1) of them.
-__global__ void k_pair_tables(const uint64_t* __restrict__ off, const uint32_t* __restrict__ adj,
+// Per upper pair tables, lists of at most kLongList entries (longer ones are k_pair_tables_long's).
+// The lane at position k of N[v] counts the direction classes of the entries after k.  At a lower
+// neighbour u = N[v][k] (k < up[v]) those are the third vertices w > u reached from v: the lane
+// writes them to sfx[lb[v] + k] (lb[v] = the lower entries of the vertices before v), where
+// k_pair_rp picks them up for the upper pair (u, v).  At an upper neighbour (k >= up[v]) they are
+// the third vertices w > N[v][k] reached from v, the u side of the pair (v, N[v][k]): us = (class-1,
+// class-2 counts).  wk[0] += the suffix lengths at lower neighbours (the N[v] entries a census
+// walks), wk[1] += those of them with ids below kMapIdsSuffix: with c the entries of N[v] below it
+// (a prefix), the walk past position k meets max(0, c - k - 1) of them.
+// The n_wide lists of more than 32 entries go a warp each, in 32-entry blocks from the end with
+// running counts; for the others a warp takes 32 vertices (rows.cuh) whose lists share its lanes
+// and are counted by one ballot per class.
+// Bound by its table writes and, per warp, by the loads' latency: at scale 20 a warp per vertex
+// took 0.68 ms.
+__global__ void __launch_bounds__(kB) k_pair_tables(const uint64_t* __restrict__ off, const uint32_t* __restrict__ adj,
                               const uint32_t* __restrict__ up, const uint64_t* __restrict__ ub,
-                              const uint64_t* __restrict__ lb, uint32_t n, uint2* sfx, uint2* us,
+                              const uint64_t* __restrict__ lb, uint32_t n,
+                              const unsigned long long* __restrict__ n_wide, uint2* sfx, uint2* us,
                               unsigned long long* wk) {
+    __shared__ uint8_t s_at[kB / 32][32];
     const uint32_t lane = threadIdx.x & 31;
-    const uint64_t warps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
     const uint32_t after = lane == 31 ? 0u : ~((2u << lane) - 1u);   // lanes above this one
+    const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
     unsigned long long walk = 0, walk_map = 0;
-    for (uint64_t v = (blockIdx.x * (uint64_t)blockDim.x + threadIdx.x) >> 5; v < n; v += warps) {
-        const uint64_t ob = off[v];
+    // the lists of more than 32 entries, a prefix of the ids, a warp each
+    const uint64_t wide = *n_wide;
+    for (uint64_t v = (blockIdx.x * (uint64_t)blockDim.x + threadIdx.x) >> 5; v < wide; v += stride >> 5) {
+        const uint64_t ob = off[v], ubv = ub[v], lbv = lb[v];
         const uint32_t dv = (uint32_t)(off[v + 1] - ob), lv = up[v];
         if (dv > kLongList) continue;                                 // k_pair_tables_long's
         uint32_t c1 = 0, c2 = 0, cmap = 0;
-        for (uint32_t cs = dv & ~31u; dv && cs <= dv; cs -= 32) {   // blocks from the last one down
+        for (uint32_t cs = dv & ~31u; cs <= dv; cs -= 32) {   // blocks from the last one down
             const uint32_t k = cs + lane;
             const uint32_t e = k < dv ? adj[ob + k] : 0u;
             const uint32_t b1 = __ballot_sync(0xffffffffu, (e & 3u) == 1u);
             const uint32_t b2 = __ballot_sync(0xffffffffu, (e & 3u) == 2u);
             if (k < lv) {
-                sfx[lb[v] + k] = make_uint2(c1 + __popc(b1 & after), c2 + __popc(b2 & after));
+                sfx[lbv + k] = make_uint2(c1 + __popc(b1 & after), c2 + __popc(b2 & after));
                 walk += dv - k - 1;
             } else if (k < dv) {
-                us[ub[v] + (k - lv)] = make_uint2(c1 + __popc(b1 & after), c2 + __popc(b2 & after));
+                us[ubv + (k - lv)] = make_uint2(c1 + __popc(b1 & after), c2 + __popc(b2 & after));
             }
             c1 += __popc(b1);
             c2 += __popc(b2);
@@ -218,7 +228,35 @@ __global__ void k_pair_tables(const uint64_t* __restrict__ off, const uint32_t* 
         const unsigned long long m = min(lv, cmap);
         if (lane == 0) walk_map += m * cmap - m * (m + 1) / 2;
     }
+    for (uint64_t x0 = wide + blockIdx.x * (uint64_t)blockDim.x + (threadIdx.x & ~31u); x0 < n; x0 += stride) {
+        const uint64_t x = x0 + lane;
+        const bool ok = x < n;
+        const uint64_t vob = ok ? off[x] : 0ull, vub = ok ? ub[x] : 0ull, vlb = ok ? lb[x] : 0ull;
+        const uint32_t vd = ok ? (uint32_t)(off[x + 1] - vob) : 0u, vl = ok ? up[x] : 0u;
+        for_rows(vd, s_at[threadIdx.x >> 5],
+            [&](const PackedEntry& p) {
+                const uint64_t ob = __shfl_sync(0xffffffffu, vob, p.row), ubv = __shfl_sync(0xffffffffu, vub, p.row);
+                const uint64_t lbv = __shfl_sync(0xffffffffu, vlb, p.row);
+                const uint32_t dv = __shfl_sync(0xffffffffu, vd, p.row), lv = __shfl_sync(0xffffffffu, vl, p.row);
+                const uint32_t k = lane - p.first;
+                const uint32_t e = p.valid ? adj[ob + k] : 0u;
+                const uint32_t m1 = __ballot_sync(0xffffffffu, (e & 3u) == 1u) & p.lanes;
+                const uint32_t m2 = __ballot_sync(0xffffffffu, (e & 3u) == 2u) & p.lanes;
+                const uint32_t mm = __ballot_sync(0xffffffffu, p.valid && (e >> 2) < kMapIdsSuffix) & p.lanes;
+                const uint2 c = make_uint2(__popc(m1 & after), __popc(m2 & after));
+                if (p.valid && k < lv) {
+                    sfx[lbv + k] = c;
+                    walk += dv - k - 1;
+                    const uint32_t cmap = __popc(mm);
+                    walk_map += cmap > k ? cmap - k - 1u : 0u;
+                } else if (p.valid) {
+                    us[ubv + (k - lv)] = c;
+                }
+            },
+            [](uint32_t) {});
+    }
     for (int o = 16; o; o >>= 1) walk += __shfl_xor_sync(0xffffffffu, walk, o);
+    for (int o = 16; o; o >>= 1) walk_map += __shfl_xor_sync(0xffffffffu, walk_map, o);
     if (lane == 0 && walk) atomicAdd(wk, walk);
     if (lane == 0 && walk_map) atomicAdd(wk + 1, walk_map);
 }
@@ -313,32 +351,62 @@ __device__ __forceinline__ uint32_t lower_position(const uint32_t* __restrict__ 
     return lo;
 }
 
-// rp and vs of the upper pairs of u: for pair (u, v = N[u][j]), rp = the position k of u in
-// N[v] and vs = sfx[lb[v] + k] (the class counts of N[v] past u, from k_pair_tables).  Entries
-// j of each upper list in order, so the table writes are coalesced.  The upper pairs of one
-// vertex u go to one warp (lists of at most kLongList entries) or, for longer lists, to one
-// CTA (rp_long; those vertices are a prefix of the ids).
-template <bool LONG>
-__global__ void k_pair_rp(const uint64_t* __restrict__ off, const uint32_t* __restrict__ adj,
+// rp and vs of one upper pair (u, v = N[u][j]), table index p: rp = the position k of u in N[v],
+// vs = sfx[lb[v] + k] (the class counts of N[v] past u, from k_pair_tables).
+__device__ __forceinline__ void pair_rp(const uint64_t* __restrict__ off, const uint32_t* __restrict__ adj,
+                                        const uint32_t* __restrict__ up, const uint64_t* __restrict__ lb,
+                                        const uint2* __restrict__ sfx, uint32_t u, uint32_t v, uint64_t p, uint32_t* rp,
+                                        uint2* vs) {
+    const uint32_t k = lower_position(adj + off[v], up[v], u);
+    rp[p] = k;
+    vs[p] = sfx[lb[v] + k];
+}
+
+// The tables of the upper pairs, each upper list in order, so the table writes are coalesced: a
+// warp per vertex of more than 32 neighbours (n_wide, a prefix of the ids; above kLongList they are
+// k_pair_rp_long's), a warp per 32 vertices for the others, whose upper lists share its lanes
+// (rows.cuh).
+__global__ void __launch_bounds__(kB) k_pair_rp(const uint64_t* __restrict__ off, const uint32_t* __restrict__ adj,
                           const uint32_t* __restrict__ up, const uint64_t* __restrict__ ub,
-                          const uint64_t* __restrict__ lb, const uint2* __restrict__ sfx, uint32_t n, uint32_t* rp,
-                          uint2* vs) {
-    const uint32_t lanes = LONG ? blockDim.x : 32u;
-    const uint32_t lane = LONG ? threadIdx.x : (threadIdx.x & 31u);
-    // LONG: one CTA per vertex of the prefix the grid covers (the long lists are among them)
-    const uint64_t stride = LONG ? n : ((uint64_t)gridDim.x * blockDim.x) >> 5;
-    for (uint64_t u = LONG ? blockIdx.x : (blockIdx.x * (uint64_t)blockDim.x + threadIdx.x) >> 5; u < n; u += stride) {
-        const uint64_t ob = off[u];
+                          const uint64_t* __restrict__ lb, const uint2* __restrict__ sfx, uint32_t n,
+                          const unsigned long long* __restrict__ n_wide, uint32_t* rp, uint2* vs) {
+    __shared__ uint8_t s_at[kB / 32][32];
+    const uint32_t lane = threadIdx.x & 31;
+    const uint64_t stride = (uint64_t)gridDim.x * blockDim.x, wide = *n_wide;
+    for (uint64_t u = (blockIdx.x * (uint64_t)blockDim.x + threadIdx.x) >> 5; u < wide; u += stride >> 5) {
+        const uint64_t ob = off[u], tb = ub[u];
         const uint32_t du = (uint32_t)(off[u + 1] - ob), upu = up[u];
-        if ((du > kLongList) != LONG) continue;      // uniform over the warp / CTA
-        const uint64_t tb = ub[u];
-        for (uint32_t j = upu + lane; j < du; j += lanes) {
-            const uint32_t v = adj[ob + j] >> 2;
-            const uint32_t k = lower_position(adj + off[v], up[v], (uint32_t)u);
-            rp[tb + (j - upu)] = k;
-            vs[tb + (j - upu)] = sfx[lb[v] + k];
-        }
+        if (du > kLongList) continue;                                 // k_pair_rp_long's
+        for (uint32_t j = upu + lane; j < du; j += 32)
+            pair_rp(off, adj, up, lb, sfx, (uint32_t)u, adj[ob + j] >> 2, tb + (j - upu), rp, vs);
     }
+    for (uint64_t x0 = wide + blockIdx.x * (uint64_t)blockDim.x + (threadIdx.x & ~31u); x0 < n; x0 += stride) {
+        const uint64_t x = x0 + lane;
+        const bool ok = x < n;
+        const uint64_t vob = ok ? off[x] : 0ull, vub = ok ? ub[x] : 0ull;
+        const uint32_t vd = ok ? (uint32_t)(off[x + 1] - vob) : 0u, vl = ok ? up[x] : 0u;
+        for_rows(vd - vl, s_at[threadIdx.x >> 5],
+            [&](const PackedEntry& p) {
+                const uint64_t first = __shfl_sync(0xffffffffu, vob + vl, p.row), ubu = __shfl_sync(0xffffffffu, vub, p.row);
+                const uint32_t k = lane - p.first;
+                if (p.valid) pair_rp(off, adj, up, lb, sfx, (uint32_t)x0 + p.row, adj[first + k] >> 2, ubu + k, rp, vs);
+            },
+            [](uint32_t) {});
+    }
+}
+
+// One CTA per vertex of the prefix of the ids that holds the long lists.
+__global__ void k_pair_rp_long(const uint64_t* __restrict__ off, const uint32_t* __restrict__ adj,
+                               const uint32_t* __restrict__ up, const uint64_t* __restrict__ ub,
+                               const uint64_t* __restrict__ lb, const uint2* __restrict__ sfx, uint32_t n, uint32_t* rp,
+                               uint2* vs) {
+    const uint64_t u = blockIdx.x;
+    if (u >= n) return;
+    const uint64_t ob = off[u];
+    const uint32_t du = (uint32_t)(off[u + 1] - ob), upu = up[u];
+    if (du <= kLongList) return;
+    for (uint32_t j = upu + threadIdx.x; j < du; j += blockDim.x)
+        pair_rp(off, adj, up, lb, sfx, (uint32_t)u, adj[ob + j] >> 2, ub[u] + (j - upu), rp, vs);
 }
 
 // upper pairs per vertex: deg - up
@@ -472,9 +540,10 @@ tc_status finish_graph(GraphStore& g, uint64_t E, int B, uint64_t* ukey, uint32_
             TC_TRY(sfx.alloc(sizeof(uint2) * E, st));
             TC_TRY(scan_u32_to_u64(g.up.as<uint32_t>(), lb.as<uint64_t>(), n, st));
             // the walk lengths go to stats[8..9]
-            k_pair_tables<<<grid_for((uint64_t)n * 32, kB, 1u << 16), kB, 0, st>>>(
+            k_pair_tables<<<grid_for(n, kB, 1u << 16), kB, 0, st>>>(
                 g.off.as<uint64_t>(), g.adj.as<uint32_t>(), g.up.as<uint32_t>(), g.ub.as<uint64_t>(),
-                lb.as<uint64_t>(), n, sfx.as<uint2>(), g.us.as<uint2>(), stats.as<unsigned long long>() + 8);
+                lb.as<uint64_t>(), n, stats.as<unsigned long long>() + 12, sfx.as<uint2>(), g.us.as<uint2>(),
+                stats.as<unsigned long long>() + 8);
             TC_LAUNCH("k_pair_tables");
             // lists longer than kLongList: at most 2E / kLongList of them, the first ids
             const uint64_t n_long = std::min<uint64_t>(n, 2ull * E / kLongList + 1);
@@ -482,21 +551,23 @@ tc_status finish_graph(GraphStore& g, uint64_t E, int B, uint64_t* ukey, uint32_
                 g.off.as<uint64_t>(), g.adj.as<uint32_t>(), g.up.as<uint32_t>(), g.ub.as<uint64_t>(),
                 lb.as<uint64_t>(), n, sfx.as<uint2>(), g.us.as<uint2>(), stats.as<unsigned long long>() + 8);
             TC_LAUNCH("k_pair_tables_long");
-            k_pair_rp<false><<<grid_for((uint64_t)n * 32, kB, 1u << 16), kB, 0, st>>>(
+            k_pair_rp<<<grid_for(n, kB, 1u << 16), kB, 0, st>>>(
                 g.off.as<uint64_t>(), g.adj.as<uint32_t>(), g.up.as<uint32_t>(), g.ub.as<uint64_t>(),
-                lb.as<uint64_t>(), sfx.as<uint2>(), n, g.rp.as<uint32_t>(), g.vs.as<uint2>());
+                lb.as<uint64_t>(), sfx.as<uint2>(), n, stats.as<unsigned long long>() + 12, g.rp.as<uint32_t>(),
+                g.vs.as<uint2>());
             TC_LAUNCH("k_pair_rp");
-            k_pair_rp<true><<<(unsigned)n_long, kLongThreads, 0, st>>>(
+            k_pair_rp_long<<<(unsigned)n_long, kLongThreads, 0, st>>>(
                 g.off.as<uint64_t>(), g.adj.as<uint32_t>(), g.up.as<uint32_t>(), g.ub.as<uint64_t>(),
                 lb.as<uint64_t>(), sfx.as<uint2>(), n, g.rp.as<uint32_t>(), g.vs.as<uint2>());
             TC_LAUNCH("k_pair_rp_long");
         }
     }
-    unsigned long long hs[12];
+    unsigned long long hs[13];
     TC_CUDA(cudaMemcpyAsync(hs, stats.p, sizeof(hs), cudaMemcpyDeviceToHost, st));
     TC_CUDA(cudaStreamSynchronize(st));
     g.sum_tri_walk = hs[10];
     g.n_hub = (uint32_t)hs[11];
+    g.n_wide = (uint32_t)hs[12];
     g.sum_walk = hs[8];
     g.sum_walk_map = hs[9];
     g.e_sym = E;
@@ -568,8 +639,8 @@ tc_status build_from_arcs(GraphStore& g, uint64_t m, const uint32_t* d_src, cons
     const int B = bits_for(n);
     if (m >= (1ull << 32)) return fail(TC_ERR_RANGE, "more than 2^32-1 arcs");
     DevBuf stats, keys, tmp;
-    TC_TRY(stats.alloc(sizeof(unsigned long long) * 12, st));
-    TC_CUDA(cudaMemsetAsync(stats.p, 0, sizeof(unsigned long long) * 12, st));
+    TC_TRY(stats.alloc(sizeof(unsigned long long) * 13, st));
+    TC_CUDA(cudaMemsetAsync(stats.p, 0, sizeof(unsigned long long) * 13, st));
     TC_TRY(keys.alloc(sizeof(uint64_t) * (m ? m : 1), st));
     TC_TRY(tmp.alloc(sizeof(uint64_t) * (m ? m : 1), st));
     if (m) {
@@ -600,8 +671,8 @@ tc_status build_from_sorted_arcs(GraphStore& g, const uint64_t* d_keys, uint64_t
     const int B = bits_for(g.n);
     if (m >= (1ull << 32)) return fail(TC_ERR_RANGE, "more than 2^32-1 arcs");
     DevBuf stats, ukey, udir;
-    TC_TRY(stats.alloc(sizeof(unsigned long long) * 12, st));
-    TC_CUDA(cudaMemsetAsync(stats.p, 0, sizeof(unsigned long long) * 12, st));
+    TC_TRY(stats.alloc(sizeof(unsigned long long) * 13, st));
+    TC_CUDA(cudaMemsetAsync(stats.p, 0, sizeof(unsigned long long) * 13, st));
     uint32_t E = 0;
     TC_TRY(pairs_from_sorted(d_keys, m, ukey, udir, E, st));
     TC_TRY(graph_from_pairs(g, B, E, ukey, udir, stats, st));
@@ -620,8 +691,8 @@ tc_status build_from_csr(GraphStore& g, const uint64_t* d_off, const uint32_t* d
     if (total_h & 1) return fail(TC_ERR_ARG, "CSR is not symmetric (odd number of entries)");
     if (total_h >= (1ull << 32)) return fail(TC_ERR_RANGE, "more than 2^32-1 CSR entries");
     DevBuf stats;
-    TC_TRY(stats.alloc(sizeof(unsigned long long) * 12, st));
-    TC_CUDA(cudaMemsetAsync(stats.p, 0, sizeof(unsigned long long) * 12, st));
+    TC_TRY(stats.alloc(sizeof(unsigned long long) * 13, st));
+    TC_CUDA(cudaMemsetAsync(stats.p, 0, sizeof(unsigned long long) * 13, st));
     const unsigned gridN = grid_for(n, kB, 1u << 16);
     k_check_csr<<<gridN, kB, 0, st>>>(d_off, d_adj, n, total_h, stats.as<unsigned long long>());
     TC_LAUNCH("k_check_csr");

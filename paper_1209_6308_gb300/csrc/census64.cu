@@ -19,10 +19,12 @@
 //   - no link: C(n,3) less the rest (128-bit).
 // The sorted neighbour lists in caller ids come from one radix sort of (caller id of the row,
 // caller id of the neighbour) keys of the stored lists.
+#include <algorithm>
 #include <cstring>
 #include <vector>
 
 #include "graph.cuh"
+#include "rows.cuh"
 
 namespace tc {
 namespace {
@@ -43,17 +45,45 @@ __global__ void k_deg_old(const uint64_t* __restrict__ off, const uint32_t* __re
 }
 
 // One key per stored entry (row r, neighbour s): (old[r] << (B + 2)) | (old[s] << 2) | dir, with
-// dir seen from r (1 r->s, 2 s->r).  One warp per row.
-__global__ void k_keys64(GraphDev g, const uint32_t* __restrict__ old, int B, uint64_t* keys) {
+// dir seen from r (1 r->s, 2 s->r).  The entries of the n_wide rows of more than 32 come first:
+// kKeyChunk of them to a warp; then a warp takes 32 rows (rows.cuh).
+constexpr uint32_t kKeyChunk = 1024;
+__global__ void __launch_bounds__(256) k_keys64(GraphDev g, uint32_t n_wide, const uint32_t* __restrict__ old, int B,
+                                                uint64_t* keys) {
+    __shared__ uint8_t s_at[8][32];
     const uint32_t lane = threadIdx.x & 31;
-    const uint64_t warps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
-    for (uint64_t r = (blockIdx.x * (uint64_t)blockDim.x + threadIdx.x) >> 5; r < g.n; r += warps) {
-        const uint64_t b = g.off[r], e = g.off[r + 1];
-        const uint64_t hi = (uint64_t)old[r] << (B + 2);
-        for (uint64_t k = b + lane; k < e; k += 32) {
-            const uint32_t x = g.adj[k];
-            keys[k] = hi | ((uint64_t)old[x >> 2] << 2) | (x & 3u);
+    const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
+    auto put = [&](uint64_t row, uint64_t k) {
+        const uint32_t x = g.adj[k];
+        keys[k] = row << (B + 2) | ((uint64_t)old[x >> 2] << 2) | (x & 3u);
+    };
+    const uint64_t wide = g.off[n_wide];
+    for (uint64_t k0 = ((blockIdx.x * (uint64_t)blockDim.x + threadIdx.x) >> 5) * kKeyChunk; k0 < wide;
+         k0 += (stride >> 5) * kKeyChunk) {
+        const uint64_t end = k0 + kKeyChunk < wide ? k0 + kKeyChunk : wide;
+        uint32_t r = 0, hi = n_wide;   // the row of entry k0: the last one with off <= k0
+        while (hi - r > 1u) {
+            const uint32_t mid = (r + hi) >> 1;
+            if (g.off[mid] <= k0) r = mid;
+            else hi = mid;
         }
+        for (uint64_t k = k0; k < end; ++r) {
+            const uint64_t e = g.off[r + 1] < end ? g.off[r + 1] : end, row = old[r];
+#pragma unroll 4
+            for (uint64_t i = k + lane; i < e; i += 32) put(row, i);
+            k = e;
+        }
+    }
+    for (uint64_t x0 = n_wide + blockIdx.x * (uint64_t)blockDim.x + (threadIdx.x & ~31u); x0 < g.n; x0 += stride) {
+        const bool ok = x0 + lane < g.n;
+        const uint64_t base = ok ? g.off[x0 + lane] : 0ull;
+        const uint32_t deg = ok ? (uint32_t)(g.off[x0 + lane + 1] - base) : 0u, mine = ok ? old[x0 + lane] : 0u;
+        for_rows(deg, s_at[threadIdx.x >> 5],
+            [&](const PackedEntry& p) {
+                const uint64_t row = __shfl_sync(0xffffffffu, mine, p.row), b = __shfl_sync(0xffffffffu, base, p.row);
+                if (p.valid) put(row, b + (lane - p.first));
+            },
+            [](uint32_t) {});
     }
 }
 
@@ -63,42 +93,41 @@ __global__ void k_keys64(GraphDev g, const uint32_t* __restrict__ old, int B, ui
 //   raw[18..27) X:  (neighbours below c of class d1) x (above c of class d2)  (c is y)
 //   raw[27..36) R:  per pair (a, b), a < b, of direction class k = d1 (1 a->b, 2 b->a, 3 both):
 //               position d2 = 1 above b (n - 1 - b), 2 between (b - a - 1), 3 below a (a)
-// Classes are seen from c (1 c->nbr, 2 nbr->c).  One warp per vertex (caller ids).
-__global__ void k_wedges64(const uint64_t* __restrict__ keys, const uint64_t* __restrict__ off_old, uint32_t n, int B,
-                           unsigned long long* raw) {
+// Classes are seen from c (1 c->nbr, 2 nbr->c).  A warp over 32 vertices (caller ids, rows.cuh):
+// per entry, the earlier entries of its row by side and class.
+__global__ void __launch_bounds__(256) k_wedges64(const uint64_t* __restrict__ keys, const uint64_t* __restrict__ off_old,
+                                                  uint32_t n, int B, unsigned long long* raw) {
+    __shared__ uint8_t s_at[8][32];
     const uint32_t lane = threadIdx.x & 31;
-    const uint64_t warps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
     const uint64_t idmask = (1ull << B) - 1ull;
     const uint32_t lt = (1u << lane) - 1u;
+    const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
     unsigned long long pb[3][3], pa[3][3], xx[3][3], rr[3][3];
 #pragma unroll
     for (int i = 0; i < 3; ++i)
 #pragma unroll
         for (int j = 0; j < 3; ++j) pb[i][j] = pa[i][j] = xx[i][j] = rr[i][j] = 0ull;
-    for (uint64_t cx = (blockIdx.x * (uint64_t)blockDim.x + threadIdx.x) >> 5; cx < n; cx += warps) {
-        const uint32_t c = (uint32_t)cx;
-        const uint64_t kb = off_old[c], ke = off_old[c + 1];
-        uint32_t rb[3] = {0u, 0u, 0u}, ra[3] = {0u, 0u, 0u};
-        for (uint64_t k0 = kb; k0 < ke; k0 += 32) {
-            const uint64_t k = k0 + lane;
-            const bool valid = k < ke;
-            const uint64_t key = valid ? keys[k] : 0ull;
+    for (uint64_t x0 = blockIdx.x * (uint64_t)blockDim.x + (threadIdx.x & ~31u); x0 < n; x0 += stride) {
+        const bool ok = x0 + lane < n;
+        const uint64_t vb = ok ? off_old[x0 + lane] : 0ull;
+        const uint32_t vd = ok ? (uint32_t)(off_old[x0 + lane + 1] - vb) : 0u;
+        // one block of entries: this lane's key of centre c, its row's lanes, and the counts of the row's
+        // earlier blocks, which it advances
+        auto block = [&](bool valid, uint64_t key, uint32_t c, uint32_t lanes, uint32_t (&rb)[3], uint32_t (&ra)[3]) {
             const uint32_t nb = (uint32_t)((key >> 2) & idmask), d = (uint32_t)(key & 3ull);
             const bool below = valid && nb < c, above = valid && nb > c;
-            uint32_t bb[3], ba[3];
-#pragma unroll
-            for (int q = 0; q < 3; ++q) {
-                bb[q] = __ballot_sync(0xffffffffu, below && d == (uint32_t)(q + 1));
-                ba[q] = __ballot_sync(0xffffffffu, above && d == (uint32_t)(q + 1));
-            }
 #pragma unroll
             for (int q1 = 0; q1 < 3; ++q1) {
-                const uint32_t before_b = rb[q1] + __popc(bb[q1] & lt), before_a = ra[q1] + __popc(ba[q1] & lt);
+                const uint32_t bb = __ballot_sync(0xffffffffu, below && d == (uint32_t)(q1 + 1)) & lanes;
+                const uint32_t ba = __ballot_sync(0xffffffffu, above && d == (uint32_t)(q1 + 1)) & lanes;
+                const uint32_t before_b = rb[q1] + __popc(bb & lt), before_a = ra[q1] + __popc(ba & lt);
 #pragma unroll
                 for (int q2 = 0; q2 < 3; ++q2) {
                     if (below && d == (uint32_t)(q2 + 1)) pb[q1][q2] += before_b;
                     if (above && d == (uint32_t)(q2 + 1)) pa[q1][q2] += before_a;
                 }
+                rb[q1] += __popc(bb);
+                ra[q1] += __popc(ba);
             }
             if (above) {
                 const unsigned long long vals[3] = {(unsigned long long)n - 1ull - nb, (unsigned long long)(nb - c - 1u),
@@ -109,17 +138,34 @@ __global__ void k_wedges64(const uint64_t* __restrict__ keys, const uint64_t* __
 #pragma unroll
                         for (int q2 = 0; q2 < 3; ++q2) rr[q1][q2] += vals[q2];
             }
-#pragma unroll
-            for (int q = 0; q < 3; ++q) {
-                rb[q] += __popc(bb[q]);
-                ra[q] += __popc(ba[q]);
-            }
-        }
-        if (lane == 0)
+        };
+        auto products = [&](const uint32_t (&rb)[3], const uint32_t (&ra)[3]) {
 #pragma unroll
             for (int q1 = 0; q1 < 3; ++q1)
 #pragma unroll
                 for (int q2 = 0; q2 < 3; ++q2) xx[q1][q2] += (unsigned long long)rb[q1] * ra[q2];
+        };
+        for_rows(vd, s_at[threadIdx.x >> 5],
+            [&](const PackedEntry& p) {
+                const uint64_t b = __shfl_sync(0xffffffffu, vb, p.row);
+                uint32_t rb[3] = {0u, 0u, 0u}, ra[3] = {0u, 0u, 0u};
+                const uint64_t key = p.valid ? keys[b + (lane - p.first)] : 0ull;
+                block(p.valid, key, (uint32_t)x0 + p.row, p.lanes, rb, ra);
+                if (p.valid && lane == p.first) products(rb, ra);   // the row's totals
+            },
+            [&](uint32_t row) {
+                const uint64_t b = __shfl_sync(0xffffffffu, vb, row);
+                const uint32_t d = __shfl_sync(0xffffffffu, vd, row);
+                uint32_t rb[3] = {0u, 0u, 0u}, ra[3] = {0u, 0u, 0u};
+                uint64_t next = keys[b + lane];   // more than 32 entries
+                for (uint32_t k0 = 0; k0 < d; k0 += 32) {
+                    const uint64_t key = next;
+                    const uint32_t k = k0 + lane;
+                    next = k + 32u < d ? keys[b + k + 32u] : 0ull;
+                    block(k < d, key, (uint32_t)x0 + row, 0xffffffffu, rb, ra);
+                }
+                if (lane == 0) products(rb, ra);
+            });
     }
 #pragma unroll
     for (int q1 = 0; q1 < 3; ++q1)
@@ -205,14 +251,14 @@ tc_status tc_census64(tc_graph* g, void* stream, tc_u128 out[64]) {
                                                             deg.as<uint32_t>());
         TC_LAUNCH("k_deg_old");
         TC_TRY(scan_u32_to_u64(deg.as<uint32_t>(), offo.as<uint64_t>(), G.n, st));
-        k_keys64<<<grid_for((uint64_t)G.n * 32, 256, 8192), 256, 0, st>>>(gd, old.as<uint32_t>(), B,
+        k_keys64<<<grid_for(std::max<uint64_t>(G.n, E2 / (kKeyChunk / 32)), 256, 1u << 16), 256, 0, st>>>(gd, G.n_wide, old.as<uint32_t>(), B,
                                                                           keys.as<uint64_t>());
         TC_LAUNCH("k_keys64");
         uint64_t* kp = keys.as<uint64_t>();
         uint64_t* tp = tmp.as<uint64_t>();
         TC_TRY(radix_sort_u64(&kp, &tp, E2, 2, 2 * B + 2, st));
         unsigned long long* d_raw = acc.as<unsigned long long>();
-        k_wedges64<<<grid_for((uint64_t)G.n * 32, 256, 8u * (unsigned)sm_count()), 256, 0, st>>>(
+        k_wedges64<<<grid_for(G.n, 256, 4u * (unsigned)sm_count()), 256, 0, st>>>(
             kp, offo.as<uint64_t>(), G.n, B, d_raw);
         TC_LAUNCH("k_wedges64");
         // triangles, in caller-id states, through the triangle form's plan
