@@ -94,45 +94,66 @@ __global__ void k_relabel_keys(const uint32_t* deg, uint32_t n, int B, uint64_t*
         rk[x] = ((top - deg[x]) << B) | x;
 }
 
-__global__ void k_perm(const uint64_t* rk, uint32_t n, int B, const uint32_t* deg, uint32_t* new_of_old,
-                       uint32_t* new_deg) {
+__global__ void k_perm(const uint64_t* rk, uint32_t n, int B, uint32_t* new_of_old) {
     const uint64_t mask = (1ull << B) - 1;
-    for (uint64_t r = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; r < n; r += (uint64_t)gridDim.x * blockDim.x) {
-        uint32_t x = (uint32_t)(rk[r] & mask);
-        new_of_old[x] = (uint32_t)r;
-        new_deg[r] = deg[x];
-    }
+    for (uint64_t r = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; r < n; r += (uint64_t)gridDim.x * blockDim.x)
+        new_of_old[rk[r] & mask] = (uint32_t)r;
 }
 
-// Both directions of each pair in the new ids: (owner << (B+2)) | (nbr << 2) | dir(owner).
-__global__ void k_entries(const uint64_t* ukey, const uint32_t* udir, uint64_t E, int B, const uint32_t* new_of_old,
-                          uint64_t* ek) {
+// Each pair once in the new ids, from its smaller one: (lo << (B+2)) | (hi << 2) | dir(lo).
+__global__ void k_upper_keys(const uint64_t* ukey, const uint32_t* udir, uint64_t E, int B, const uint32_t* new_of_old,
+                             uint64_t* key) {
     const uint64_t mask = (1ull << B) - 1;
     for (uint64_t r = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; r < E; r += (uint64_t)gridDim.x * blockDim.x) {
-        uint64_t k = ukey[r];
-        uint64_t a = new_of_old[k >> B], b = new_of_old[k & mask];
-        uint32_t d = udir[r];
-        ek[2 * r] = (a << (B + 2)) | (b << 2) | d;
-        ek[2 * r + 1] = (b << (B + 2)) | (a << 2) | swap_dir(d);
+        const uint64_t k = ukey[r];
+        const uint64_t a = new_of_old[k >> B], b = new_of_old[k & mask];
+        const uint32_t d = udir[r];
+        key[r] = a < b ? (a << (B + 2)) | (b << 2) | d : (b << (B + 2)) | (a << 2) | swap_dir(d);
     }
 }
 
-__global__ void k_adj_from_entries(const uint64_t* ek, uint64_t cnt, int B, uint32_t* adj) {
-    const uint64_t mask = (1ull << (B + 2)) - 1;
-    for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < cnt; i += (uint64_t)gridDim.x * blockDim.x)
-        adj[i] = (uint32_t)(ek[i] & mask);
+// With the pairs sorted by (lo, hi), pair p's key in the transpose: (hi << 32) | p.  Sorted by hi,
+// stably, vertex v's pairs stand in the order of their lo: its lower list.
+__global__ void k_transpose_keys(const uint64_t* __restrict__ key, uint64_t E, int B, uint64_t* __restrict__ tkey) {
+    const uint64_t mask = (1ull << B) - 1;
+    for (uint64_t p = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; p < E; p += (uint64_t)gridDim.x * blockDim.x)
+        tkey[p] = ((key[p] >> 2) & mask) << 32 | p;
 }
 
-// up[x] = number of neighbours with id < x (lists ascend, so a lower_bound).
-__global__ void k_up(const uint64_t* off, const uint32_t* adj, uint32_t n, uint32_t* up) {
-    for (uint64_t x = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; x < n; x += (uint64_t)gridDim.x * blockDim.x) {
-        uint64_t lo = off[x], hi = off[x + 1], b = lo;
-        uint32_t key = (uint32_t)x << 2;
-        while (lo < hi) {
-            uint64_t mid = (lo + hi) >> 1;
-            if (adj[mid] < key) lo = mid + 1; else hi = mid;
-        }
-        up[x] = (uint32_t)(lo - b);
+// start[x] = the first of the E > 0 sorted keys whose row (key >> shift) is >= x, for x in [0, n].
+__global__ void k_row_starts(const uint64_t* __restrict__ key, uint64_t E, int shift, uint32_t n, uint64_t* __restrict__ start) {
+    const uint64_t t0 = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x, stride = (uint64_t)gridDim.x * blockDim.x;
+    for (uint64_t p = t0; p < E; p += stride) {
+        const uint64_t row = key[p] >> shift;
+        for (uint64_t x = p ? (key[p - 1] >> shift) + 1 : 0; x <= row; ++x) start[x] = p;
+    }
+    for (uint64_t x = (key[E - 1] >> shift) + 1 + t0; x <= n; x += stride) start[x] = E;
+}
+
+// off and up from the starts of the upper pairs (ub) and of the lower entries (lb) of each vertex.
+__global__ void k_offsets(const uint64_t* __restrict__ ub, const uint64_t* __restrict__ lb, uint32_t n, uint64_t* __restrict__ off,
+                          uint32_t* __restrict__ up) {
+    for (uint64_t x = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; x <= n; x += (uint64_t)gridDim.x * blockDim.x) {
+        const uint64_t l = lb[x];
+        off[x] = ub[x] + l;
+        if (x < n) up[x] = (uint32_t)(lb[x + 1] - l);
+    }
+}
+
+// The lists: the i-th sorted pair is u's upper entry (behind the lower entries of the vertices up to
+// u), the i-th transposed one v's lower entry (behind the upper entries of the vertices below v),
+// whose position in v's list is its pair's rp.
+__global__ void k_lists(const uint64_t* __restrict__ key, const uint64_t* __restrict__ tkey, uint64_t E, int B,
+                        const uint64_t* __restrict__ ub, const uint64_t* __restrict__ lb, uint32_t* __restrict__ adj,
+                        uint32_t* __restrict__ rp) {
+    const uint64_t mask = (1ull << (B + 2)) - 1;
+    for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < E; i += (uint64_t)gridDim.x * blockDim.x) {
+        const uint64_t k = key[i], t = tkey[i], v = t >> 32;
+        adj[i + lb[(k >> (B + 2)) + 1]] = (uint32_t)(k & mask);
+        const uint32_t p = (uint32_t)t;
+        const uint64_t kt = key[p];
+        adj[i + ub[v]] = (uint32_t)(kt >> (B + 2)) << 2 | swap_dir((uint32_t)kt & 3u);
+        rp[p] = (uint32_t)(i - lb[v]);
     }
 }
 
@@ -180,9 +201,9 @@ constexpr int kLongThreads = 1024;
 
 // Per upper pair tables, lists of at most kLongList entries (longer ones are k_pair_tables_long's).
 // The lane at position k of N[v] counts the direction classes of the entries after k.  At a lower
-// neighbour u = N[v][k] (k < up[v]) those are the third vertices w > u reached from v: the lane
-// writes them to sfx[lb[v] + k] (lb[v] = the lower entries of the vertices before v), where
-// k_pair_rp picks them up for the upper pair (u, v).  At an upper neighbour (k >= up[v]) they are
+// neighbour u = N[v][k] (k < up[v]) those are the third vertices w > u reached from v: vs of the
+// upper pair (u, v), whose index is the low half of tkey[lb[v] + k] (k_transpose_keys; lb[v] = the
+// lower entries of the vertices before v).  At an upper neighbour (k >= up[v]) they are
 // the third vertices w > N[v][k] reached from v, the u side of the pair (v, N[v][k]): us = (class-1,
 // class-2 counts).  wk[0] += the suffix lengths at lower neighbours (the N[v] entries a census
 // walks), wk[1] += those of them with ids below kMapIdsSuffix: with c the entries of N[v] below it
@@ -195,7 +216,8 @@ constexpr int kLongThreads = 1024;
 __global__ void __launch_bounds__(kB) k_pair_tables(const uint64_t* __restrict__ off, const uint32_t* __restrict__ adj,
                               const uint32_t* __restrict__ up, const uint64_t* __restrict__ ub,
                               const uint64_t* __restrict__ lb, uint32_t n,
-                              const unsigned long long* __restrict__ n_wide, uint2* sfx, uint2* us,
+                              const unsigned long long* __restrict__ n_wide, const uint64_t* __restrict__ tkey, uint2* vs,
+                              uint2* us,
                               unsigned long long* wk) {
     __shared__ uint8_t s_at[kB / 32][32];
     const uint32_t lane = threadIdx.x & 31;
@@ -215,7 +237,7 @@ __global__ void __launch_bounds__(kB) k_pair_tables(const uint64_t* __restrict__
             const uint32_t b1 = __ballot_sync(0xffffffffu, (e & 3u) == 1u);
             const uint32_t b2 = __ballot_sync(0xffffffffu, (e & 3u) == 2u);
             if (k < lv) {
-                sfx[lbv + k] = make_uint2(c1 + __popc(b1 & after), c2 + __popc(b2 & after));
+                vs[(uint32_t)tkey[lbv + k]] = make_uint2(c1 + __popc(b1 & after), c2 + __popc(b2 & after));
                 walk += dv - k - 1;
             } else if (k < dv) {
                 us[ubv + (k - lv)] = make_uint2(c1 + __popc(b1 & after), c2 + __popc(b2 & after));
@@ -245,7 +267,7 @@ __global__ void __launch_bounds__(kB) k_pair_tables(const uint64_t* __restrict__
                 const uint32_t mm = __ballot_sync(0xffffffffu, p.valid && (e >> 2) < kMapIdsSuffix) & p.lanes;
                 const uint2 c = make_uint2(__popc(m1 & after), __popc(m2 & after));
                 if (p.valid && k < lv) {
-                    sfx[lbv + k] = c;
+                    vs[(uint32_t)tkey[lbv + k]] = c;
                     walk += dv - k - 1;
                     const uint32_t cmap = __popc(mm);
                     walk_map += cmap > k ? cmap - k - 1u : 0u;
@@ -268,8 +290,8 @@ __global__ void __launch_bounds__(kB) k_pair_tables(const uint64_t* __restrict__
 // it, as k_pair_tables walks a whole list.
 __global__ void __launch_bounds__(kLongThreads) k_pair_tables_long(
         const uint64_t* __restrict__ off, const uint32_t* __restrict__ adj, const uint32_t* __restrict__ up,
-        const uint64_t* __restrict__ ub, const uint64_t* __restrict__ lb, uint32_t n, uint2* sfx, uint2* us,
-        unsigned long long* wk) {
+        const uint64_t* __restrict__ ub, const uint64_t* __restrict__ lb, uint32_t n, const uint64_t* __restrict__ tkey,
+        uint2* vs, uint2* us, unsigned long long* wk) {
     __shared__ uint32_t s_c1[kLongThreads / 32], s_c2[kLongThreads / 32], s_map[kLongThreads / 32];
     const uint64_t v = blockIdx.x;
     if (v >= n) return;
@@ -313,7 +335,7 @@ __global__ void __launch_bounds__(kLongThreads) k_pair_tables_long(
             const uint32_t b1 = __ballot_sync(0xffffffffu, (e & 3u) == 1u);
             const uint32_t b2 = __ballot_sync(0xffffffffu, (e & 3u) == 2u);
             if (k < lv) {
-                sfx[lb[v] + k] = make_uint2(c1 + __popc(b1 & after), c2 + __popc(b2 & after));
+                vs[(uint32_t)tkey[lb[v] + k]] = make_uint2(c1 + __popc(b1 & after), c2 + __popc(b2 & after));
                 walk += dv - k - 1;
             } else if (k < s1) {
                 us[ub[v] + (k - lv)] = make_uint2(c1 + __popc(b1 & after), c2 + __popc(b2 & after));
@@ -330,89 +352,6 @@ __global__ void __launch_bounds__(kLongThreads) k_pair_tables_long(
         const unsigned long long wm = m * cmap - m * (m + 1) / 2;
         if (wm) atomicAdd(wk + 1, wm);
     }
-}
-
-// Position of u in the lower part L = N[v][0, len) of a list (u is there: u < v and u ~ v).
-// The degree order puts u, of degree at least v's, near the front of L, so the search gallops
-// from the front (probes 1, 3, 7, ...) and then bisects the last gap: a hub's position costs a
-// probe or two in the first sector of L.
-__device__ __forceinline__ uint32_t lower_position(const uint32_t* __restrict__ L, uint32_t len, uint32_t u) {
-    uint32_t lo = 0, hi = 1;
-    while (hi < len && (L[hi] >> 2) < u) {
-        lo = hi + 1;
-        hi = 2 * hi + 1;
-    }
-    hi = min(hi, len);
-    while (lo < hi) {
-        const uint32_t mid = (lo + hi) >> 1;
-        if ((L[mid] >> 2) < u) lo = mid + 1;
-        else hi = mid;
-    }
-    return lo;
-}
-
-// rp and vs of one upper pair (u, v = N[u][j]), table index p: rp = the position k of u in N[v],
-// vs = sfx[lb[v] + k] (the class counts of N[v] past u, from k_pair_tables).
-__device__ __forceinline__ void pair_rp(const uint64_t* __restrict__ off, const uint32_t* __restrict__ adj,
-                                        const uint32_t* __restrict__ up, const uint64_t* __restrict__ lb,
-                                        const uint2* __restrict__ sfx, uint32_t u, uint32_t v, uint64_t p, uint32_t* rp,
-                                        uint2* vs) {
-    const uint32_t k = lower_position(adj + off[v], up[v], u);
-    rp[p] = k;
-    vs[p] = sfx[lb[v] + k];
-}
-
-// The tables of the upper pairs, each upper list in order, so the table writes are coalesced: a
-// warp per vertex of more than 32 neighbours (n_wide, a prefix of the ids; above kLongList they are
-// k_pair_rp_long's), a warp per 32 vertices for the others, whose upper lists share its lanes
-// (rows.cuh).
-__global__ void __launch_bounds__(kB) k_pair_rp(const uint64_t* __restrict__ off, const uint32_t* __restrict__ adj,
-                          const uint32_t* __restrict__ up, const uint64_t* __restrict__ ub,
-                          const uint64_t* __restrict__ lb, const uint2* __restrict__ sfx, uint32_t n,
-                          const unsigned long long* __restrict__ n_wide, uint32_t* rp, uint2* vs) {
-    __shared__ uint8_t s_at[kB / 32][32];
-    const uint32_t lane = threadIdx.x & 31;
-    const uint64_t stride = (uint64_t)gridDim.x * blockDim.x, wide = *n_wide;
-    for (uint64_t u = (blockIdx.x * (uint64_t)blockDim.x + threadIdx.x) >> 5; u < wide; u += stride >> 5) {
-        const uint64_t ob = off[u], tb = ub[u];
-        const uint32_t du = (uint32_t)(off[u + 1] - ob), upu = up[u];
-        if (du > kLongList) continue;                                 // k_pair_rp_long's
-        for (uint32_t j = upu + lane; j < du; j += 32)
-            pair_rp(off, adj, up, lb, sfx, (uint32_t)u, adj[ob + j] >> 2, tb + (j - upu), rp, vs);
-    }
-    for (uint64_t x0 = wide + blockIdx.x * (uint64_t)blockDim.x + (threadIdx.x & ~31u); x0 < n; x0 += stride) {
-        const uint64_t x = x0 + lane;
-        const bool ok = x < n;
-        const uint64_t vob = ok ? off[x] : 0ull, vub = ok ? ub[x] : 0ull;
-        const uint32_t vd = ok ? (uint32_t)(off[x + 1] - vob) : 0u, vl = ok ? up[x] : 0u;
-        for_rows(vd - vl, s_at[threadIdx.x >> 5],
-            [&](const PackedEntry& p) {
-                const uint64_t first = __shfl_sync(0xffffffffu, vob + vl, p.row), ubu = __shfl_sync(0xffffffffu, vub, p.row);
-                const uint32_t k = lane - p.first;
-                if (p.valid) pair_rp(off, adj, up, lb, sfx, (uint32_t)x0 + p.row, adj[first + k] >> 2, ubu + k, rp, vs);
-            },
-            [](uint32_t) {});
-    }
-}
-
-// One CTA per vertex of the prefix of the ids that holds the long lists.
-__global__ void k_pair_rp_long(const uint64_t* __restrict__ off, const uint32_t* __restrict__ adj,
-                               const uint32_t* __restrict__ up, const uint64_t* __restrict__ ub,
-                               const uint64_t* __restrict__ lb, const uint2* __restrict__ sfx, uint32_t n, uint32_t* rp,
-                               uint2* vs) {
-    const uint64_t u = blockIdx.x;
-    if (u >= n) return;
-    const uint64_t ob = off[u];
-    const uint32_t du = (uint32_t)(off[u + 1] - ob), upu = up[u];
-    if (du <= kLongList) return;
-    for (uint32_t j = upu + threadIdx.x; j < du; j += blockDim.x)
-        pair_rp(off, adj, up, lb, sfx, (uint32_t)u, adj[ob + j] >> 2, ub[u] + (j - upu), rp, vs);
-}
-
-// upper pairs per vertex: deg - up
-__global__ void k_upper_of(const uint64_t* off, const uint32_t* up, uint32_t n, uint32_t* cnt) {
-    for (uint64_t x = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; x < n; x += (uint64_t)gridDim.x * blockDim.x)
-        cnt[x] = (uint32_t)(off[x + 1] - off[x]) - up[x];
 }
 
 // ---- CSR input validation: stats[6] = number of violations
@@ -478,89 +417,76 @@ tc_status finish_graph(GraphStore& g, uint64_t E, int B, uint64_t* ukey, uint32_
     const uint32_t n = g.n;
     const unsigned gridE = grid_for(E, kB, 1u << 16), gridN = grid_for(n, kB, 1u << 16);
     // relabel by descending degree
-    DevBuf rk, rtmp, ndeg;
+    DevBuf rk, rtmp;
     TC_TRY(rk.alloc(sizeof(uint64_t) * n, st));
     TC_TRY(rtmp.alloc(sizeof(uint64_t) * n, st));
-    TC_TRY(ndeg.alloc(sizeof(uint32_t) * n, st));
     TC_TRY(g.new_of_old.alloc_persistent(sizeof(uint32_t) * n));
     k_relabel_keys<<<gridN, kB, 0, st>>>(deg, n, B, rk.as<uint64_t>());
     TC_LAUNCH("k_relabel_keys");
     uint64_t* kp = rk.as<uint64_t>();
     uint64_t* tp = rtmp.as<uint64_t>();
     TC_TRY(radix_sort_u64(&kp, &tp, n, B, 2 * B, st));   // stable: ties stay in id order
-    k_perm<<<gridN, kB, 0, st>>>(kp, n, B, deg, g.new_of_old.as<uint32_t>(), ndeg.as<uint32_t>());
+    k_perm<<<gridN, kB, 0, st>>>(kp, n, B, g.new_of_old.as<uint32_t>());
     TC_LAUNCH("k_perm");
     rk.release();
     rtmp.release();
-    // offsets
     TC_TRY(g.off.alloc_persistent(sizeof(uint64_t) * (n + 1ull)));
-    TC_TRY(scan_u32_to_u64(ndeg.as<uint32_t>(), g.off.as<uint64_t>(), n, st));
-    // entries in new ids, sorted by (owner, neighbour)
-    uint64_t total = 2 * E;
-    DevBuf ek, etmp;
-    TC_TRY(ek.alloc(sizeof(uint64_t) * (total ? total : 1), st));
-    TC_TRY(etmp.alloc(sizeof(uint64_t) * (total ? total : 1), st));
-    if (E) {
-        k_entries<<<gridE, kB, 0, st>>>(ukey, udir, E, B, g.new_of_old.as<uint32_t>(), ek.as<uint64_t>());
-        TC_LAUNCH("k_entries");
-    }
-    kp = ek.as<uint64_t>();
-    tp = etmp.as<uint64_t>();
-    TC_TRY(radix_sort_u64(&kp, &tp, total, 2, 2 * B + 2, st));
-    TC_TRY(g.adj.alloc_persistent(sizeof(uint32_t) * (total + 4)));   // read in aligned blocks of four
-    if (total) {
-        k_adj_from_entries<<<grid_for(total, kB, 1u << 16), kB, 0, st>>>(kp, total, B, g.adj.as<uint32_t>());
-        TC_LAUNCH("k_adj_from_entries");
-    }
-    ek.release();
-    etmp.release();
+    TC_TRY(g.ub.alloc_persistent(sizeof(uint64_t) * (n + 1ull)));
     TC_TRY(g.up.alloc_persistent(sizeof(uint32_t) * n));
-    k_up<<<gridN, kB, 0, st>>>(g.off.as<uint64_t>(), g.adj.as<uint32_t>(), n, g.up.as<uint32_t>());
-    TC_LAUNCH("k_up");
-    k_graph_sums<<<gridN, kB, 0, st>>>(g.off.as<uint64_t>(), g.adj.as<uint32_t>(), g.up.as<uint32_t>(), n,
-                                       stats.as<unsigned long long>());
+    TC_TRY(g.adj.alloc_persistent(sizeof(uint32_t) * (2 * E + 4)));   // read in aligned blocks of four
+    TC_TRY(g.rp.alloc_persistent(sizeof(uint32_t) * (E ? E : 1)));
+    TC_TRY(g.vs.alloc_persistent(sizeof(uint2) * (E ? E : 1)));
+    TC_TRY(g.us.alloc_persistent(sizeof(uint2) * (E ? E : 1)));
+    uint64_t *off = g.off.as<uint64_t>(), *ub = g.ub.as<uint64_t>();
+    unsigned long long* d_stats = stats.as<unsigned long long>();
+    // the pairs in the new ids, sorted by (lo, hi): the upper lists in order, a pair's place its table
+    // index; and their transpose, sorted by hi: the lower lists in order
+    DevBuf key, tmp, tkey, lbuf;
+    TC_TRY(lbuf.alloc(sizeof(uint64_t) * (n + 1ull), st));
+    uint64_t* lb = lbuf.as<uint64_t>();
+    const uint64_t* ks = nullptr;
+    const uint64_t* ts = nullptr;
+    if (E) {
+        TC_TRY(key.alloc(sizeof(uint64_t) * E, st));
+        TC_TRY(tmp.alloc(sizeof(uint64_t) * E, st));
+        TC_TRY(tkey.alloc(sizeof(uint64_t) * E, st));
+        k_upper_keys<<<gridE, kB, 0, st>>>(ukey, udir, E, B, g.new_of_old.as<uint32_t>(), key.as<uint64_t>());
+        TC_LAUNCH("k_upper_keys");
+        kp = key.as<uint64_t>();
+        tp = tmp.as<uint64_t>();
+        TC_TRY(radix_sort_u64(&kp, &tp, E, 2, 2 * B + 2, st));
+        ks = kp;
+        kp = tkey.as<uint64_t>();   // tp, the buffer the sort left over, is the transpose's second one
+        k_transpose_keys<<<gridE, kB, 0, st>>>(ks, E, B, kp);
+        TC_LAUNCH("k_transpose_keys");
+        TC_TRY(radix_sort_u64(&kp, &tp, E, 32, 32 + B, st));
+        ts = kp;
+        k_row_starts<<<gridE, kB, 0, st>>>(ks, E, B + 2, n, ub);
+        TC_LAUNCH("k_row_starts (upper)");
+        k_row_starts<<<gridE, kB, 0, st>>>(ts, E, 32, n, lb);
+        TC_LAUNCH("k_row_starts (lower)");
+    } else {
+        TC_CUDA(cudaMemsetAsync(ub, 0, sizeof(uint64_t) * (n + 1ull), st));
+        TC_CUDA(cudaMemsetAsync(lb, 0, sizeof(uint64_t) * (n + 1ull), st));
+    }
+    k_offsets<<<grid_for(n + 1ull, kB, 1u << 16), kB, 0, st>>>(ub, lb, n, off, g.up.as<uint32_t>());
+    TC_LAUNCH("k_offsets");
+    if (E) {
+        k_lists<<<gridE, kB, 0, st>>>(ks, ts, E, B, ub, lb, g.adj.as<uint32_t>(), g.rp.as<uint32_t>());
+        TC_LAUNCH("k_lists");
+    }
+    k_graph_sums<<<gridN, kB, 0, st>>>(off, g.adj.as<uint32_t>(), g.up.as<uint32_t>(), n, d_stats);
     TC_LAUNCH("k_graph_sums");
-    // per upper pair tables: ub = exclusive scan of the upper pairs per vertex
-    {
-        DevBuf ucnt;
-        TC_TRY(ucnt.alloc(sizeof(uint32_t) * (n ? n : 1), st));
-        TC_TRY(g.ub.alloc_persistent(sizeof(uint64_t) * (n + 1ull)));
-        TC_TRY(g.rp.alloc_persistent(sizeof(uint32_t) * (E ? E : 1)));
-        TC_TRY(g.vs.alloc_persistent(sizeof(uint2) * (E ? E : 1)));
-        TC_TRY(g.us.alloc_persistent(sizeof(uint2) * (E ? E : 1)));
-        if (n) {
-            k_upper_of<<<gridN, kB, 0, st>>>(g.off.as<uint64_t>(), g.up.as<uint32_t>(), n, ucnt.as<uint32_t>());
-            TC_LAUNCH("k_upper_of");
-        }
-        TC_TRY(scan_u32_to_u64(ucnt.as<uint32_t>(), g.ub.as<uint64_t>(), n, st));
-        if (E) {
-            // lower entries before each vertex (lb[n] = E), and their suffix counts
-            DevBuf lb, sfx;
-            TC_TRY(lb.alloc(sizeof(uint64_t) * (n + 1ull), st));
-            TC_TRY(sfx.alloc(sizeof(uint2) * E, st));
-            TC_TRY(scan_u32_to_u64(g.up.as<uint32_t>(), lb.as<uint64_t>(), n, st));
-            // the walk lengths go to stats[8..9]
-            k_pair_tables<<<grid_for(n, kB, 1u << 16), kB, 0, st>>>(
-                g.off.as<uint64_t>(), g.adj.as<uint32_t>(), g.up.as<uint32_t>(), g.ub.as<uint64_t>(),
-                lb.as<uint64_t>(), n, stats.as<unsigned long long>() + 12, sfx.as<uint2>(), g.us.as<uint2>(),
-                stats.as<unsigned long long>() + 8);
-            TC_LAUNCH("k_pair_tables");
-            // lists longer than kLongList: at most 2E / kLongList of them, the first ids
-            const uint64_t n_long = std::min<uint64_t>(n, 2ull * E / kLongList + 1);
-            k_pair_tables_long<<<(unsigned)n_long, kLongThreads, 0, st>>>(
-                g.off.as<uint64_t>(), g.adj.as<uint32_t>(), g.up.as<uint32_t>(), g.ub.as<uint64_t>(),
-                lb.as<uint64_t>(), n, sfx.as<uint2>(), g.us.as<uint2>(), stats.as<unsigned long long>() + 8);
-            TC_LAUNCH("k_pair_tables_long");
-            k_pair_rp<<<grid_for(n, kB, 1u << 16), kB, 0, st>>>(
-                g.off.as<uint64_t>(), g.adj.as<uint32_t>(), g.up.as<uint32_t>(), g.ub.as<uint64_t>(),
-                lb.as<uint64_t>(), sfx.as<uint2>(), n, stats.as<unsigned long long>() + 12, g.rp.as<uint32_t>(),
-                g.vs.as<uint2>());
-            TC_LAUNCH("k_pair_rp");
-            k_pair_rp_long<<<(unsigned)n_long, kLongThreads, 0, st>>>(
-                g.off.as<uint64_t>(), g.adj.as<uint32_t>(), g.up.as<uint32_t>(), g.ub.as<uint64_t>(),
-                lb.as<uint64_t>(), sfx.as<uint2>(), n, g.rp.as<uint32_t>(), g.vs.as<uint2>());
-            TC_LAUNCH("k_pair_rp_long");
-        }
+    if (E) {
+        // the suffix counts of the per upper pair tables; the walk lengths go to stats[8..9]
+        k_pair_tables<<<gridN, kB, 0, st>>>(off, g.adj.as<uint32_t>(), g.up.as<uint32_t>(), ub, lb, n, d_stats + 12, ts,
+                                            g.vs.as<uint2>(), g.us.as<uint2>(), d_stats + 8);
+        TC_LAUNCH("k_pair_tables");
+        // lists longer than kLongList: at most 2E / kLongList of them, the first ids
+        const uint64_t n_long = std::min<uint64_t>(n, 2ull * E / kLongList + 1);
+        k_pair_tables_long<<<(unsigned)n_long, kLongThreads, 0, st>>>(off, g.adj.as<uint32_t>(), g.up.as<uint32_t>(), ub, lb, n,
+                                                                      ts, g.vs.as<uint2>(), g.us.as<uint2>(), d_stats + 8);
+        TC_LAUNCH("k_pair_tables_long");
     }
     unsigned long long hs[13];
     TC_CUDA(cudaMemcpyAsync(hs, stats.p, sizeof(hs), cudaMemcpyDeviceToHost, st));
