@@ -392,7 +392,28 @@ __global__ void __launch_bounds__(256, 4) k_pair_bulk(BulkParams P) {
             bulk_pair(G, n, sD, j, G.adj[sB + j], pstart + i, acc);
         }
     }
-    if (MODE == kTriSingle || cur_graph != 0xffffffffu) flush_bulk(acc, raw, lane);
+    if (MODE == kTriSingle) {
+        // one graph: the warps' sums meet in shared memory, so a CTA adds 21 counters once (a small
+        // census waited for its warps' atomics on them)
+        __shared__ unsigned long long s_sum[kWarps][21];
+#pragma unroll
+        for (int c = 0; c < 3; ++c)
+#pragma unroll
+            for (int k = 0; k < 7; ++k) {
+                unsigned long long s = acc[c][k];
+                for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+                if (lane == 0) s_sum[threadIdx.x >> 5][7 * c + k] = s;
+            }
+        __syncthreads();
+        if (threadIdx.x < 21) {
+            unsigned long long s = 0;
+#pragma unroll
+            for (int w = 0; w < kWarps; ++w) s += s_sum[w][threadIdx.x];
+            if (s) atomicAdd(&raw[threadIdx.x], s);
+        }
+    } else if (cur_graph != 0xffffffffu) {
+        flush_bulk(acc, raw, lane);
+    }
 }
 
 struct Table64 {
