@@ -135,11 +135,13 @@ tc_status tc_graph_create_csr(uint32_t n, const uint64_t* off, const uint32_t* a
                               int ptr_is_device, void* stream, const tc_options* opt, tc_graph** out);
 
 /* Full census (Fig. 5): 16 counts, the null count (index 0) computed as C(n,3) minus the
- * rest in 128-bit (steps 3-5).  Enqueues the kernels on `stream` and synchronises it. */
+ * rest in 128-bit (steps 3-5).  Enqueues the kernels on `stream` and synchronises it.  A graph
+ * made without options (opt NULL) is counted in the fastest form (TC_ALGO_TRIANGLE). */
 tc_status tc_census(tc_graph* g, void* stream, tc_u128 out[16]);
 
 /* Same census with options overriding the graph's creation options (algo, schedule,
- * tiers) for this call only.  opt may be NULL. */
+ * tiers) for this call only.  opt may be NULL; if the graph was made with NULL too, the form is
+ * the library's to choose (TC_ALGO_TRIANGLE), else an algo of 0 is TC_ALGO_UNION. */
 tc_status tc_census_opts(tc_graph* g, void* stream, const tc_options* opt, tc_u128 out[16]);
 
 /* Asynchronous census: enqueues the kernels on `stream` and writes, when they finish,

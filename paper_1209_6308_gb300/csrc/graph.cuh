@@ -68,11 +68,12 @@ struct GraphStore {
     DevBuf off, adj, up, new_of_old;
     DevBuf ub, rp, vs, us;   // per upper pair tables (see GraphDev)
     DevBuf rec, blk16;   // 16-bit lower lists (see GraphDev): rec holds rec, rec2 and n16 of the active vertices
-    DevBuf ctr;        // census work counters (uint32 x 8)
+    DevBuf ctr;        // census work counters (uint32 x 4)
     DevBuf acc;        // census accumulators (uint64 x 16)
     DevBuf cost;       // optional per-vertex predicted cost (float x n) for the learned schedule
-    DevBuf tri;        // triangle form: bulk sums and triangle tricode histogram (uint64 x 96)
+    DevBuf tri;        // triangle form: bulk sums and triangle tricode histogram (uint64 x 96), counters (uint32 x 8)
     Opts opts;
+    bool no_opts = false;   // made without a tc_options
     static constexpr int kPlans = 4;
     Plan plans[kPlans];
     int next_plan = 0;
@@ -132,8 +133,7 @@ int bits_for(uint32_t n);
 tc_status graph_create_sorted(uint32_t n, const uint64_t* d_keys, uint64_t m, cudaStream_t st, const tc_options* opt,
                               tc_graph** out);
 
-// Enqueue one census on `st`; counts of classes 1..15 are added to d_out16 (which the
-// caller zeroes; index 0 is never touched).  No host synchronisation, no allocation once
+// Enqueue one census on `st`; counts of classes 1..15 go to d_out16, index 0 is 0.  No host synchronisation, no allocation once
 // the plan for `o` exists (get_plan allocates it on first use).
 tc_status get_plan(GraphStore& g, const Opts& o, cudaStream_t st, Plan** out);
 // The single-graph census's form (map or not) and, for an automatic chunk, its size: call

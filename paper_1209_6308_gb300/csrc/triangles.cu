@@ -420,9 +420,8 @@ struct Table64 {
     uint8_t t[64];
 };
 
-// 16 classes from the bulk sums and the triangle tricodes (see the file comment); adds
-// classes 1..15 into out16 (index 0 untouched).  One block of 64 threads.
-// Batched: block g folds raw + kBatchStride g and hist + kBatchStride g into out16 + 16 g.
+// 16 classes from the bulk sums and the triangle tricodes (see the file comment) into out16 (index
+// 0 gets 0).  One block of 64 threads.  Batched: block g folds raw + kBatchStride g and hist + kBatchStride g into out16 + 16 g.
 __global__ void k_tri_fold(const unsigned long long* __restrict__ raw, const unsigned long long* __restrict__ hist,
                            Table64 T, unsigned long long* out16) {
     __shared__ unsigned long long s[16];
@@ -458,7 +457,7 @@ __global__ void k_tri_fold(const unsigned long long* __restrict__ raw, const uns
         atomicAdd(&s[dbc == 3u ? 2u : 1u], h);
     }
     __syncthreads();
-    if (t >= 1 && t < 16 && s[t]) atomicAdd(&out16[t], s[t]);
+    if (t < 16) out16[t] = t ? s[t] : 0ull;
 }
 
 // Serving: fold each finished request's scratch (block r) into its 16 counts in mapped host
@@ -572,13 +571,18 @@ tc_status triangles_launch(const GraphDev& gd, const Opts& o, const Item* items,
 tc_status triangle_census_enqueue(GraphStore& g, const Opts& o, const Plan& p, uint32_t item0, uint32_t n_items,
                                   uint32_t warp_begin, uint32_t warp_end, cudaStream_t st, unsigned long long* d_out16,
                                   unsigned long long* d_vcost, unsigned long long* d_phase) {
-    if (g.e_sym == 0) return TC_OK;
+    if (g.e_sym == 0) {
+        TC_CUDA(cudaMemsetAsync(d_out16, 0, sizeof(unsigned long long) * 16, st));
+        return TC_OK;
+    }
     if (!g.vs.p) return fail(TC_ERR_ARG, "the triangle form needs the per upper pair tables");
-    if (!g.tri.p) TC_TRY(g.tri.alloc_persistent(sizeof(unsigned long long) * kBatchStride));
-    unsigned long long* raw = g.tri.as<unsigned long long>();   // [0, 21) bulk sums, [32, 96) triangle tricodes
+    // [0, 21) bulk sums, [32, 96) triangle tricodes, then 8 work counters: zeroed at once
+    constexpr size_t kScratch = sizeof(unsigned long long) * kBatchStride + sizeof(uint32_t) * 8;
+    if (!g.tri.p) TC_TRY(g.tri.alloc_persistent(kScratch));
+    unsigned long long* raw = g.tri.as<unsigned long long>();
     unsigned long long* hist = raw + 32;
-    TC_CUDA(cudaMemsetAsync(raw, 0, sizeof(unsigned long long) * kBatchStride, st));
-    TC_CUDA(cudaMemsetAsync(g.ctr.p, 0, sizeof(uint32_t) * 8, st));
+    uint32_t* ctr = reinterpret_cast<uint32_t*>(raw + kBatchStride);
+    TC_CUDA(cudaMemsetAsync(raw, 0, kScratch, st));
     const Item* items = p.items.as<Item>() + item0;
     // the range's part of each of the plan's splits
     const uint32_t split[2] = {std::min(std::max(p.split[0], item0) - item0, n_items),
@@ -595,12 +599,12 @@ tc_status triangle_census_enqueue(GraphStore& g, const Opts& o, const Plan& p, u
         B.n_items = n_items;
         B.wb = warp_begin;
         B.we = warp_end;
-        B.ctr = g.ctr.as<uint32_t>();
+        B.ctr = ctr;
         B.raw = raw;
         k_pair_bulk<kTriSingle><<<grid_for(units * 32, 256, 4u * (unsigned)sm_count()), 256, 0, st>>>(B);
         TC_LAUNCH("k_pair_bulk");
     }
-    TC_TRY(triangles_launch(gd, o, items, n_items, warp_begin, warp_end, g.ctr.as<uint32_t>(), nullptr, nullptr, hist,
+    TC_TRY(triangles_launch(gd, o, items, n_items, warp_begin, warp_end, ctr, nullptr, nullptr, hist,
                             d_vcost, st, d_phase, walk16 ? split : nullptr));
     Table64 T;
     TC_TRY(fold_table(&T));
