@@ -4,6 +4,7 @@
 #include <cstring>
 #include <mutex>
 #include <string>
+#include <vector>
 
 #include "graph.cuh"
 
@@ -116,13 +117,14 @@ tc_status DevBuf::alloc_persistent(size_t b) {
 }
 
 void DevBuf::release() {
-    if (p) {
+    if (p && owned) {
         // a persistent buffer may be in use on any stream: like cudaFree, wait for the device
         if (!async) cudaDeviceSynchronize();
         cudaFreeAsync(p, st);
     }
     p = nullptr;
     bytes = 0;
+    owned = true;
 }
 
 int sm_count() {
@@ -175,6 +177,50 @@ tc_status resolve_opts(const tc_options* in, const Opts* base, Opts* out) {
 
 namespace {
 
+// Page-locked staging for a graph's 16 counts: making and freeing page-locked memory takes longer
+// than a small build, so graphs share pages of it.  A page is freed when its last graph goes,
+// except for one that is kept for the next.
+struct StagingPage {
+    unsigned char* p;
+    uint32_t used;   // bit per slot
+};
+constexpr size_t kStagingSlot = sizeof(unsigned long long) * 16, kStagingPage = 32 * kStagingSlot;
+std::mutex g_staging_mu;
+std::vector<StagingPage> g_staging;
+
+tc_status staging_take(unsigned long long** out) {
+    std::lock_guard<std::mutex> lk(g_staging_mu);
+    for (auto& pg : g_staging)
+        for (uint32_t i = 0; i < 32 && pg.used != 0xffffffffu; ++i)
+            if (!((pg.used >> i) & 1u)) {
+                pg.used |= 1u << i;
+                *out = reinterpret_cast<unsigned long long*>(pg.p + i * kStagingSlot);
+                return TC_OK;
+            }
+    StagingPage pg = {nullptr, 1u};
+    TC_CUDA(cudaHostAlloc((void**)&pg.p, kStagingPage, cudaHostAllocPortable));
+    g_staging.push_back(pg);
+    *out = reinterpret_cast<unsigned long long*>(pg.p);
+    return TC_OK;
+}
+
+void staging_give(unsigned long long* slot) {
+    std::lock_guard<std::mutex> lk(g_staging_mu);
+    unsigned char* at = reinterpret_cast<unsigned char*>(slot);
+    size_t empty = 0, mine = g_staging.size();
+    for (size_t k = 0; k < g_staging.size(); ++k) {
+        if (at >= g_staging[k].p && at < g_staging[k].p + kStagingPage) {
+            g_staging[k].used &= ~(1u << ((at - g_staging[k].p) / kStagingSlot));
+            mine = k;
+        }
+        empty += g_staging[k].used == 0u;
+    }
+    if (mine < g_staging.size() && g_staging[mine].used == 0u && empty > 1) {
+        cudaFreeHost(g_staging[mine].p);
+        g_staging.erase(g_staging.begin() + (std::ptrdiff_t)mine);
+    }
+}
+
 // The options of a whole census.  Where neither the graph nor the call was given any, the kernel
 // form is the library's to choose: the counts are the same in every form.  Chung-Lu n = 300007,
 // union / suffix / triangle: 7554 / 1319 / 266 us; R-MAT 14 138 / 99 / 82; below that all are
@@ -193,16 +239,17 @@ tc_status init_graph(tc_graph* g, uint32_t n, const tc_options* opt) {
     TC_TRY(resolve_opts(opt, nullptr, &check));
     g->s.opts = merge_opts(opt, nullptr);
     g->s.no_opts = opt == nullptr;
-    TC_TRY(g->s.ctr.alloc_persistent(sizeof(uint32_t) * 4));
-    TC_TRY(g->s.acc.alloc_persistent(sizeof(unsigned long long) * 16));
-    TC_CUDA(cudaMallocHost(&g->s.h_counts, sizeof(unsigned long long) * 16));
-    return TC_OK;
+    TC_TRY(g->s.scratch.alloc_persistent(1280));
+    g->s.ctr.carve(g->s.scratch, 0, sizeof(uint32_t) * 4);
+    g->s.acc.carve(g->s.scratch, 128, sizeof(unsigned long long) * 16);
+    g->s.tri.carve(g->s.scratch, 256, sizeof(unsigned long long) * 96 + sizeof(uint32_t) * 8);
+    return staging_take(&g->s.h_counts);
 }
 
 void destroy(tc_graph* g) {
     if (!g) return;
     cudaDeviceSynchronize();
-    if (g->s.h_counts) cudaFreeHost(g->s.h_counts);
+    if (g->s.h_counts) staging_give(g->s.h_counts);
     delete g;
 }
 

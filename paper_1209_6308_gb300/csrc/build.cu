@@ -19,6 +19,7 @@ namespace tc {
 namespace {
 
 constexpr int kB = 256;
+constexpr int kStats = 15;   // of the build: what each kernel adds where is said at the kernel
 
 __device__ __forceinline__ uint32_t swap_dir(uint32_t d) { return ((d & 1u) << 1) | ((d >> 1) & 1u); }
 
@@ -50,13 +51,14 @@ __global__ void k_make_keys(const uint32_t* src, const uint32_t* dst, uint64_t m
 
 __global__ void k_head_flags(const uint64_t* keys, uint64_t cnt, uint32_t* flag) {
     for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < cnt; i += (uint64_t)gridDim.x * blockDim.x)
-        flag[i] = (i == 0 || (keys[i] >> 2) != (keys[i - 1] >> 2)) ? 1u : 0u;
+        flag[i] = keys[i] != ~0ull && (i == 0 || (keys[i] >> 2) != (keys[i - 1] >> 2)) ? 1u : 0u;
 }
 
 // Runs of equal pairs -> one pair key (lo<<B | hi) and the OR of their direction bits.
 __global__ void k_unique(const uint64_t* keys, uint64_t cnt, const uint32_t* flag, const uint32_t* pos,
                          uint64_t* ukey, uint32_t* udir) {
     for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < cnt; i += (uint64_t)gridDim.x * blockDim.x) {
+        if (keys[i] == ~0ull) continue;   // a dropped arc's key, past the others
         uint32_t r = pos[i] + flag[i] - 1u;
         if (flag[i]) ukey[r] = keys[i] >> 2;
         atomicOr(&udir[r], (uint32_t)(keys[i] & 3u));
@@ -160,11 +162,11 @@ __global__ void k_lists(const uint64_t* __restrict__ key, const uint64_t* __rest
 // stats[3] sum deg^2, stats[4] sum over upper pairs of deg(v), stats[5] max degree,
 // stats[7] vertices with deg > 0, stats[10] sum of up (up - 1) / 2 (the entries the triangle form
 // walks: for every upper pair (b, c), the neighbours of c below b), stats[11] vertices with deg > kHubDeg,
-// stats[12] vertices with deg > 32
+// stats[12] vertices with deg > 32, stats[13] with deg > 64
 __global__ void k_graph_sums(const uint64_t* off, const uint32_t* adj, const uint32_t* up, uint32_t n,
                              unsigned long long* stats) {
     unsigned long long d2 = 0, dv = 0, tw = 0;
-    uint32_t mx = 0, act = 0, hub = 0, wide = 0;
+    uint32_t mx = 0, act = 0, hub = 0, wide = 0, gt64 = 0;
     for (uint64_t x = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; x < n; x += (uint64_t)gridDim.x * blockDim.x) {
         uint64_t d = off[x + 1] - off[x];
         d2 += d * d;
@@ -172,6 +174,7 @@ __global__ void k_graph_sums(const uint64_t* off, const uint32_t* adj, const uin
         act += (d > 0);
         hub += (d > kHubDeg);
         wide += (d > 32);
+        gt64 += (d > 64);
         // x is the v of every pair (u, x) with u < x: the first up[x] neighbours
         dv += (unsigned long long)up[x] * d;
         tw += (unsigned long long)up[x] * (up[x] ? up[x] - 1ull : 0ull) / 2ull;
@@ -184,11 +187,13 @@ __global__ void k_graph_sums(const uint64_t* off, const uint32_t* adj, const uin
         act += __shfl_xor_sync(0xffffffffu, act, o);
         hub += __shfl_xor_sync(0xffffffffu, hub, o);
         wide += __shfl_xor_sync(0xffffffffu, wide, o);
+        gt64 += __shfl_xor_sync(0xffffffffu, gt64, o);
     }
     if ((threadIdx.x & 31) == 0) {
         if (act) atomicAdd(&stats[7], (unsigned long long)act);
         if (hub) atomicAdd(&stats[11], (unsigned long long)hub);
         if (wide) atomicAdd(&stats[12], (unsigned long long)wide);
+        if (gt64) atomicAdd(&stats[13], (unsigned long long)gt64);
         atomicAdd(&stats[3], d2);
         atomicAdd(&stats[4], dv);
         atomicAdd(&stats[10], tw);
@@ -420,7 +425,22 @@ tc_status finish_graph(GraphStore& g, uint64_t E, int B, uint64_t* ukey, uint32_
     DevBuf rk, rtmp;
     TC_TRY(rk.alloc(sizeof(uint64_t) * n, st));
     TC_TRY(rtmp.alloc(sizeof(uint64_t) * n, st));
-    TC_TRY(g.new_of_old.alloc_persistent(sizeof(uint32_t) * n));
+    // the graph's buffers, carved from one (an allocation that outlives its stream is synchronised)
+    {
+        struct { DevBuf* b; size_t bytes; } parts[] = {
+            {&g.off, sizeof(uint64_t) * (n + 1ull)}, {&g.ub, sizeof(uint64_t) * (n + 1ull)},
+            {&g.adj, sizeof(uint32_t) * (2 * E + 4)},   // read in aligned blocks of four
+            {&g.up, sizeof(uint32_t) * n}, {&g.new_of_old, sizeof(uint32_t) * n}, {&g.rp, sizeof(uint32_t) * E},
+            {&g.vs, sizeof(uint2) * E}, {&g.us, sizeof(uint2) * E}};
+        size_t total = 0;
+        for (const auto& q : parts) total += (q.bytes + 255u) & ~(size_t)255u;
+        TC_TRY(g.store.alloc_persistent(total));
+        size_t at = 0;
+        for (const auto& q : parts) {
+            q.b->carve(g.store, at, q.bytes);
+            at += (q.bytes + 255u) & ~(size_t)255u;
+        }
+    }
     k_relabel_keys<<<gridN, kB, 0, st>>>(deg, n, B, rk.as<uint64_t>());
     TC_LAUNCH("k_relabel_keys");
     uint64_t* kp = rk.as<uint64_t>();
@@ -430,13 +450,6 @@ tc_status finish_graph(GraphStore& g, uint64_t E, int B, uint64_t* ukey, uint32_
     TC_LAUNCH("k_perm");
     rk.release();
     rtmp.release();
-    TC_TRY(g.off.alloc_persistent(sizeof(uint64_t) * (n + 1ull)));
-    TC_TRY(g.ub.alloc_persistent(sizeof(uint64_t) * (n + 1ull)));
-    TC_TRY(g.up.alloc_persistent(sizeof(uint32_t) * n));
-    TC_TRY(g.adj.alloc_persistent(sizeof(uint32_t) * (2 * E + 4)));   // read in aligned blocks of four
-    TC_TRY(g.rp.alloc_persistent(sizeof(uint32_t) * (E ? E : 1)));
-    TC_TRY(g.vs.alloc_persistent(sizeof(uint2) * (E ? E : 1)));
-    TC_TRY(g.us.alloc_persistent(sizeof(uint2) * (E ? E : 1)));
     uint64_t *off = g.off.as<uint64_t>(), *ub = g.ub.as<uint64_t>();
     unsigned long long* d_stats = stats.as<unsigned long long>();
     // the pairs in the new ids, sorted by (lo, hi): the upper lists in order, a pair's place its table
@@ -488,12 +501,13 @@ tc_status finish_graph(GraphStore& g, uint64_t E, int B, uint64_t* ukey, uint32_
                                                                       ts, g.vs.as<uint2>(), g.us.as<uint2>(), d_stats + 8);
         TC_LAUNCH("k_pair_tables_long");
     }
-    unsigned long long hs[13];
+    unsigned long long hs[kStats];
     TC_CUDA(cudaMemcpyAsync(hs, stats.p, sizeof(hs), cudaMemcpyDeviceToHost, st));
     TC_CUDA(cudaStreamSynchronize(st));
     g.sum_tri_walk = hs[10];
     g.n_hub = (uint32_t)hs[11];
     g.n_wide = (uint32_t)hs[12];
+    g.n_gt64 = (uint32_t)hs[13];
     g.sum_walk = hs[8];
     g.sum_walk_map = hs[9];
     g.e_sym = E;
@@ -518,27 +532,28 @@ int bits_for(uint32_t n) {
 
 namespace {
 
-// Runs of one pair among mv keys sorted by pair (direction bits in bits 0..1, runs adjacent)
-// -> E unique pairs (ukey = lo<<B | hi) with the OR of their direction bits.
-tc_status pairs_from_sorted(const uint64_t* kp, uint64_t mv, DevBuf& ukey, DevBuf& udir, uint32_t& E, cudaStream_t st) {
-    DevBuf flag, pos, total;
-    TC_TRY(flag.alloc(sizeof(uint32_t) * (mv ? mv : 1), st));
-    TC_TRY(pos.alloc(sizeof(uint32_t) * (mv ? mv : 1), st));
-    TC_TRY(total.alloc(sizeof(uint32_t), st));
-    E = 0;
-    if (mv) {
-        k_head_flags<<<grid_for(mv, kB, 1u << 16), kB, 0, st>>>(kp, mv, flag.as<uint32_t>());
+// Runs of one pair among m keys sorted by pair (direction bits in bits 0..1, runs adjacent, the
+// all-ones keys of dropped arcs last) -> E unique pairs (ukey = lo<<B | hi) with the OR of their
+// direction bits.  hs receives the stats so far (synchronises st).
+tc_status pairs_from_sorted(const uint64_t* kp, uint64_t m, DevBuf& ukey, DevBuf& udir, uint32_t& E, DevBuf& stats,
+                            unsigned long long hs[kStats], cudaStream_t st) {
+    DevBuf flag, pos;
+    TC_TRY(flag.alloc(sizeof(uint32_t) * (m ? m : 1), st));
+    TC_TRY(pos.alloc(sizeof(uint32_t) * (m ? m : 1), st));
+    if (m) {
+        k_head_flags<<<grid_for(m, kB, 1u << 16), kB, 0, st>>>(kp, m, flag.as<uint32_t>());
         TC_LAUNCH("k_head_flags");
-        TC_TRY(scan_u32(flag.as<uint32_t>(), pos.as<uint32_t>(), mv, total.as<uint32_t>(), st));
-        TC_CUDA(cudaMemcpyAsync(&E, total.p, sizeof(uint32_t), cudaMemcpyDeviceToHost, st));
-        TC_CUDA(cudaStreamSynchronize(st));
+        TC_TRY(scan_u32(flag.as<uint32_t>(), pos.as<uint32_t>(), m, reinterpret_cast<uint32_t*>(stats.as<uint64_t>() + 14), st));
     }
+    TC_CUDA(cudaMemcpyAsync(hs, stats.p, sizeof(unsigned long long) * kStats, cudaMemcpyDeviceToHost, st));
+    TC_CUDA(cudaStreamSynchronize(st));
+    E = (uint32_t)hs[14];   // little-endian: the scan's total in the low half
     TC_TRY(ukey.alloc(sizeof(uint64_t) * (E ? E : 1), st));
     TC_TRY(udir.alloc(sizeof(uint32_t) * (E ? E : 1), st));
     TC_CUDA(cudaMemsetAsync(udir.p, 0, sizeof(uint32_t) * (E ? E : 1), st));
-    if (mv) {
-        k_unique<<<grid_for(mv, kB, 1u << 16), kB, 0, st>>>(kp, mv, flag.as<uint32_t>(), pos.as<uint32_t>(),
-                                                             ukey.as<uint64_t>(), udir.as<uint32_t>());
+    if (E) {
+        k_unique<<<grid_for(m, kB, 1u << 16), kB, 0, st>>>(kp, m, flag.as<uint32_t>(), pos.as<uint32_t>(),
+                                                          ukey.as<uint64_t>(), udir.as<uint32_t>());
         TC_LAUNCH("k_unique");
     }
     return TC_OK;
@@ -565,8 +580,8 @@ tc_status build_from_arcs(GraphStore& g, uint64_t m, const uint32_t* d_src, cons
     const int B = bits_for(n);
     if (m >= (1ull << 32)) return fail(TC_ERR_RANGE, "more than 2^32-1 arcs");
     DevBuf stats, keys, tmp;
-    TC_TRY(stats.alloc(sizeof(unsigned long long) * 13, st));
-    TC_CUDA(cudaMemsetAsync(stats.p, 0, sizeof(unsigned long long) * 13, st));
+    TC_TRY(stats.alloc(sizeof(unsigned long long) * kStats, st));
+    TC_CUDA(cudaMemsetAsync(stats.p, 0, sizeof(unsigned long long) * kStats, st));
     TC_TRY(keys.alloc(sizeof(uint64_t) * (m ? m : 1), st));
     TC_TRY(tmp.alloc(sizeof(uint64_t) * (m ? m : 1), st));
     if (m) {
@@ -574,18 +589,15 @@ tc_status build_from_arcs(GraphStore& g, uint64_t m, const uint32_t* d_src, cons
                                                                stats.as<unsigned long long>());
         TC_LAUNCH("k_make_keys");
     }
-    unsigned long long hs[2];
-    TC_CUDA(cudaMemcpyAsync(hs, stats.p, sizeof(hs), cudaMemcpyDeviceToHost, st));
-    TC_CUDA(cudaStreamSynchronize(st));
-    if (hs[1]) return fail(TC_ERR_RANGE, "arc list holds a vertex id >= n");
-    uint64_t mv = m - hs[0];
     uint64_t* kp = keys.as<uint64_t>();
     uint64_t* tp = tmp.as<uint64_t>();
     TC_TRY(radix_sort_u64(&kp, &tp, m, 2, 2 * B + 2, st));
-    // unique pairs (the self-loops' all-ones keys sort past the mv valid ones)
+    // unique pairs (the keys of self-loops and of ids out of range are all ones and sort past the others)
     DevBuf ukey, udir;
     uint32_t E = 0;
-    TC_TRY(pairs_from_sorted(kp, mv, ukey, udir, E, st));
+    unsigned long long hs[kStats];
+    TC_TRY(pairs_from_sorted(kp, m, ukey, udir, E, stats, hs, st));
+    if (hs[1]) return fail(TC_ERR_RANGE, "arc list holds a vertex id >= n");
     keys.release();
     tmp.release();
     TC_TRY(graph_from_pairs(g, B, E, ukey, udir, stats, st));
@@ -597,10 +609,11 @@ tc_status build_from_sorted_arcs(GraphStore& g, const uint64_t* d_keys, uint64_t
     const int B = bits_for(g.n);
     if (m >= (1ull << 32)) return fail(TC_ERR_RANGE, "more than 2^32-1 arcs");
     DevBuf stats, ukey, udir;
-    TC_TRY(stats.alloc(sizeof(unsigned long long) * 13, st));
-    TC_CUDA(cudaMemsetAsync(stats.p, 0, sizeof(unsigned long long) * 13, st));
+    TC_TRY(stats.alloc(sizeof(unsigned long long) * kStats, st));
+    TC_CUDA(cudaMemsetAsync(stats.p, 0, sizeof(unsigned long long) * kStats, st));
     uint32_t E = 0;
-    TC_TRY(pairs_from_sorted(d_keys, m, ukey, udir, E, st));
+    unsigned long long hs[kStats];
+    TC_TRY(pairs_from_sorted(d_keys, m, ukey, udir, E, stats, hs, st));
     TC_TRY(graph_from_pairs(g, B, E, ukey, udir, stats, st));
     g.dups = m - g.arcs;
     return TC_OK;
@@ -617,8 +630,8 @@ tc_status build_from_csr(GraphStore& g, const uint64_t* d_off, const uint32_t* d
     if (total_h & 1) return fail(TC_ERR_ARG, "CSR is not symmetric (odd number of entries)");
     if (total_h >= (1ull << 32)) return fail(TC_ERR_RANGE, "more than 2^32-1 CSR entries");
     DevBuf stats;
-    TC_TRY(stats.alloc(sizeof(unsigned long long) * 13, st));
-    TC_CUDA(cudaMemsetAsync(stats.p, 0, sizeof(unsigned long long) * 13, st));
+    TC_TRY(stats.alloc(sizeof(unsigned long long) * kStats, st));
+    TC_CUDA(cudaMemsetAsync(stats.p, 0, sizeof(unsigned long long) * kStats, st));
     const unsigned gridN = grid_for(n, kB, 1u << 16);
     k_check_csr<<<gridN, kB, 0, st>>>(d_off, d_adj, n, total_h, stats.as<unsigned long long>());
     TC_LAUNCH("k_check_csr");

@@ -1025,14 +1025,16 @@ tc_status get_plan(GraphStore& g, const Opts& o, cudaStream_t st, Plan** out) {
     p.items.release();
     p.key = o;
     const GraphDev gd = g.dev();
-    DevBuf cnt1;
-    TC_TRY(cnt1.alloc(sizeof(uint32_t), st));
-    TC_CUDA(cudaMemsetAsync(cnt1.p, 0, sizeof(uint32_t), st));
-    k_count_gt<<<grid_for(g.n, 256, 4096), 256, 0, st>>>(gd.off, g.n, o.warp_max_deg, cnt1.as<uint32_t>());
-    TC_LAUNCH("k_count_gt");
-    uint32_t u_end = 0;
-    TC_CUDA(cudaMemcpyAsync(&u_end, cnt1.p, sizeof(uint32_t), cudaMemcpyDeviceToHost, st));
-    TC_CUDA(cudaStreamSynchronize(st));
+    uint32_t u_end = g.n_gt64;   // counted by the build
+    if (o.warp_max_deg != 64u) {
+        DevBuf cnt1;
+        TC_TRY(cnt1.alloc(sizeof(uint32_t), st));
+        TC_CUDA(cudaMemsetAsync(cnt1.p, 0, sizeof(uint32_t), st));
+        k_count_gt<<<grid_for(g.n, 256, 4096), 256, 0, st>>>(gd.off, g.n, o.warp_max_deg, cnt1.as<uint32_t>());
+        TC_LAUNCH("k_count_gt");
+        TC_CUDA(cudaMemcpyAsync(&u_end, cnt1.p, sizeof(uint32_t), cudaMemcpyDeviceToHost, st));
+        TC_CUDA(cudaStreamSynchronize(st));
+    }
     p.warp_begin = u_end;
     p.warp_end = g.n_active;
     p.n_items = 0;

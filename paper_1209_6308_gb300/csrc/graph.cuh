@@ -64,7 +64,8 @@ struct GraphStore {
     uint64_t sum_walk_map = 0;   // walked entries with ids below kMapIdsSuffix
     uint64_t sum_tri_walk = 0;   // sum of up (up - 1) / 2: the entries the triangle form walks
     uint32_t n_hub = 0;          // vertices with deg > kHubDeg: ids [0, n_hub)
-    uint32_t n_wide = 0;         // vertices with deg > 32
+    uint32_t n_gt64 = 0, n_wide = 0;   // vertices with deg > 64, > 32
+    DevBuf store, scratch;       // what the buffers below are carved from (not rec, blk16, cost)
     DevBuf off, adj, up, new_of_old;
     DevBuf ub, rp, vs, us;   // per upper pair tables (see GraphDev)
     DevBuf rec, blk16;   // 16-bit lower lists (see GraphDev): rec holds rec, rec2 and n16 of the active vertices

@@ -33,18 +33,26 @@ tc_status cuda_fail(cudaError_t e, const char* what);
     } while (0)
 
 // Device buffer: alloc() is stream-ordered (freed on the same stream when released),
-// alloc_persistent() is a plain cudaMalloc for buffers that outlive the creating stream.
+// alloc_persistent() is a plain cudaMalloc for buffers that outlive the creating stream, and
+// carve() a part of another buffer, which must live as long.
 struct DevBuf {
     void* p = nullptr;
     size_t bytes = 0;
     cudaStream_t st = nullptr;
     bool async = false;
+    bool owned = true;
     DevBuf() = default;
     DevBuf(const DevBuf&) = delete;
     DevBuf& operator=(const DevBuf&) = delete;
     ~DevBuf() { release(); }
     tc_status alloc(size_t b, cudaStream_t s);
     tc_status alloc_persistent(size_t b);
+    void carve(const DevBuf& from, size_t at, size_t b) {
+        release();
+        p = static_cast<unsigned char*>(from.p) + at;
+        bytes = b;
+        owned = false;
+    }
     void release();
     template <typename T> T* as() const { return static_cast<T*>(p); }
 };

@@ -500,7 +500,7 @@ __global__ void k_tri_collect(TriCollect a, Table64 T) {
     for (uint32_t k = t; k < kBatchStride; k += blockDim.x) sc[k] = 0ull;
 }
 
-std::atomic<uint64_t> g_tri_attr[4] = {};
+std::atomic<int> g_tri_limit[4][64] = {};   // dynamic shared memory the form's kernel was set to, per device
 
 size_t tri_smem(uint32_t chunk, bool old) {
     const size_t slots = 2ull * chunk;
@@ -512,20 +512,20 @@ size_t tri_smem(uint32_t chunk, bool old) {
 tc_status tri_prepare(int form, size_t smem) {
     int dev = 0;
     TC_CUDA(cudaGetDevice(&dev));
-    const uint64_t bit = 1ull << (dev & 63);
-    const void* fns[4] = {(const void*)k_triangles<false, kTriSingle>, (const void*)k_triangles<true, kTriSingle>,
-                          (const void*)k_triangles<false, kTriBatch>, (const void*)k_triangles<false, kTriWave>};
-    const void* fn = fns[form];
-    int optin = 0;
-    TC_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-    cudaFuncAttributes fa;
-    TC_CUDA(cudaFuncGetAttributes(&fa, fn));
-    const int lim = optin - (int)fa.sharedSizeBytes;
-    if ((int)smem > lim) return fail(TC_ERR_ARG, "chunk_entries too large for this GPU's shared memory");
-    if (!(g_tri_attr[form].load() & bit)) {
-        TC_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, lim));
-        g_tri_attr[form].fetch_or(bit);
+    std::atomic<int>& limit = g_tri_limit[form][dev & 63];
+    int lim = limit.load();
+    if (!lim) {
+        const void* fns[4] = {(const void*)k_triangles<false, kTriSingle>, (const void*)k_triangles<true, kTriSingle>,
+                              (const void*)k_triangles<false, kTriBatch>, (const void*)k_triangles<false, kTriWave>};
+        int optin = 0;
+        TC_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+        cudaFuncAttributes fa;
+        TC_CUDA(cudaFuncGetAttributes(&fa, fns[form]));
+        lim = optin - (int)fa.sharedSizeBytes;
+        TC_CUDA(cudaFuncSetAttribute(fns[form], cudaFuncAttributeMaxDynamicSharedMemorySize, lim));
+        limit.store(lim);
     }
+    if ((int)smem > lim) return fail(TC_ERR_ARG, "chunk_entries too large for this GPU's shared memory");
     return TC_OK;
 }
 
@@ -576,9 +576,8 @@ tc_status triangle_census_enqueue(GraphStore& g, const Opts& o, const Plan& p, u
         return TC_OK;
     }
     if (!g.vs.p) return fail(TC_ERR_ARG, "the triangle form needs the per upper pair tables");
-    // [0, 21) bulk sums, [32, 96) triangle tricodes, then 8 work counters: zeroed at once
+    // [0, 21) bulk sums, [32, 96) triangle tricodes, then 8 work counters: zeroed at once (g.tri holds them)
     constexpr size_t kScratch = sizeof(unsigned long long) * kBatchStride + sizeof(uint32_t) * 8;
-    if (!g.tri.p) TC_TRY(g.tri.alloc_persistent(kScratch));
     unsigned long long* raw = g.tri.as<unsigned long long>();
     unsigned long long* hist = raw + 32;
     uint32_t* ctr = reinterpret_cast<uint32_t*>(raw + kBatchStride);
