@@ -52,6 +52,7 @@ __global__ void __launch_bounds__(kThreads, 8) k_triangles(TriParams P) {
     uint32_t* sHist = sWO + (OLD ? kWarps * kWarpSlots : 0u);         // [kWarps][64]
     uint8_t* sPerm = reinterpret_cast<uint8_t*>(sHist + kWarps * 64);  // [9][64] OLD
     __shared__ uint32_t s_item, s_next;
+    __shared__ uint8_t s_at[kWarps][32];   // walk_pairs' scratch
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     // the whole-warp walk of long prefixes, except in a batch of graphs (small graphs, short
@@ -119,7 +120,7 @@ __global__ void __launch_bounds__(kThreads, 8) k_triangles(TriParams P) {
                 grab_pairs(&s_next, w.j1, lane, jb, g);
                 if (jb >= w.j1) break;
                 since_flush += walk_pairs<OLD, true, kLongWalk>(P, G, bbase, pb, jb, min(jb + g, w.j1), sH, nullptr, 0, 0u, ob,
-                                                     sPerm, myHist, lane);
+                                                     sPerm, myHist, s_at[warp], lane);
                 if (since_flush >= kFlushElems) {
                     flush_warp_hist(myHist, ghist, lane);
                     since_flush = 0;
@@ -148,7 +149,7 @@ __global__ void __launch_bounds__(kThreads, 8) k_triangles(TriParams P) {
                 grab_pairs(&s_next, w.j1, lane, jb, g);
                 if (jb >= w.j1) break;
                 since_flush += walk_pairs<OLD, false, kLongWalk>(P, G, bbase, pb, jb, min(jb + g, w.j1), sH, sO, hb, hmask, ob,
-                                                      sPerm, myHist, lane);
+                                                      sPerm, myHist, s_at[warp], lane);
                 if (since_flush >= kFlushElems) {
                     flush_warp_hist(myHist, ghist, lane);
                     since_flush = 0;
@@ -212,7 +213,7 @@ __global__ void __launch_bounds__(kThreads, 8) k_triangles(TriParams P) {
             }
             __syncwarp();
             since_flush += walk_pairs<OLD, false, false>(P, G, bbase, G.ub[b] - lb, lb, db, wH, wO, hb, hmask,
-                                                  OLD ? P.old[b] : 0u, sPerm, myHist, lane);
+                                                  OLD ? P.old[b] : 0u, sPerm, myHist, s_at[warp], lane);
             if (since_flush >= kFlushElems) {
                 flush_warp_hist(myHist, ghist, lane);
                 since_flush = 0;
@@ -284,6 +285,7 @@ __device__ __forceinline__ void flush_bulk(unsigned long long (&acc)[3][7], unsi
 
 template <int MODE>
 __global__ void __launch_bounds__(256, 4) k_pair_bulk(BulkParams P) {
+    __shared__ uint8_t s_at[kWarps][32];
     const uint32_t lane = threadIdx.x & 31;
     const uint32_t le_mask = (2u << lane) - 1u;
     unsigned long long acc[3][7];
@@ -362,7 +364,7 @@ __global__ void __launch_bounds__(256, 4) k_pair_bulk(BulkParams P) {
         const uint32_t nz = __ballot_sync(0xffffffffu, cnt != 0u);
         if (!nz) continue;
         const uint32_t nv = __popc(nz);
-        const uint32_t src = __fns(nz, 0, lane + 1) & 31u;
+        const uint32_t src = nth_set(nz, cnt != 0u, s_at[threadIdx.x >> 5], (int)lane);
         ubase = __shfl_sync(0xffffffffu, ubase, src);
         du = __shfl_sync(0xffffffffu, du, src);
         upu = __shfl_sync(0xffffffffu, upu, src);

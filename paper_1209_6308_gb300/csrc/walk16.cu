@@ -51,6 +51,7 @@ struct Flat {
     uint32_t start[kWindow / 32];               // bit per block of the window that starts a segment
     uint16_t at[kWindow / 32];                  // the segment of each 32nd block of the window
     uint32_t hist[kW16][64];                    // the warps' tricodes
+    uint8_t lanes[kW16][32];                    // walk_pairs' scratch
     uint32_t nblk[kW16], nseg[kW16];
     Item item;                                  // the next item and its vertex's list: offset, table index,
     uint64_t base, table;                       // lower entries, entries in the 16-bit list
@@ -408,7 +409,7 @@ struct Runner {
                 grab_pairs(&F.next, j1, lane, jb, g);
                 if (jb >= j1) break;
                 walked += walk_pairs<false, false, true, REST>(P, P.g, bbase, pb, jb, min(jb + g, j1), sH, nullptr, hb,
-                                                               hmask, 0u, nullptr, F.hist[warp], lane);
+                                                               hmask, 0u, nullptr, F.hist[warp], F.lanes[warp], lane);
                 if (walked >= kFlushElems) flush_all();
             }
         }
@@ -676,6 +677,7 @@ __global__ void __launch_bounds__(kT16, kCtas16) k_walk_table(TriParams P, Stamp
 // The small vertices' items and the one-warp vertices, a warp each.
 __global__ void __launch_bounds__(kT16, kCtasWarp) k_walk_warp(TriParams P, Stamps T) {
     __shared__ uint32_t s_hash[kW16][kWarpSlots16], s_hist[kW16][64];
+    __shared__ uint8_t s_at[kW16][32];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const GraphDev& G = P.g;
     if (P.phase && T.start) Runner::stamp(P, 0, T.grid, tri_clock_ns());
@@ -705,7 +707,7 @@ __global__ void __launch_bounds__(kT16, kCtasWarp) k_walk_warp(TriParams P, Stam
         }
         __syncwarp();
         walked += walk_pairs<false, false, false>(P, G, bbase, G.ub[b] - lb, j0, j1, wH, nullptr, hb, hmask, 0u, nullptr,
-                                                 s_hist[warp], lane);
+                                                 s_hist[warp], s_at[warp], lane);
         if (walked >= kFlushElems) {
             flush_warp_hist(s_hist[warp], P.hist, lane);
             walked = 0;
