@@ -226,6 +226,160 @@ __device__ __forceinline__ uint32_t walk_pairs(const TriParams& P, const GraphDe
     return walked;
 }
 
+// Walk the entries adj[cb, cb + len) of each lane's pair as one flattened range: count(e, tag) for each
+// entry e, with its pair's tag (e = 0 past the end).  Returns the entries (warp-uniform).
+template <typename Count>
+__device__ __forceinline__ uint32_t walk_flat(const uint32_t* __restrict__ adj, uint64_t cb, uint32_t len, uint32_t tag,
+                                              volatile uint8_t* at, int lane, Count count) {
+    const uint32_t le_mask = (2u << lane) - 1u;
+    const uint32_t nz = __ballot_sync(0xffffffffu, len != 0u);
+    if (!nz) return 0u;
+    const uint32_t cnt = __popc(nz), src = nth_set(nz, len != 0u, at, lane);
+    cb = __shfl_sync(0xffffffffu, cb, src);
+    len = __shfl_sync(0xffffffffu, len, src);
+    tag = __shfl_sync(0xffffffffu, tag, src);
+    if ((uint32_t)lane >= cnt) len = 0u;
+    uint32_t incl = len;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += y;
+    }
+    const uint32_t excl = incl - len, total = __shfl_sync(0xffffffffu, incl, 31);
+    const uint64_t cbx = cb - excl;   // entry i of the range is adj[cbx + i] for the pair that holds it
+    int before = -1;
+    // two rounds of 32 entries at a time: lane i's pair is the last one started at or before its entry
+    for (uint32_t base = 0; base < total; base += 64) {
+        const bool st = (uint32_t)lane < cnt;
+        const uint32_t ra = excl - base, rb = ra - 32u;
+        const uint32_t MA = __reduce_or_sync(0xffffffffu, st && ra < 32u ? 1u << ra : 0u);
+        const uint32_t MB = __reduce_or_sync(0xffffffffu, st && rb < 32u ? 1u << rb : 0u);
+        const uint32_t sa = (uint32_t)(before + __popc(MA & le_mask)) & 31u;
+        before += __popc(MA);
+        const uint32_t sb = (uint32_t)(before + __popc(MB & le_mask)) & 31u;
+        before += __popc(MB);
+        const uint64_t BA = __shfl_sync(0xffffffffu, cbx, sa), BB = __shfl_sync(0xffffffffu, cbx, sb);
+        const uint32_t TA = __shfl_sync(0xffffffffu, tag, sa), TB = __shfl_sync(0xffffffffu, tag, sb);
+        const uint32_t iA = base + lane, iB = iA + 32u;
+        const uint32_t xA = iA < total ? __ldg(adj + (BA + iA)) : 0u;
+        const uint32_t xB = iB < total ? __ldg(adj + (BB + iB)) : 0u;
+        count(xA, TA);
+        count(xB, TB);
+    }
+    return total;
+}
+
+// The one-warp vertices b in [b0, b1), at most 32 consecutive ones.  Most have a handful of pairs, so
+// one at a time leaves the lanes idle and waits for each one's loads in turn: here as many as fit
+// (32 upper pairs, kPackLower lower entries, 2^rb rows) are walked together, a lane per pair,
+// against one hash of all their lower neighbours, keyed by (a, row): (a << rb | row) << 2 | dir fits
+// a 32-bit slot, rb = the bits an id leaves over, at most 5.  A vertex with more than 32 upper pairs
+// goes alone.  1024 batched Chung-Lu graphs (mean degree 8): 5.54 -> 4.53 ms.  Returns the entries walked.
+constexpr uint32_t kPackLower = kWarpSlots / 2;
+__device__ __forceinline__ uint32_t walk_rows(const TriParams& P, const GraphDev& G, uint32_t b0, uint32_t b1, uint32_t* wH,
+                                              uint32_t* myHist, volatile uint8_t* at, int lane) {
+    const uint32_t* __restrict__ adj = G.adj;
+    const uint32_t rb = min(5u, 30u - (32u - __clz(G.n - 1u | 1u)));
+    const uint32_t x = b0 + lane;
+    const bool ok = x < b1;
+    const uint64_t base = ok ? G.off[x] : 0ull, pb = ok ? G.ub[x] : 0ull;
+    uint32_t low = ok ? G.up[x] : 0u;
+    uint32_t pairs = ok ? (uint32_t)(G.off[x + 1] - base) - low : 0u;
+    // no lower or no upper neighbour: no triangle has b in the middle
+    if (!low || !pairs) low = pairs = 0u;
+    const bool alone = pairs > 32u;
+    // both counts' prefixes in one scan (at most 32 x 128 and 32 x 32)
+    uint32_t incl = alone ? 0u : low << 16 | pairs;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += y;
+    }
+    const uint32_t excl = incl - (alone ? 0u : low << 16 | pairs);
+    uint32_t rest = __ballot_sync(0xffffffffu, pairs != 0u), walked = 0;
+    while (rest) {
+        const uint32_t r = __ffs(rest) - 1u;
+        if (__shfl_sync(0xffffffffu, alone, r)) {
+            rest &= rest - 1u;
+            const uint64_t bb = __shfl_sync(0xffffffffu, base, r), pr = __shfl_sync(0xffffffffu, pb, r);
+            const uint32_t lb = __shfl_sync(0xffffffffu, low, r), cnt = __shfl_sync(0xffffffffu, pairs, r);
+            int hb = 6;
+            while ((1u << hb) < 2u * lb) ++hb;
+            const uint32_t hmask = (1u << hb) - 1u;
+            __syncwarp();
+            for (uint32_t k = lane; k < (1u << hb); k += 32) wH[k] = 0u;
+            __syncwarp();
+            for (uint32_t k = lane; k < lb; k += 32) {
+                const uint32_t e = adj[bb + k];
+                uint32_t h = tri_hash(e >> 2, hb);
+                while (atomicCAS(&wH[h], 0u, e) != 0u) h = (h + 1u) & hmask;
+            }
+            __syncwarp();
+            walked += walk_pairs<false, false, false>(P, G, bb, pr - lb, lb, lb + cnt, wH, nullptr, hb, hmask, 0u, nullptr,
+                                                      myHist, at, lane);
+            continue;
+        }
+        const uint32_t from = __shfl_sync(0xffffffffu, excl, r);
+        const uint32_t mine = incl - from;   // rows r .. lane: lower entries << 16 | pairs
+        const uint32_t over = __ballot_sync(0xffffffffu, (uint32_t)lane >= r && (alone || (mine & 0xffffu) > 32u ||
+                                                                               (mine >> 16) > kPackLower || lane - r >= 1u << rb));
+        const uint32_t end = over ? __ffs(over) - 1u : 32u;
+        rest &= end == 32u ? 0u : ~((1u << end) - 1u);
+        const uint32_t sum = __shfl_sync(0xffffffffu, mine, end - 1u), n_low = sum >> 16, n_pairs = sum & 0xffffu;
+        // the row of the pack's i-th lower entry (sh = 16) or pair (sh = 0): the first one whose prefix passes i
+        auto row_of = [&](uint32_t i, uint32_t sh) {
+            uint32_t lo = r, hi = end - 1u;
+#pragma unroll
+            for (int s = 0; s < 5; ++s) {
+                const uint32_t mid = (lo + hi) >> 1;
+                const uint32_t v = __shfl_sync(0xffffffffu, mine, mid) >> sh & 0xffffu;
+                if (lo < hi) {
+                    if (v > i) hi = mid;
+                    else lo = mid + 1u;
+                }
+            }
+            return lo;
+        };
+        int hb = 6;
+        while ((1u << hb) < 2u * n_low) ++hb;
+        const uint32_t hmask = (1u << hb) - 1u;
+        __syncwarp();
+        for (uint32_t k = lane; k < (1u << hb); k += 32) wH[k] = 0u;
+        // this lane's pair, its loads on their way while the hash is filled
+        uint32_t row = row_of(lane, 0u);
+        const uint32_t my = lane - ((__shfl_sync(0xffffffffu, excl, row) - from) & 0xffffu);
+        const uint64_t rbase = __shfl_sync(0xffffffffu, base, row), rpb = __shfl_sync(0xffffffffu, pb, row);
+        const uint32_t rlow = __shfl_sync(0xffffffffu, low, row);
+        const bool valid = (uint32_t)lane < n_pairs;
+        const uint32_t e_bc = valid ? __ldg(adj + rbase + rlow + my) : 0u;
+        const uint32_t len = valid ? __ldg(G.rp + rpb + my) : 0u;
+        __syncwarp();
+        for (uint32_t i0 = 0; i0 < n_low; i0 += 32) {
+            const uint32_t i = i0 + lane, q = row_of(i, 16u);
+            const uint64_t qb = __shfl_sync(0xffffffffu, base, q);
+            const uint32_t first = (__shfl_sync(0xffffffffu, excl, q) - from) >> 16;
+            if (i < n_low) {
+                const uint32_t e = __ldg(adj + qb + (i - first)), key = ((e >> 2) << rb | (q - r)) << 2 | (e & 3u);
+                uint32_t h = tri_hash(key >> 2, hb);
+                while (atomicCAS(&wH[h], 0u, key) != 0u) h = (h + 1u) & hmask;
+            }
+        }
+        const uint64_t cb = len ? G.off[e_bc >> 2] : 0ull;
+        __syncwarp();
+        walked += walk_flat(adj, cb, len, (row - r) << 8 | (e_bc & 3u) << 2, at, lane, [&](uint32_t e_ca, uint32_t tag) {
+            if (!e_ca) return;
+            const uint32_t key = (e_ca >> 2) << rb | tag >> 8;
+            uint32_t h = tri_hash(key, hb), e = wH[h];
+            while (e != 0u && (e >> 2) != key) {
+                h = (h + 1u) & hmask;
+                e = wH[h];
+            }
+            if (e) atomicAdd(&myHist[tri_code(e & 3u, tag & 255u, e_ca)], 1u);
+        });
+    }
+    return walked;
+}
+
 // A warp's next pairs of the CTA's item: guided sizes, 32 pairs while many remain, then fewer
 // (down to 4) as the item runs out, so that the warps reach the item's end barrier together.
 __device__ __forceinline__ void grab_pairs(uint32_t* s_next, uint32_t j1, int lane, uint32_t& jb, uint32_t& g) {

@@ -33,7 +33,7 @@ namespace {
 constexpr int kT16 = 256;                       // threads of a CTA = pairs of a batch
 constexpr int kW16 = kT16 / 32;
 constexpr int kCtas16 = 4;                      // resident CTAs per SM (shared memory, 64 registers)
-constexpr int kCtasWarp = 8;                    // of k_walk_warp
+constexpr int kCtasWarp = 6;                    // of k_walk_warp
 // rounds of a warp in flight (scale 26, k_walk16 at 2 / 3 / 4: 282 / 279 / 330 ms, 4 spills)
 constexpr int kRing = 3, kRingTable = 2;
 constexpr uint32_t kWindow = 8192;              // blocks of the flattened range per window
@@ -685,15 +685,11 @@ __global__ void __launch_bounds__(kT16, kCtasWarp) k_walk_warp(TriParams P, Stam
     __syncwarp();
     uint32_t* wH = s_hash[warp];
     uint32_t walked = 0;
-    // the pairs [j0, j1) of b (j1 = 0: all of its upper pairs) against a hash of L(b)
+    // the pairs [j0, j1) of b against a hash of L(b)
     auto walk = [&](uint32_t b, uint32_t j0, uint32_t j1) {
         const uint64_t bbase = G.off[b];
         const uint32_t lb = G.up[b];
-        if (j1 == 0u) {
-            j0 = lb;
-            j1 = (uint32_t)(G.off[b + 1] - bbase);
-        }
-        if (lb == 0u || j0 >= j1) return;   // no lower or no upper neighbour: no triangle has b in the middle
+        if (lb == 0u || j0 >= j1) return;   // no triangle has b in the middle
         int hb = 6;
         while ((1u << hb) < 2u * lb) ++hb;
         const uint32_t hmask = (1u << hb) - 1u;
@@ -734,7 +730,11 @@ __global__ void __launch_bounds__(kT16, kCtasWarp) k_walk_warp(TriParams P, Stam
         vb = __shfl_sync(0xffffffffu, vb, 0);
         if (vb >= P.warp_end - P.warp_begin) break;
         const uint32_t b0 = P.warp_begin + vb, b1 = min(b0 + (1u << P.wshift), P.warp_end);
-        for (uint32_t b = b0; b < b1; ++b) walk(b, 0u, 0u);
+        walked += walk_rows(P, G, b0, b1, wH, s_hist[warp], s_at[warp], lane);
+        if (walked >= kFlushElems) {
+            flush_warp_hist(s_hist[warp], P.hist, lane);
+            walked = 0;
+        }
     }
     flush_warp_hist(s_hist[warp], P.hist, lane);
     if (P.phase) {
