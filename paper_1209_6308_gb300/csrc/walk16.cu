@@ -25,6 +25,7 @@
 #include <cstring>
 
 #include "graph.cuh"
+#include "rows.cuh"
 #include "triangles.cuh"
 
 namespace tc {
@@ -94,135 +95,151 @@ __global__ void k_count16(const uint64_t* __restrict__ off, const uint32_t* __re
 }
 
 // The 16-bit lower lists of the vertices that have entries in them (only those are ever a walked
-// pair's c).  A warp takes 32 consecutive vertices, reads their bounds together, and then one vertex
-// at a time, the next one's first entries on their way.  Up to 32 entries are placed at once;
-// longer lists take two passes per window, one that counts the classes and one (from the caches)
-// that places each entry behind the earlier ones of its class.
-__global__ void __launch_bounds__(256) k_lists16(GraphDev g, uint32_t n, const uint32_t* __restrict__ first, uint4* rec,
+// pair's c).  The n_wide vertices of more than 32 neighbours go a warp each, in two passes per window,
+// one that counts the classes and one (from the caches) that places each entry behind the earlier
+// ones of its class; for the others a warp takes 32 vertices (rows.cuh) whose lists share its lanes,
+// an entry's place counted by one ballot per segment (one with entries past the windows goes alone).
+__global__ void __launch_bounds__(256) k_lists16(GraphDev g, uint32_t n, uint32_t n_wide, const uint32_t* __restrict__ first, uint4* rec,
                                                  uint4* rec2, uint16_t* ids) {
+    __shared__ uint8_t s_at[8][32];
     const uint32_t lane = threadIdx.x & 31, lt = (1u << lane) - 1u;
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-    for (uint64_t x0 = blockIdx.x * (uint64_t)blockDim.x + (threadIdx.x & ~31u); x0 < n; x0 += stride) {
+    // classes 1 and 2 of the upper entries of x: the first one, and those after it from its pair's table
+    auto upper = [&](uint64_t x, uint64_t base, uint32_t low, uint32_t deg) {
+        if (low >= deg) return make_uint2(0u, 0u);
+        const uint2 after = g.us[g.ub[x]];
+        const uint32_t d = g.adj[base + low] & 3u;
+        return make_uint2(after.x + (d == 1u), after.y + (d == 2u));
+    };
+    // one list by the whole warp
+    auto long_list = [&](uint64_t x, uint64_t base, uint32_t h, uint32_t f, uint32_t low, uint32_t v1, uint32_t v2) {
+        const uint32_t* __restrict__ L = g.adj + base;
+        uint16_t* lens = reinterpret_cast<uint16_t*>(rec2 + 2 * x);
+        // classes 1 and 2 of all of N[x]: the lower entries past the lists here, those of the lists below
+        uint32_t t1 = 0, t2 = 0;
+        for (uint32_t k = h + lane; k < low; k += 32) {
+            const uint32_t e = L[k];
+            t1 += (e & 3u) == 1u;
+            t2 += (e & 3u) == 2u;
+        }
+        t1 = __reduce_add_sync(0xffffffffu, t1) + v1;
+        t2 = __reduce_add_sync(0xffffffffu, t2) + v2;
+        uint64_t at = 8ull * f;
+        uint32_t k1 = 0;
+        for (uint32_t w = 0; w < 4u; ++w) {
+            const uint32_t k0 = k1;
+            k1 = x <= kWin16 ? h : k0 < h ? entries_below(L, h, (w + 1u) * kWin16) : h;
+            uint32_t a1 = 0, a2 = 0;
+#pragma unroll 4
+            for (uint32_t k = k0 + lane; k < k1; k += 32) {
+                const uint32_t e = L[k];
+                a1 += (e & 3u) == 1u;
+                a2 += (e & 3u) == 2u;
+            }
+            a1 = __reduce_add_sync(0xffffffffu, a1);
+            a2 = __reduce_add_sync(0xffffffffu, a2);
+            const uint32_t a3 = k1 - k0 - a1 - a2;
+            t1 += a1;
+            t2 += a2;
+            if (lane == 0) {
+                if (w == 0) {
+                    rec[x].x = f;
+                    rec[x].y = a1 | (a2 << 16);
+                    if (x >= kWin16) lens[0] = (uint16_t)a3;
+                } else {
+                    lens[3 * w - 2] = (uint16_t)a1;
+                    lens[3 * w - 1] = (uint16_t)a2;
+                    lens[3 * w] = (uint16_t)a3;
+                }
+            }
+            uint64_t p1 = at, p2 = p1 + ((a1 + 7u) & ~7u), p3 = p2 + ((a2 + 7u) & ~7u);
+            at = p3 + ((a3 + 7u) & ~7u);
+            for (uint32_t kb = k0; kb < k1; kb += 32) {
+                const uint32_t k = kb + lane, e = k < k1 ? L[k] : 0u, d = e & 3u;
+                const uint32_t b1 = __ballot_sync(0xffffffffu, d == 1u), b2 = __ballot_sync(0xffffffffu, d == 2u);
+                const uint32_t b3 = __ballot_sync(0xffffffffu, d == 3u);
+                const uint64_t p = d == 1u ? p1 + __popc(b1 & lt)
+                                           : d == 2u ? p2 + __popc(b2 & lt) : p3 + __popc(b3 & lt);
+                if (d) ids[p] = (uint16_t)((e >> 2) & (kWin16 - 1u));
+                p1 += __popc(b1);
+                p2 += __popc(b2);
+                p3 += __popc(b3);
+            }
+            if (lane < 7u) {
+                if (p1 + lane < ((p1 + 7u) & ~7ull)) ids[p1 + lane] = (uint16_t)kPad16;
+                if (p2 + lane < ((p2 + 7u) & ~7ull)) ids[p2 + lane] = (uint16_t)kPad16;
+                if (p3 + lane < ((p3 + 7u) & ~7ull)) ids[p3 + lane] = (uint16_t)kPad16;
+            }
+            if (x < kWin16) break;
+            if (k1 == h) {   // nothing in the windows after this one
+                if (lane >= 3 * w && lane < 9u) lens[lane + 1u] = 0u;
+                break;
+            }
+        }
+        if (lane == 0) {
+            rec[x].z = t1;
+            rec[x].w = t2;
+        }
+    };
+    for (uint64_t x = (blockIdx.x * (uint64_t)blockDim.x + threadIdx.x) >> 5; x < n_wide; x += stride >> 5) {
+        const uint64_t base = g.off[x];
+        const uint32_t h = g.n16[x], low = g.up[x];
+        if (!h) continue;
+        const uint2 v = upper(x, base, low, (uint32_t)(g.off[x + 1] - base));
+        long_list(x, base, h, first[x], low, v.x, v.y);
+    }
+    for (uint64_t x0 = n_wide + blockIdx.x * (uint64_t)blockDim.x + (threadIdx.x & ~31u); x0 < n; x0 += stride) {
         const bool ok = x0 + lane < n;
         const uint64_t vbase = ok ? g.off[x0 + lane] : 0ull;
         const uint32_t vdeg = ok ? (uint32_t)(g.off[x0 + lane + 1] - vbase) : 0u, vlow = ok ? g.up[x0 + lane] : 0u;
         const uint32_t vh = ok ? g.n16[x0 + lane] : 0u, vf = ok ? first[x0 + lane] : 0u;
-        uint2 vup = make_uint2(0u, 0u);   // classes 1 and 2 after the first upper entry, from its pair's table
-        if (vh && vlow < vdeg) vup = g.us[g.ub[x0 + lane]];
-        uint32_t todo = __ballot_sync(0xffffffffu, vh != 0u);
-        uint32_t e_next = 0;
-        if (todo) {
-            const int v = __ffs(todo) - 1;
-            const uint64_t b0 = __shfl_sync(0xffffffffu, vbase, v);
-            if (lane < __shfl_sync(0xffffffffu, vh, v)) e_next = g.adj[b0 + lane];
-        }
-        while (todo) {
-            const int v = __ffs(todo) - 1;
-            todo &= todo - 1u;
-            const uint64_t x = x0 + v, base = __shfl_sync(0xffffffffu, vbase, v);
-            const uint32_t h = __shfl_sync(0xffffffffu, vh, v), f = __shfl_sync(0xffffffffu, vf, v);
-            const uint32_t low = __shfl_sync(0xffffffffu, vlow, v), deg = __shfl_sync(0xffffffffu, vdeg, v);
-            const uint32_t e0 = e_next;
-            const int vn = todo ? __ffs(todo) - 1 : v;
-            const uint64_t bn = __shfl_sync(0xffffffffu, vbase, vn);
-            const uint32_t hn = __shfl_sync(0xffffffffu, vh, vn);
-            e_next = todo && lane < hn ? g.adj[bn + lane] : 0u;
-            const uint32_t* __restrict__ L = g.adj + base;
-            uint16_t* lens = reinterpret_cast<uint16_t*>(rec2 + 2 * x);   // from window 0's class 3 on
-            // classes 1 and 2 of all of N[x]: the lower entries past the lists and the first upper one
-            // here, the later upper ones from the table, those of the lists below
-            uint32_t t1 = 0, t2 = 0;
-            for (uint32_t k = h + lane; k < min(low + 1u, deg); k += 32) {
-                const uint32_t e = L[k];
-                t1 += (e & 3u) == 1u;
-                t2 += (e & 3u) == 2u;
-            }
-            if (h < min(low + 1u, deg)) {   // the same for the whole warp
-                t1 = __reduce_add_sync(0xffffffffu, t1);
-                t2 = __reduce_add_sync(0xffffffffu, t2);
-            }
-            t1 += __shfl_sync(0xffffffffu, vup.x, v);
-            t2 += __shfl_sync(0xffffffffu, vup.y, v);
-            uint64_t at = 8ull * f;
-            uint32_t k1 = 0;
-            for (uint32_t w = 0; w < 4u; ++w) {
-                const uint32_t k0 = k1;
-                uint32_t a1, a2, a3;
-                uint64_t p1, p2, p3;
-                if (h <= 32u) {
-                    const uint32_t d = e0 >> 17 == w ? e0 & 3u : 0u;   // lanes past the list hold 0
-                    const uint32_t b1 = __ballot_sync(0xffffffffu, d == 1u), b2 = __ballot_sync(0xffffffffu, d == 2u);
-                    const uint32_t b3 = __ballot_sync(0xffffffffu, d == 3u);
-                    a1 = __popc(b1);
-                    a2 = __popc(b2);
-                    a3 = __popc(b3);
-                    k1 = k0 + a1 + a2 + a3;
-                    p1 = at;
-                    p2 = p1 + ((a1 + 7u) & ~7u);
-                    p3 = p2 + ((a2 + 7u) & ~7u);
-                    at = p3 + ((a3 + 7u) & ~7u);
-                    const uint64_t p = d == 1u ? p1 + __popc(b1 & lt) : d == 2u ? p2 + __popc(b2 & lt) : p3 + __popc(b3 & lt);
-                    if (d) ids[p] = (uint16_t)((e0 >> 2) & (kWin16 - 1u));
-                    p1 += a1;
-                    p2 += a2;
-                    p3 += a3;
-                } else {
-                    k1 = x <= kWin16 ? h : k0 < h ? entries_below(L, h, (w + 1u) * kWin16) : h;
-                    a1 = a2 = 0;
-#pragma unroll 4
-                    for (uint32_t k = k0 + lane; k < k1; k += 32) {
-                        const uint32_t e = L[k];
-                        a1 += (e & 3u) == 1u;
-                        a2 += (e & 3u) == 2u;
+        const uint2 vu = vh ? upper(x0 + lane, vbase, vlow, vdeg) : make_uint2(0u, 0u);
+        const uint32_t v1 = vu.x, v2 = vu.y;
+        for_rows(vlow != vh ? 33u : vh, s_at[threadIdx.x >> 5],
+            [&](const PackedEntry& p) {
+                const uint64_t base = __shfl_sync(0xffffffffu, vbase, p.row), x = x0 + p.row;
+                const uint32_t f = __shfl_sync(0xffffffffu, vf, p.row);
+                uint32_t t1 = __shfl_sync(0xffffffffu, v1, p.row), t2 = __shfl_sync(0xffffffffu, v2, p.row);
+                const uint32_t e = p.valid ? g.adj[base + (lane - p.first)] : 0u, d = e & 3u, w = e >> 17;
+                const uint32_t last = __reduce_max_sync(0xffffffffu, w);   // windows the pack's entries lie in
+                const bool head = p.valid && lane == p.first;
+                uint16_t* lens = reinterpret_cast<uint16_t*>(rec2 + 2 * x);   // from window 0's class 3 on
+                uint32_t blocks = 0, at = 0, cls1 = 0;   // of the row's segments so far; this entry's place
+                uint32_t pads = 0;
+                for (uint32_t v = 0; v <= last; ++v)
+#pragma unroll
+                    for (uint32_t q = 1; q <= 3; ++q) {
+                        const uint32_t m = __ballot_sync(0xffffffffu, d == q && w == v) & p.lanes, cnt = __popc(m);
+                        if (d == q && w == v) {
+                            at = 8u * blocks + __popc(m & lt);
+                            pads = (m & lt) ? 0u : (0u - cnt) & 7u;   // the segment's first entry pads it
+                            if (pads) pads |= (8u * blocks + cnt) << 8;
+                        }
+                        blocks += (cnt + 7u) >> 3;
+                        t1 += q == 1u ? cnt : 0u;
+                        t2 += q == 2u ? cnt : 0u;
+                        if (head) {
+                            if (v == 0u && q == 1u) cls1 = cnt;
+                            else if (v == 0u && q == 2u) rec[x] = make_uint4(f, cls1 | (cnt << 16), 0u, 0u);
+                            else if (x >= kWin16) lens[v == 0u ? 0u : 3u * v - 3u + q] = (uint16_t)cnt;
+                        }
                     }
-                    a1 = __reduce_add_sync(0xffffffffu, a1);
-                    a2 = __reduce_add_sync(0xffffffffu, a2);
-                    a3 = k1 - k0 - a1 - a2;
-                    p1 = at;
-                    p2 = p1 + ((a1 + 7u) & ~7u);
-                    p3 = p2 + ((a2 + 7u) & ~7u);
-                    at = p3 + ((a3 + 7u) & ~7u);
-                    for (uint32_t kb = k0; kb < k1; kb += 32) {
-                        const uint32_t k = kb + lane, e = k < k1 ? L[k] : 0u, d = e & 3u;
-                        const uint32_t b1 = __ballot_sync(0xffffffffu, d == 1u), b2 = __ballot_sync(0xffffffffu, d == 2u);
-                        const uint32_t b3 = __ballot_sync(0xffffffffu, d == 3u);
-                        const uint64_t p = d == 1u ? p1 + __popc(b1 & lt)
-                                                   : d == 2u ? p2 + __popc(b2 & lt) : p3 + __popc(b3 & lt);
-                        if (d) ids[p] = (uint16_t)((e >> 2) & (kWin16 - 1u));
-                        p1 += __popc(b1);
-                        p2 += __popc(b2);
-                        p3 += __popc(b3);
-                    }
+                if (p.valid) {
+                    ids[8ull * f + at] = (uint16_t)((e >> 2) & (kWin16 - 1u));
+                    for (uint32_t k = 0; k < (pads & 255u); ++k) ids[8ull * f + (pads >> 8) + k] = (uint16_t)kPad16;
                 }
-                t1 += a1;
-                t2 += a2;
-                if (lane == 0) {
-                    if (w == 0) {
-                        rec[x].x = f;
-                        rec[x].y = a1 | (a2 << 16);
-                        if (x >= kWin16) lens[0] = (uint16_t)a3;
-                    } else {
-                        lens[3 * w - 2] = (uint16_t)a1;
-                        lens[3 * w - 1] = (uint16_t)a2;
-                        lens[3 * w] = (uint16_t)a3;
-                    }
+                if (head) {
+                    if (x >= kWin16)
+                        for (uint32_t k = 3u * last + 1u; k < 10u; ++k) lens[k] = 0u;
+                    rec[x].z = t1;
+                    rec[x].w = t2;
                 }
-                if (lane < 7u) {
-                    if (p1 + lane < ((p1 + 7u) & ~7ull)) ids[p1 + lane] = (uint16_t)kPad16;
-                    if (p2 + lane < ((p2 + 7u) & ~7ull)) ids[p2 + lane] = (uint16_t)kPad16;
-                    if (p3 + lane < ((p3 + 7u) & ~7ull)) ids[p3 + lane] = (uint16_t)kPad16;
-                }
-                if (x < kWin16) break;
-                if (k1 == h) {   // nothing in the windows after this one
-                    if (lane >= 3 * w && lane < 9u) lens[lane + 1u] = 0u;
-                    break;
-                }
-            }
-            if (lane == 0) {
-                rec[x].z = t1;
-                rec[x].w = t2;
-            }
-        }
+            },
+            [&](uint32_t row) {
+                long_list(x0 + row, __shfl_sync(0xffffffffu, vbase, row), __shfl_sync(0xffffffffu, vh, row),
+                          __shfl_sync(0xffffffffu, vf, row), __shfl_sync(0xffffffffu, vlow, row),
+                          __shfl_sync(0xffffffffu, v1, row), __shfl_sync(0xffffffffu, v2, row));
+            });
     }
 }
 
@@ -771,7 +788,7 @@ tc_status lists16_build(GraphStore& g, cudaStream_t st) {
     TC_CUDA(cudaStreamSynchronize(st));
     DevBuf blk;
     TC_TRY(blk.alloc_persistent(sizeof(uint4) * (n_blocks ? n_blocks : 1u)));
-    k_lists16<<<grid_for(n, 256, 1u << 16), 256, 0, st>>>(gd, n, first.as<uint32_t>(), g.rec.as<uint4>(),
+    k_lists16<<<grid_for(n, 256, 1u << 16), 256, 0, st>>>(gd, n, g.n_wide, first.as<uint32_t>(), g.rec.as<uint4>(),
                                                           g.rec.as<uint4>() + n, blk.as<uint16_t>());
     TC_LAUNCH("k_lists16");
     TC_CUDA(cudaStreamSynchronize(st));   // later censuses may come on other streams
