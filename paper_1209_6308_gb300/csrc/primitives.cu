@@ -10,7 +10,7 @@
 // Scan: tiles of 4096 values, one kernel.
 // Radix sort: 8-bit digits; one kernel counts every digit of every pass, then one kernel per pass
 // ranks a tile's keys stably (per warp: the lanes sharing a digit, by eight ballots, against the
-// warp's running counts), looks back per digit, stages the tile in shared memory in digit order
+// running counts of its half of the warp's keys), looks back per digit, stages the tile in shared memory in digit order
 // and writes contiguous runs per digit ("onesweep", Adinets and Merrill 2022).  16 bytes per key and
 // pass where a histogram, a scan and a scatter per pass moved 24 in five kernels.
 #include <algorithm>
@@ -23,12 +23,15 @@ namespace {
 constexpr int kScanThreads = 256;
 constexpr int kScanPer = 16;
 constexpr int kScanTile = kScanThreads * kScanPer;
-constexpr int kSortThreads = 512;
+// (scale-25 build in ms with 512 / 384 / 256 threads of 16 keys: 139.5 / 137.3 / 147.7; 384 of 12 keys or
+// __match_any_sync in place of the ballots are slower.)
+constexpr int kSortThreads = 384;
 constexpr int kSortWarps = kSortThreads / 32;
 constexpr int kSortPer = 16;
 constexpr int kSortTile = kSortThreads * kSortPer;
 constexpr int kPasses = 8;                      // of 8 bits
 constexpr uint32_t kPatience = 1u << 16;
+constexpr int kLook = 4;   // predecessors a sort tile looks at together
 
 // A tile's published sums: the value, and in the top bits which one it is.
 constexpr unsigned long long kOwn = 1ull << 62, kUpTo = 2ull << 62, kValue = kOwn - 1ull;
@@ -202,16 +205,15 @@ __global__ void __launch_bounds__(kSortThreads) k_digit_counts(const uint64_t* _
 
 struct SortShared {
     uint64_t keys[kSortTile];
-    uint32_t wh[kSortWarps][256];   // a warp's keys per digit; then its first place behind the earlier warps'
-    uint32_t start[256];            // first place of a digit in the tile
-    uint32_t to[256];               // first place of a digit of this tile in the output, less start
+    uint16_t wh[2 * kSortWarps][256];   // a half warp-segment's keys per digit; then its first place in the tile
+    uint32_t to[256];                   // first place of a digit of this tile in the output, less that in the tile
     uint32_t tile, gave_up;
 };
 
 // One pass: out = in stably sorted by its digit at `shift`; hist = the digit's counts, ticket and
 // state (256 words per tile) as for k_scan but state words of other passes are left over: they
 // carry their pass in bits 32..39 of the value.
-__global__ void __launch_bounds__(kSortThreads, 2) k_radix_pass(const uint64_t* __restrict__ in, uint64_t* __restrict__ out,
+__global__ void __launch_bounds__(kSortThreads, 3) k_radix_pass(const uint64_t* __restrict__ in, uint64_t* __restrict__ out,
                                                                 uint64_t n, int shift, const uint32_t* __restrict__ hist,
                                                                 uint32_t* ticket, unsigned long long* state, uint32_t pass) {
     extern __shared__ __align__(16) unsigned char raw[];
@@ -222,7 +224,7 @@ __global__ void __launch_bounds__(kSortThreads, 2) k_radix_pass(const uint64_t* 
         S.tile = atomicAdd(ticket, 1u);
         S.gave_up = 0u;
     }
-    for (int k = tid; k < kSortWarps * 256; k += kSortThreads) (&S.wh[0][0])[k] = 0u;
+    for (int k = tid; k < kSortWarps * 256; k += kSortThreads) reinterpret_cast<uint32_t*>(&S.wh[0][0])[k] = 0u;
     __syncthreads();
     const uint32_t tile = S.tile;
     const uint64_t base = (uint64_t)tile * kSortTile, wbase = base + (uint64_t)warp * (32 * kSortPer);
@@ -234,34 +236,33 @@ __global__ void __launch_bounds__(kSortThreads, 2) k_radix_pass(const uint64_t* 
         const uint64_t i = wbase + 32 * r + lane;
         key[r] = i < n ? in[i] : ~0ull;
     }
-    uint32_t rank[kSortPer / 2];   // 16 bits each: the key's place among its warp's keys of its digit
+    // the first and the second half of the warp's keys are ranked side by side, each against its own
+    // counts: two independent chains of ballots, a count read and a count written
+    uint32_t rank[kSortPer / 2];   // 16 bits each: the key's place among its half's keys of its digit
+    uint16_t *w0 = S.wh[2 * warp], *w1 = S.wh[2 * warp + 1];
 #pragma unroll
-    for (int r = 0; r < kSortPer; ++r) {
-        const uint32_t d = (uint32_t)(key[r] >> shift) & 255u;
-        uint32_t peers = 0xffffffffu;
+    for (int r = 0; r < kSortPer / 2; ++r) {
+        const uint32_t d0 = (uint32_t)(key[r] >> shift) & 255u, d1 = (uint32_t)(key[r + kSortPer / 2] >> shift) & 255u;
+        uint32_t p0 = 0xffffffffu, p1 = 0xffffffffu;
 #pragma unroll
         for (int b = 0; b < 8; ++b) {
-            const uint32_t bal = __ballot_sync(0xffffffffu, (d >> b) & 1u);
-            peers &= ((d >> b) & 1u) ? bal : ~bal;
+            const uint32_t b0 = __ballot_sync(0xffffffffu, (d0 >> b) & 1u), b1 = __ballot_sync(0xffffffffu, (d1 >> b) & 1u);
+            p0 &= ((d0 >> b) & 1u) ? b0 : ~b0;
+            p1 &= ((d1 >> b) & 1u) ? b1 : ~b1;
         }
-        const uint32_t before = S.wh[warp][d];
+        const uint32_t c0 = w0[d0], c1 = w1[d1];
         __syncwarp();
-        if ((peers & lt_mask) == 0u) S.wh[warp][d] = before + __popc(peers);
+        if ((p0 & lt_mask) == 0u) w0[d0] = (uint16_t)(c0 + __popc(p0));
+        if ((p1 & lt_mask) == 0u) w1[d1] = (uint16_t)(c1 + __popc(p1));
         __syncwarp();
-        const uint32_t k = before + __popc(peers & lt_mask);
-        if (r & 1) rank[r / 2] |= k << 16;
-        else rank[r / 2] = k;
+        rank[r] = (c0 + __popc(p0 & lt_mask)) | (c1 + __popc(p1 & lt_mask)) << 16;
     }
     __syncthreads();
     const unsigned long long mark = (unsigned long long)(pass + 1u) << 32;
     uint32_t count = 0, first = 0;
     if (tid < 256) {
 #pragma unroll
-        for (int w = 0; w < kSortWarps; ++w) {
-            const uint32_t c = S.wh[w][tid];
-            S.wh[w][tid] = count;
-            count += c;
-        }
+        for (int w = 0; w < 2 * kSortWarps; ++w) count += S.wh[w][tid];
     }
     const uint32_t all = count;
     if (tid == 255) count -= (uint32_t)kSortTile - tile_n;
@@ -269,31 +270,46 @@ __global__ void __launch_bounds__(kSortThreads, 2) k_radix_pass(const uint64_t* 
     uint32_t unused;
     const uint32_t start = block_excl_scan<uint32_t>(all, &unused);
     const uint32_t digit0 = block_excl_scan<uint32_t>(tid < 256 ? hist[tid] : 0u, &unused);
-    if (tid < 256) S.start[tid] = start;
+    if (tid < 256) {
+        uint32_t at = start;
+#pragma unroll
+        for (int w = 0; w < 2 * kSortWarps; ++w) {
+            const uint32_t c = S.wh[w][tid];
+            S.wh[w][tid] = (uint16_t)at;
+            at += c;
+        }
+    }
     __syncthreads();
 #pragma unroll
-    for (int r = 0; r < kSortPer; ++r) {
-        const uint32_t d = (uint32_t)(key[r] >> shift) & 255u;
-        S.keys[S.start[d] + S.wh[warp][d] + ((rank[r / 2] >> (16 * (r & 1))) & 0xffffu)] = key[r];
+    for (int r = 0; r < kSortPer / 2; ++r) {
+        S.keys[w0[(uint32_t)(key[r] >> shift) & 255u] + (rank[r] & 0xffffu)] = key[r];
+        S.keys[w1[(uint32_t)(key[r + kSortPer / 2] >> shift) & 255u] + (rank[r] >> 16)] = key[r + kSortPer / 2];
     }
     if (tid < 256) {
+        // kLook predecessors' words on their way at a time: many tiles run at once, so the nearest
+        // inclusive sum is often tens of tiles back
         bool waits = tile != 0u;
-        for (uint64_t t = tile; waits;) {
-            --t;
-            unsigned long long v;
-            uint32_t looks = 0;
-            while (((v = peek(&state[256ull * t + tid])) & (0xffull << 32)) != mark && ++looks < kPatience) {}
-            if (looks == kPatience) {
-                S.gave_up = 1u;
-                break;
+        for (int64_t t = (int64_t)tile - 1; waits; t -= kLook) {
+            unsigned long long v[kLook];
+#pragma unroll
+            for (int j = 0; j < kLook; ++j) v[j] = t >= j ? peek(&state[256ull * (uint64_t)(t - j) + tid]) : kUpTo | mark;
+#pragma unroll
+            for (int j = 0; j < kLook; ++j) {
+                if (!waits) continue;
+                uint32_t looks = 0;
+                while ((v[j] & (0xffull << 32)) != mark && ++looks < kPatience) v[j] = peek(&state[256ull * (uint64_t)(t - j) + tid]);
+                if (looks == kPatience) {
+                    S.gave_up = 1u;
+                    waits = false;
+                }
+                first += (uint32_t)v[j];
+                waits = waits && v[j] < kUpTo;   // tile 0's sum is inclusive
             }
-            first += (uint32_t)v;
-            waits = v < kUpTo;   // tile 0's sum is inclusive
         }
     }
     __syncthreads();
     if (S.gave_up) {   // uniform: count the predecessors' keys themselves
-        uint32_t* h = &S.wh[0][0];
+        __shared__ uint32_t h[256];
         if (tid < 256) h[tid] = 0u;
         __syncthreads();
         for (uint64_t i = tid; i < base; i += kSortThreads) atomicAdd(&h[(uint32_t)(in[i] >> shift) & 255u], 1u);
