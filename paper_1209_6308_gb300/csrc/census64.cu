@@ -265,8 +265,8 @@ tc_status tc_census64(tc_graph* g, void* stream, tc_u128 out[64]) {
         tc_options to;
         std::memset(&to, 0, sizeof(to));
         to.algo = TC_ALGO_TRIANGLE;
-        to.chunk_entries = 2048;
-        to.ctas_per_sm = 4;   // the caller-id hash doubles the shared memory of a CTA
+        to.chunk_entries = 1024;
+        to.ctas_per_sm = 5;   // the caller-id hash doubles the shared memory of a CTA
         Opts o;
         TC_TRY(resolve_opts(&to, nullptr, &o));
         Plan* p = nullptr;

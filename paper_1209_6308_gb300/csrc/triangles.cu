@@ -42,8 +42,10 @@ tc_status walk16_launch(const TriParams& P, const uint32_t split[2], uint32_t gr
 namespace {
 
 template <bool OLD, int MODE>
-// (1024 batched graphs at 8 / 6 / 5 resident CTAs: 4.67 / 4.53 / 4.66 ms; 8 spill 500 bytes.)
-__global__ void __launch_bounds__(kThreads, OLD ? 8 : 6) k_triangles(TriParams P) {
+// 1024 batched graphs at 8 / 6 / 5 resident CTAs: 4.67 / 4.53 / 4.66 ms (8 spill 500 bytes).  The
+// 64-state census of scale 20 with 4 CTAs and 2048-entry chunks / 5 and 1024 / 8 and 512: 5.94 / 5.49 /
+// 5.46 ms (at the 32 registers of 8 CTAs, 4 resident: 6.32).
+__global__ void __launch_bounds__(kThreads, OLD ? 5 : 6) k_triangles(TriParams P) {
     extern __shared__ __align__(16) unsigned char smem[];
     const uint32_t slots = 2u * P.chunk;
     uint32_t* sH = reinterpret_cast<uint32_t*>(smem);                 // [slots] CTA hash of L(b)

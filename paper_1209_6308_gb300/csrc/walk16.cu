@@ -34,7 +34,7 @@ namespace {
 constexpr int kT16 = 256;                       // threads of a CTA = pairs of a batch
 constexpr int kW16 = kT16 / 32;
 constexpr int kCtas16 = 4;                      // resident CTAs per SM (shared memory, 64 registers)
-constexpr int kCtasWarp = 6;                    // of k_walk_warp
+constexpr int kCtasWarp = 8;                    // of k_walk_warp (scale 20 / 24 / 26 at 6: 1.623 / 48.6 / 279.2 ms, at 8: 1.636 / 48.0 / 277.8)
 // rounds of a warp in flight (scale 26, k_walk16 at 2 / 3 / 4: 282 / 279 / 330 ms, 4 spills)
 constexpr int kRing = 3, kRingTable = 2;
 constexpr uint32_t kWindow = 8192;              // blocks of the flattened range per window
