@@ -93,65 +93,81 @@ __global__ void __launch_bounds__(256) k_keys64(GraphDev g, uint32_t n_wide, con
 //   raw[18..27) X:  (neighbours below c of class d1) x (above c of class d2)  (c is y)
 //   raw[27..36) R:  per pair (a, b), a < b, of direction class k = d1 (1 a->b, 2 b->a, 3 both):
 //               position d2 = 1 above b (n - 1 - b), 2 between (b - a - 1), 3 below a (a)
-// Classes are seen from c (1 c->nbr, 2 nbr->c).  A warp over 32 vertices (caller ids, rows.cuh):
-// per entry, the earlier entries of its row by side and class.
+// Classes are seen from c (1 c->nbr, 2 nbr->c).
+struct Wedges {
+    unsigned long long pb[3][3] = {}, pa[3][3] = {}, xx[3][3] = {}, rr[3][3] = {};
+
+    // One block of entries: this lane's key of centre c (n vertices, ids of B bits), its row's lanes, and
+    // the counts of the row's earlier blocks by side and class, which it advances.
+    __device__ __forceinline__ void block(bool valid, uint64_t key, uint32_t c, uint32_t n, int B, uint32_t lanes,
+                                          uint32_t (&rb)[3], uint32_t (&ra)[3]) {
+        const uint32_t lt = (1u << (threadIdx.x & 31u)) - 1u;
+        const uint32_t nb = (uint32_t)((key >> 2) & ((1ull << B) - 1ull)), d = (uint32_t)(key & 3ull);
+        const bool below = valid && nb < c, above = valid && nb > c;
+#pragma unroll
+        for (int q1 = 0; q1 < 3; ++q1) {
+            const uint32_t bb = __ballot_sync(0xffffffffu, below && d == (uint32_t)(q1 + 1)) & lanes;
+            const uint32_t ba = __ballot_sync(0xffffffffu, above && d == (uint32_t)(q1 + 1)) & lanes;
+            const uint32_t before_b = rb[q1] + __popc(bb & lt), before_a = ra[q1] + __popc(ba & lt);
+#pragma unroll
+            for (int q2 = 0; q2 < 3; ++q2) {
+                if (below && d == (uint32_t)(q2 + 1)) pb[q1][q2] += before_b;
+                if (above && d == (uint32_t)(q2 + 1)) pa[q1][q2] += before_a;
+            }
+            rb[q1] += __popc(bb);
+            ra[q1] += __popc(ba);
+        }
+        if (above) {
+            const unsigned long long vals[3] = {(unsigned long long)n - 1ull - nb, (unsigned long long)(nb - c - 1u),
+                                                (unsigned long long)c};
+#pragma unroll
+            for (int q1 = 0; q1 < 3; ++q1)
+                if (d == (uint32_t)(q1 + 1))
+#pragma unroll
+                    for (int q2 = 0; q2 < 3; ++q2) rr[q1][q2] += vals[q2];
+        }
+    }
+    // A row's counts below and above its centre (one lane per row).
+    __device__ __forceinline__ void products(const uint32_t (&rb)[3], const uint32_t (&ra)[3]) {
+#pragma unroll
+        for (int q1 = 0; q1 < 3; ++q1)
+#pragma unroll
+            for (int q2 = 0; q2 < 3; ++q2) xx[q1][q2] += (unsigned long long)rb[q1] * ra[q2];
+    }
+    __device__ __forceinline__ void flush(unsigned long long* raw) const {
+#pragma unroll
+        for (int q1 = 0; q1 < 3; ++q1)
+#pragma unroll
+            for (int q2 = 0; q2 < 3; ++q2) {
+                const unsigned long long v[4] = {pb[q1][q2], pa[q1][q2], xx[q1][q2], rr[q1][q2]};
+#pragma unroll
+                for (int t = 0; t < 4; ++t) {
+                    unsigned long long s = v[t];
+                    for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+                    if ((threadIdx.x & 31u) == 0 && s) atomicAdd(&raw[9 * t + 3 * q1 + q2], s);
+                }
+            }
+    }
+};
+
+// Rows of at most kHubDeg entries: a warp over 32 vertices (caller ids, rows.cuh).
 __global__ void __launch_bounds__(256) k_wedges64(const uint64_t* __restrict__ keys, const uint64_t* __restrict__ off_old,
                                                   uint32_t n, int B, unsigned long long* raw) {
     __shared__ uint8_t s_at[8][32];
     const uint32_t lane = threadIdx.x & 31;
-    const uint64_t idmask = (1ull << B) - 1ull;
-    const uint32_t lt = (1u << lane) - 1u;
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-    unsigned long long pb[3][3], pa[3][3], xx[3][3], rr[3][3];
-#pragma unroll
-    for (int i = 0; i < 3; ++i)
-#pragma unroll
-        for (int j = 0; j < 3; ++j) pb[i][j] = pa[i][j] = xx[i][j] = rr[i][j] = 0ull;
+    Wedges W;
     for (uint64_t x0 = blockIdx.x * (uint64_t)blockDim.x + (threadIdx.x & ~31u); x0 < n; x0 += stride) {
         const bool ok = x0 + lane < n;
         const uint64_t vb = ok ? off_old[x0 + lane] : 0ull;
         const uint32_t vd = ok ? (uint32_t)(off_old[x0 + lane + 1] - vb) : 0u;
-        // one block of entries: this lane's key of centre c, its row's lanes, and the counts of the row's
-        // earlier blocks, which it advances
-        auto block = [&](bool valid, uint64_t key, uint32_t c, uint32_t lanes, uint32_t (&rb)[3], uint32_t (&ra)[3]) {
-            const uint32_t nb = (uint32_t)((key >> 2) & idmask), d = (uint32_t)(key & 3ull);
-            const bool below = valid && nb < c, above = valid && nb > c;
-#pragma unroll
-            for (int q1 = 0; q1 < 3; ++q1) {
-                const uint32_t bb = __ballot_sync(0xffffffffu, below && d == (uint32_t)(q1 + 1)) & lanes;
-                const uint32_t ba = __ballot_sync(0xffffffffu, above && d == (uint32_t)(q1 + 1)) & lanes;
-                const uint32_t before_b = rb[q1] + __popc(bb & lt), before_a = ra[q1] + __popc(ba & lt);
-#pragma unroll
-                for (int q2 = 0; q2 < 3; ++q2) {
-                    if (below && d == (uint32_t)(q2 + 1)) pb[q1][q2] += before_b;
-                    if (above && d == (uint32_t)(q2 + 1)) pa[q1][q2] += before_a;
-                }
-                rb[q1] += __popc(bb);
-                ra[q1] += __popc(ba);
-            }
-            if (above) {
-                const unsigned long long vals[3] = {(unsigned long long)n - 1ull - nb, (unsigned long long)(nb - c - 1u),
-                                                    (unsigned long long)c};
-#pragma unroll
-                for (int q1 = 0; q1 < 3; ++q1)
-                    if (d == (uint32_t)(q1 + 1))
-#pragma unroll
-                        for (int q2 = 0; q2 < 3; ++q2) rr[q1][q2] += vals[q2];
-            }
-        };
-        auto products = [&](const uint32_t (&rb)[3], const uint32_t (&ra)[3]) {
-#pragma unroll
-            for (int q1 = 0; q1 < 3; ++q1)
-#pragma unroll
-                for (int q2 = 0; q2 < 3; ++q2) xx[q1][q2] += (unsigned long long)rb[q1] * ra[q2];
-        };
-        for_rows(vd, s_at[threadIdx.x >> 5],
+        for_rows(vd > kHubDeg ? 0u : vd, s_at[threadIdx.x >> 5],
             [&](const PackedEntry& p) {
                 const uint64_t b = __shfl_sync(0xffffffffu, vb, p.row);
                 uint32_t rb[3] = {0u, 0u, 0u}, ra[3] = {0u, 0u, 0u};
                 const uint64_t key = p.valid ? keys[b + (lane - p.first)] : 0ull;
-                block(p.valid, key, (uint32_t)x0 + p.row, p.lanes, rb, ra);
-                if (p.valid && lane == p.first) products(rb, ra);   // the row's totals
+                W.block(p.valid, key, (uint32_t)x0 + p.row, n, B, p.lanes, rb, ra);
+                if (p.valid && lane == p.first) W.products(rb, ra);   // the row's totals
             },
             [&](uint32_t row) {
                 const uint64_t b = __shfl_sync(0xffffffffu, vb, row);
@@ -162,23 +178,61 @@ __global__ void __launch_bounds__(256) k_wedges64(const uint64_t* __restrict__ k
                     const uint64_t key = next;
                     const uint32_t k = k0 + lane;
                     next = k + 32u < d ? keys[b + k + 32u] : 0ull;
-                    block(k < d, key, (uint32_t)x0 + row, 0xffffffffu, rb, ra);
+                    W.block(k < d, key, (uint32_t)x0 + row, n, B, 0xffffffffu, rb, ra);
                 }
-                if (lane == 0) products(rb, ra);
+                if (lane == 0) W.products(rb, ra);
             });
     }
+    W.flush(raw);
+}
+
+// The longer rows, those of the first n_hub stored vertices: a CTA each, its warps over segments of the
+// row from the counts of the segments before.  (One warp per row made the largest hub's 65 k entries
+// the kernel's length: scale 20 1.16 ms.)
+__global__ void __launch_bounds__(256) k_wedges64_hub(const uint64_t* __restrict__ keys, const uint64_t* __restrict__ off_old,
+                                                      const uint32_t* __restrict__ old, uint32_t n_hub, uint32_t n, int B,
+                                                      unsigned long long* raw) {
+    __shared__ uint32_t s_cnt[8][6];
+    const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint64_t idmask = (1ull << B) - 1ull;
+    Wedges W;
+    for (uint32_t r = blockIdx.x; r < n_hub; r += gridDim.x) {
+        const uint32_t c = old[r];
+        const uint64_t b = off_old[c];
+        const uint32_t d = (uint32_t)(off_old[c + 1] - b), seg = ((d + 7u) / 8u + 31u) & ~31u;
+        const uint32_t s0 = min(d, warp * seg), s1 = min(d, s0 + seg);
+        uint32_t cnt[6] = {0u, 0u, 0u, 0u, 0u, 0u};   // below by class, above by class
+#pragma unroll 4
+        for (uint32_t k = s0 + lane; k < s1; k += 32) {
+            const uint64_t key = keys[b + k];
+            const uint32_t q = (uint32_t)(key & 3ull) + ((uint32_t)((key >> 2) & idmask) < c ? 0u : 3u);
 #pragma unroll
-    for (int q1 = 0; q1 < 3; ++q1)
-#pragma unroll
-        for (int q2 = 0; q2 < 3; ++q2) {
-            unsigned long long v[4] = {pb[q1][q2], pa[q1][q2], xx[q1][q2], rr[q1][q2]};
-#pragma unroll
-            for (int t = 0; t < 4; ++t) {
-                unsigned long long s = v[t];
-                for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-                if (lane == 0 && s) atomicAdd(&raw[9 * t + 3 * q1 + q2], s);
-            }
+            for (uint32_t i = 0; i < 6; ++i) cnt[i] += q == i + 1u;
         }
+#pragma unroll
+        for (uint32_t i = 0; i < 6; ++i) {
+            cnt[i] = __reduce_add_sync(0xffffffffu, cnt[i]);
+            if (lane == 0) s_cnt[warp][i] = cnt[i];
+        }
+        __syncthreads();
+        uint32_t rb[3] = {0u, 0u, 0u}, ra[3] = {0u, 0u, 0u};
+        for (uint32_t w = 0; w < warp; ++w)
+#pragma unroll
+            for (uint32_t i = 0; i < 3; ++i) {
+                rb[i] += s_cnt[w][i];
+                ra[i] += s_cnt[w][3 + i];
+            }
+        uint64_t next = s0 + lane < s1 ? keys[b + s0 + lane] : 0ull;
+        for (uint32_t k0 = s0; k0 < s1; k0 += 32) {
+            const uint64_t key = next;
+            const uint32_t k = k0 + lane;
+            next = k + 32u < s1 ? keys[b + k + 32u] : 0ull;
+            W.block(k < s1, key, c, n, B, 0xffffffffu, rb, ra);
+        }
+        if (warp == 7u && lane == 0) W.products(rb, ra);   // the last segment ends with the row's totals
+        __syncthreads();   // the counts are read before the next row writes its own
+    }
+    W.flush(raw);
 }
 
 // states of wedges and one-link triads (see the file comment); d = direction class seen
@@ -261,6 +315,11 @@ tc_status tc_census64(tc_graph* g, void* stream, tc_u128 out[64]) {
         k_wedges64<<<grid_for(G.n, 256, 4u * (unsigned)sm_count()), 256, 0, st>>>(
             kp, offo.as<uint64_t>(), G.n, B, d_raw);
         TC_LAUNCH("k_wedges64");
+        if (G.n_hub) {
+            k_wedges64_hub<<<grid_for(256ull * G.n_hub, 256, 2u * (unsigned)sm_count()), 256, 0, st>>>(
+                kp, offo.as<uint64_t>(), old.as<uint32_t>(), G.n_hub, G.n, B, d_raw);
+            TC_LAUNCH("k_wedges64_hub");
+        }
         // triangles, in caller-id states, through the triangle form's plan
         tc_options to;
         std::memset(&to, 0, sizeof(to));
