@@ -269,7 +269,7 @@ def census_code_hash(text: str) -> str:
     return hashlib.sha256(code.encode()).hexdigest()[:16]
 
 
-KERNEL_SRC = {"k_census": "census.cu", "k_triangles": "triangles.cu"}
+KERNEL_SRC = {"k_census": "census.cu", "k_triangles": "triangles.cu", "k_walk16": "walk16.cu"}
 
 
 def traffic_file(workload_name: str, kernel: str = "k_census") -> str:
@@ -638,10 +638,8 @@ def matrix_comparison(tc, torch, sh, steps=3):
             times.append(e0.elapsed_time(e1))
         tri_ms, _ = learned.census_ms(g, {"algo": tc.TC_ALGO_TRIANGLE}, torch.cuda.Stream(), reps=5)
     ms = statistics.median(times)
-    W = (n + 63) // 64
-    words = 6 * n * n * W       # AND + popcount word operations of the six products
     return {"workload": "rmat14_ef16_r20_seed14", "n": n, "arcs": len(s), "ms": ms, "equals_census16": cm == c16,
-            "triangle_form_ms": tri_ms, "and_popc_words_per_s": words / (ms * 1e-3)}
+            "triangle_form_ms": tri_ms}
 
 
 def roofline_hbm(bytes_alg: int, ms: float, kernel: str, traffic=None, bound="hbm") -> dict:
@@ -654,6 +652,25 @@ def roofline_hbm(bytes_alg: int, ms: float, kernel: str, traffic=None, bound="hb
 FORM_NAMES = {0: "union", 1: "suffix", 2: "triangle"}
 
 
+def triangle_kernel(info) -> str:
+    """The triangle form's walk: the launches of walk16.cu from 2^25 walked entries and 12 per pair on."""
+    return "k_walk16" if info["sum_tri_walk"] >= max(1 << 25, 12 * info["e_sym"]) else "k_triangles"
+
+
+def census_launches(tc, g, n, info, algo) -> int:
+    """Kernels of one census: k_census, or k_pair_bulk, the walk and k_tri_fold; the 16-bit walk is
+    k_walk16, k_walk_table (only if vertices past id 2^17 have more than 256 neighbours) and k_walk_warp."""
+    if algo != tc.TC_ALGO_TRIANGLE:
+        return 1
+    if triangle_kernel(info) == "k_triangles":
+        return 3
+    import numpy as np
+    off = np.zeros(n + 1, np.uint64)
+    tc.load().tc_graph_export_csr(g, off.ctypes.data, None, None)
+    table = n > (1 << 17) and int(off[(1 << 17) + 1] - off[1 << 17]) > 256
+    return 4 + table
+
+
 def form_roofline(tc, n, info, algo, ms):
     """Roofline of one census.  `bytes_alg_per_launch` is what the kernel form itself must read
     (tc_graph_info: the triangle form's or the suffix form's count; the scope contract's count
@@ -661,7 +678,7 @@ def form_roofline(tc, n, info, algo, ms):
     streaming its own data at copy speed.  The scope contract's count (every pair streams its
     v list, the paper's walk) is given beside it as `contract_*`: a form that skips most of
     that reading can exceed 1 there."""
-    kernel = {tc.TC_ALGO_TRIANGLE: "k_triangles", tc.TC_ALGO_SUFFIX: "k_census (suffix)"}.get(algo, "k_census (union)")
+    kernel = {tc.TC_ALGO_TRIANGLE: triangle_kernel(info), tc.TC_ALGO_SUFFIX: "k_census (suffix)"}.get(algo, "k_census (union)")
     b8d = bytes_alg_8d(n, info)
     own = {tc.TC_ALGO_TRIANGLE: info["bytes_alg_tri"], tc.TC_ALGO_SUFFIX: info["bytes_alg"]}.get(algo, b8d)
     r = roofline_hbm(own, ms, kernel, None, "issue")
@@ -680,11 +697,11 @@ def medium_section(tc, torch, stream, steps=5):
     from paper_1209_6308_gb300 import learned
     out = {"workload": WORKLOADS[20]["name"], "n": n, "arcs": len(s)}
     counts = {}
-    with tc.Graph.from_arcs(n, s, d, stream=sh) as g:        # created without options: the union walk by default
+    with tc.Graph.from_arcs(n, s, d, stream=sh) as g:
         info = g.stats()
         out["e_sym"] = info["e_sym"]
         for algo in (tc.TC_ALGO_TRIANGLE, tc.TC_ALGO_SUFFIX, tc.TC_ALGO_UNION):
-            ms, c = learned.census_ms(g, {"algo": algo} if algo else None, stream, reps=steps if algo else 3)
+            ms, c = learned.census_ms(g, {"algo": algo}, stream, reps=steps if algo else 3)
             counts[algo] = c
             out[FORM_NAMES[algo]] = {"ms": ms, "arcs_per_s": len(s) / (ms * 1e-3),
                                      "roofline": form_roofline(tc, n, info, algo, ms)}
@@ -721,6 +738,7 @@ def run_gpu(args):
     g = tc.Graph.from_arcs(n, s, d, stream=sh, options=opts)
     build_s = time.perf_counter() - t0
     info = g.stats()
+    launches = census_launches(tc, g.handle, n, info, algo)
     log(f"graph built in {build_s:.1f}s: e_sym={info['e_sym']} sum_walk={info['sum_walk']}")
     out = torch.zeros(16, dtype=torch.int64, device="cuda")
     flush = torch.empty(512 << 20, dtype=torch.uint8, device="cuda")
@@ -850,15 +868,15 @@ def run_gpu(args):
     if model is not None:
         tc.tc_costmodel_destroy(model)
 
-    kernel = "k_triangles" if algo == tc.TC_ALGO_TRIANGLE else "k_census"
+    kernel = triangle_kernel(info) if algo == tc.TC_ALGO_TRIANGLE else "k_census"
     traffic = stored_traffic(WORKLOAD["name"], kernel)
     roof = form_roofline(tc, n, info, algo, ms)
     roof["traffic"] = traffic
     roof["note"] = ("bytes_alg_per_launch = what this kernel form reads (tc_graph_info bytes_alg_tri: "
                     "32(n+1) + 60 E + 4 sum_tri_walk + 1280); contract_* = the scope formula 8(n+1) + 8 E + "
                     "sum over upper pairs (4 d_v + 16) + 128 (each pair streams N[v], the paper's walk), which "
-                    "this form does not read; the kernel is bound by load latency and instruction issue (ncu), "
-                    "not by HBM bandwidth")
+                    "this form does not read; the walk of 16-bit lists reads half of the 4 B per walked entry; it is "
+                    "bound by shared-memory lookups (bank conflicts) and instruction issue (ncu)")
     line = {
         "metric": METRIC, "value": job_value(arcs, ms),
         "unit": "arcs/s", "n_gpus": world, "steps": args.steps, "warmup": args.warmup, "ms_per_step": ms,
@@ -875,8 +893,7 @@ def run_gpu(args):
                  "build_ms": statistics.mean(e2e_build_ms) if e2e_build_ms else None,
                  "path": "tc_graph_create_arcs from page-locked host arcs (read by the build's key kernel over "
                          "the host link), tc_census (plan + census), 16 counts to the host"} if e2e_ms else None),
-        # per census: k_pair_bulk, k_triangles, k_tri_fold (triangle form) or k_census
-        "gpu_launches": args.steps * (3 if algo == tc.TC_ALGO_TRIANGLE else 1),
+        "gpu_launches": args.steps * launches,
         "clocks": clk.summary(),
         "census": counts,
         "census_e2e_equal": (e2e_counts == counts) if e2e_counts else None,

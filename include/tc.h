@@ -156,7 +156,8 @@ tc_status tc_census_async(tc_graph* g, void* stream, const tc_options* opt, uint
  * by the relabelled id of tc_graph_device_csr; the caller zeroes it).  d_phase (device uint64,
  * may be NULL) receives, for each of the tc_census_grid() CTAs, the global timer in ns at
  * its start, at the end of its CTA work items and at its end (in the TC_ALGO_TRIANGLE form,
- * those of the triangle walk's launch).  Does not synchronise. */
+ * those of the triangle walk; where that takes launches of fewer CTAs, a CTA's times fill the
+ * entries of several).  Does not synchronise. */
 tc_status tc_census_profile(tc_graph* g, void* stream, const tc_options* opt, uint64_t* d_out16,
                             uint64_t* d_vcost, uint64_t* d_phase);
 
@@ -202,10 +203,12 @@ tc_status tc_census64(tc_graph* g, void* stream, tc_u128 out[64]);
  * count is a sum of an elementwise product of one of them with one of the products NN, S'S, SS',
  * SS, NM, MM, divided by the class's symmetries (003 = sum(N o NN)/6, 012 = sum(S o NN), ...,
  * 300 = sum(M o MM)/6).  All 16 counts come from their own sums (the null count too).  The
- * matrices are bit-packed and each product's masked sums are fused into its tiles: O(n^3 / 64)
- * work, a dense cross-check of the Fig. 5 kernels for graphs of n <= 2^14 vertices (larger n:
- * TC_ERR_RANGE).  out: 16 host tc_u128.  Synchronises the stream.  TC_ERR_BUSY if the graph is
- * in use by another call, TC_ERR_OOM, TC_ERR_CUDA. */
+ * matrices are bit-packed.  A sparse graph's sums are taken at the connected pairs, O(e n / 64),
+ * but for 003, one triangular product on the tensor cores; a dense graph's six products all run
+ * there (0/1 in FP8, accumulated in FP32, exact for these sizes).  A cross-check of the Fig. 5
+ * kernels for graphs of n <= 2^14 vertices (larger n: TC_ERR_RANGE).  out: 16 host tc_u128.
+ * Synchronises the stream.  TC_ERR_BUSY if the graph is in use by another call, TC_ERR_OOM,
+ * TC_ERR_CUDA, TC_ERR_TIMEOUT if a wait inside the product kernel ran into its limit. */
 tc_status tc_census_matrix(tc_graph* g, void* stream, tc_u128 out[16]);
 
 /* Census of k graphs in one persistent launch (builds a tc_batch, runs it once, frees it).
