@@ -41,6 +41,14 @@ tc_status walk16_launch(const TriParams& P, const uint32_t split[2], uint32_t gr
 
 namespace {
 
+// A warp's copy of its graph's record.  No lane still reads the last one.
+__device__ __forceinline__ void load_graph(GraphDev& to, const GraphDev* from, int lane) {
+    static_assert(sizeof(GraphDev) % 8 == 0 && sizeof(GraphDev) <= 256, "a lane per word");
+    __syncwarp();
+    if (lane < (int)(sizeof(GraphDev) / 8)) reinterpret_cast<uint64_t*>(&to)[lane] = reinterpret_cast<const uint64_t*>(from)[lane];
+    __syncwarp();
+}
+
 template <bool OLD, int MODE>
 // 1024 batched graphs at 8 / 6 / 5 resident CTAs: 4.67 / 4.53 / 4.66 ms (8 spill 500 bytes).  The
 // 64-state census of scale 20 with 4 CTAs and 2048-entry chunks / 5 and 1024 / 8 and 512: 5.94 / 5.49 /
@@ -56,6 +64,7 @@ __global__ void __launch_bounds__(kThreads, OLD ? 5 : 6) k_triangles(TriParams P
     uint8_t* sPerm = reinterpret_cast<uint8_t*>(sHist + kWarps * 64);  // [9][64] OLD
     __shared__ uint32_t s_item, s_next;
     __shared__ uint8_t s_at[kWarps][32];   // walk_pairs' scratch
+    __shared__ GraphDev s_g[MODE == kTriSingle ? 1 : kWarps];
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     // the whole-warp walk of long prefixes, except in a batch of graphs (small graphs, short
@@ -68,20 +77,15 @@ __global__ void __launch_bounds__(kThreads, OLD ? 5 : 6) k_triangles(TriParams P
         for (int k = tid; k < 9 * 64; k += kThreads) sPerm[k] = P.perm_state[k];
     __syncthreads();
     uint32_t* myHist = sHist + warp * 64;
-    GraphDev G = P.g;
+    const GraphDev& G = MODE == kTriSingle ? P.g : s_g[warp];   // several graphs: the warp's
     unsigned long long* ghist = P.hist;
     uint32_t cur_graph = 0xffffffffu;   // batched: the graph whose counts the warp's bins hold
     // batched: move to graph gi, flushing this warp's bins to the graph they belong to
     auto use_graph = [&](uint32_t gi) {
         if (cur_graph != 0xffffffffu) flush_warp_hist(myHist, ghist, lane);
         cur_graph = gi;
-        if (MODE == kTriWave) {
-            G = P.reqs[gi].g;
-            ghist = P.reqs[gi].out + 32;
-        } else {
-            G = P.graphs[gi];
-            ghist = P.hist + (uint64_t)kBatchStride * gi;
-        }
+        load_graph(s_g[warp], MODE == kTriWave ? &P.reqs[gi].g : &P.graphs[gi], lane);
+        ghist = MODE == kTriWave ? P.reqs[gi].out + 32 : P.hist + (uint64_t)kBatchStride * gi;
     };
     uint32_t since_flush = 0;   // warp-uniform: entries walked since this warp's bins were flushed
     // the hash region (2 x chunk words) holds a direct map of 32 x chunk ids at two bits each
@@ -240,21 +244,32 @@ __global__ void __launch_bounds__(kThreads, OLD ? 5 : 6) k_triangles(TriParams P
 
 // One pair's bulk sums into acc (see k_pair_bulk): u of degree du, the pair's entry e = N[u][j]
 // and its table index p.
-__device__ __forceinline__ void bulk_pair(const GraphDev& g, unsigned long long n, uint32_t du, uint32_t j, uint32_t e,
-                                          uint64_t p, unsigned long long (&acc)[3][7]) {
+__device__ __forceinline__ void bulk_pair(const GraphDev& g, uint32_t du, uint32_t j, uint32_t e, uint64_t p, int (&acc)[21]) {
     const uint32_t v = e >> 2, duv = e & 3u;
     const uint32_t cuv = ((duv & 1u) << 1) | (duv >> 1);
     const uint2 vs = g.vs[p], us = g.us[p];
     const uint32_t rpv = g.rp[p];
     const uint32_t dv = (uint32_t)(g.off[v + 1] - g.off[v]);
     const uint32_t vlen = dv - 1u - rpv, ulen = du - 1u - j;
-    const unsigned long long val[7] = {vs.x, vs.y, (unsigned long long)(vlen - vs.x - vs.y),
-                                       us.x, us.y, (unsigned long long)(ulen - us.x - us.y), n - du - dv};
+    const uint32_t val[7] = {vs.x, vs.y, vlen - vs.x - vs.y, us.x, us.y, ulen - us.x - us.y, g.n - du - dv};
 #pragma unroll
     for (int c = 0; c < 3; ++c)
         if (cuv == (uint32_t)(c + 1))
 #pragma unroll
-            for (int k = 0; k < 7; ++k) acc[c][k] += val[k];
+            for (int k = 0; k < 7; ++k) acc[7 * c + k] += (int)val[k];
+}
+
+// The warp's sum of acc[k] in lane k < 21 (0 in the others); acc is left zero.  Low and high halves
+// are reduced apart, so 32 lanes cannot overflow.
+__device__ __forceinline__ long long bulk_reduce(int (&acc)[21], int lane) {
+    long long mine = 0;
+#pragma unroll
+    for (int k = 0; k < 21; ++k) {
+        const int lo = __reduce_add_sync(0xffffffffu, acc[k] & 0xffff), hi = __reduce_add_sync(0xffffffffu, acc[k] >> 16);
+        if (lane == k) mine = lo + hi * 65536ll;
+        acc[k] = 0;
+    }
+    return mine;
 }
 
 // Bulk counts of the census's pairs: per dir(u,v) code c (tricode bits 1|2, 1..3),
@@ -282,41 +297,53 @@ struct BulkParams {
     unsigned long long* raw;
 };
 
-__device__ __forceinline__ void flush_bulk(unsigned long long (&acc)[3][7], unsigned long long* raw, uint32_t lane) {
-#pragma unroll
-    for (int c = 0; c < 3; ++c)
-#pragma unroll
-        for (int k = 0; k < 7; ++k) {
-            unsigned long long s = acc[c][k];
-            for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-            if (lane == 0 && s) atomicAdd(&raw[7 * c + k], s);
-            acc[c][k] = 0ull;
-        }
+// Blocks of one-warp vertices a warp takes per grab of a serving wave: the blocks follow the
+// requests, so a warp that takes single ones meets another request, hence a reduction of its sums, at
+// nearly every block (256 requests to 16 graphs: 3.53 -> 3.39 ms).  A batch of small graphs takes
+// single blocks all the same (1024 graphs: 3.82 ms, in runs 4.08): all warps are then in the same few
+// graphs, whose offsets and lists stay in the caches.
+__device__ __forceinline__ uint32_t block_run(uint32_t blocks, uint32_t warps) {
+    return min(16u, max(1u, blocks / (4u * warps)));
 }
 
 template <int MODE>
 __global__ void __launch_bounds__(256, 4) k_pair_bulk(BulkParams P) {
     __shared__ uint8_t s_at[kWarps][32];
+    __shared__ GraphDev s_g[MODE == kTriSingle ? 1 : kWarps];
     const uint32_t lane = threadIdx.x & 31;
     const uint32_t le_mask = (2u << lane) - 1u;
-    unsigned long long acc[3][7];
+    int acc[21];
 #pragma unroll
-    for (int c = 0; c < 3; ++c)
-#pragma unroll
-        for (int k = 0; k < 7; ++k) acc[c][k] = 0ull;
-    GraphDev G = P.g;
+    for (int k = 0; k < 21; ++k) acc[k] = 0;
+    // A pair's values are at most n in size, so a lane's 32-bit sums hold `limit` rounds; then (and
+    // at the end of a graph) the warp's go to 64 bits, the k-th sum in lane k.  64-bit sums in every
+    // lane took 42 of the 64 registers, and with the graph's record per lane a tenth of the
+    // instructions were spills (1024 batched graphs 4.50 -> 3.82 ms, 256 served requests 4.11 -> 3.39
+    // ms, a census of scale 20 1.627 -> 1.602 ms; at five CTAs per SM, spilling again, slower).
+    long long sum = 0;
+    uint32_t rounds = 0, limit = MODE == kTriSingle ? 0x7fffffffu / P.g.n : 0u;
+    auto round_done = [&] {
+        if (++rounds < limit) return;
+        sum += bulk_reduce(acc, lane);
+        rounds = 0;
+    };
+    // several graphs: the warp's graph lies in shared memory (as a copy of each lane it was in local
+    // memory, and its pointers' reloads missed L1)
+    const GraphDev& G = MODE == kTriSingle ? P.g : s_g[threadIdx.x >> 5];
     unsigned long long* raw = P.raw;
     uint32_t cur_graph = 0xffffffffu;
+    auto flush = [&] {
+        sum += bulk_reduce(acc, lane);
+        if (sum) atomicAdd(&raw[lane], (unsigned long long)sum);
+        sum = 0;
+        rounds = 0;
+    };
     auto use_graph = [&](uint32_t gi) {
-        if (cur_graph != 0xffffffffu) flush_bulk(acc, raw, lane);
+        if (cur_graph != 0xffffffffu) flush();
         cur_graph = gi;
-        if (MODE == kTriWave) {
-            G = P.reqs[gi].g;
-            raw = P.reqs[gi].out;
-        } else {
-            G = P.graphs[gi];
-            raw = P.raw + (uint64_t)kBatchStride * gi;
-        }
+        load_graph(s_g[threadIdx.x >> 5], MODE == kTriWave ? &P.reqs[gi].g : &P.graphs[gi], lane);
+        raw = MODE == kTriWave ? P.reqs[gi].out : P.raw + (uint64_t)kBatchStride * gi;
+        limit = 0x7fffffffu / G.n;
     };
     // the CTA items, a warp each
     for (;;) {
@@ -333,17 +360,23 @@ __global__ void __launch_bounds__(256, 4) k_pair_bulk(BulkParams P) {
             w = P.items[it];
             if (MODE == kTriBatch && w.pad != cur_graph) use_graph(w.pad);
         }
-        const unsigned long long n = G.n;
         const uint64_t ubase = G.off[w.u];
         const uint32_t du = (uint32_t)(G.off[w.u + 1] - ubase);
         const uint64_t pb = G.ub[w.u] - G.up[w.u];
-        for (uint32_t j = w.j0 + lane; j < w.j1; j += 32) bulk_pair(G, n, du, j, G.adj[ubase + j], pb + j, acc);
+        for (uint32_t j0 = w.j0; j0 < w.j1; j0 += 32) {
+            const uint32_t j = j0 + lane;
+            if (j < w.j1) bulk_pair(G, du, j, G.adj[ubase + j], pb + j, acc);
+            round_done();
+        }
     }
-    // the one-warp vertices, 32 consecutive ones per grab
-    for (;;) {
-        uint32_t blk = 0;
-        if (lane == 0) blk = atomicAdd(&P.ctr[3], 1u);
-        blk = __shfl_sync(0xffffffffu, blk, 0);
+    // the one-warp vertices, blocks of 32 consecutive ones
+    const uint32_t run = MODE != kTriWave ? 1u : block_run(P.n_wblocks, gridDim.x * kWarps);
+    for (uint32_t blk = 0, last = 0;; ++blk) {
+        if (blk == last) {
+            if (lane == 0) blk = atomicAdd(&P.ctr[3], run);
+            blk = __shfl_sync(0xffffffffu, blk, 0);
+            last = blk + run;
+        }
         uint64_t base, end;
         if (MODE == kTriWave) {
             if (blk >= P.n_wblocks) break;
@@ -363,7 +396,6 @@ __global__ void __launch_bounds__(256, 4) k_pair_bulk(BulkParams P) {
             if (base >= P.we) break;
             end = base + 32u < P.we ? base + 32u : P.we;
         }
-        const unsigned long long n = G.n;
         const uint64_t u = base + lane;
         const bool ok = u < end;
         uint64_t ubase = ok ? G.off[u] : 0ull;
@@ -400,32 +432,27 @@ __global__ void __launch_bounds__(256, 4) k_pair_bulk(BulkParams P) {
             const uint64_t sB = __shfl_sync(0xffffffffu, ubase, sg);
             const uint32_t sD = __shfl_sync(0xffffffffu, du, sg), sU = __shfl_sync(0xffffffffu, upu, sg);
             const uint32_t i = r0 + lane;
-            if (i >= total) continue;
-            const uint32_t j = sU + (i - sP);         // the pair's position in N[u]
-            bulk_pair(G, n, sD, j, G.adj[sB + j], pstart + i, acc);
+            if (i < total) {
+                const uint32_t j = sU + (i - sP);         // the pair's position in N[u]
+                bulk_pair(G, sD, j, G.adj[sB + j], pstart + i, acc);
+            }
+            round_done();
         }
     }
     if (MODE == kTriSingle) {
         // one graph: the warps' sums meet in shared memory, so a CTA adds 21 counters once (a small
         // census waited for its warps' atomics on them)
-        __shared__ unsigned long long s_sum[kWarps][21];
-#pragma unroll
-        for (int c = 0; c < 3; ++c)
-#pragma unroll
-            for (int k = 0; k < 7; ++k) {
-                unsigned long long s = acc[c][k];
-                for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-                if (lane == 0) s_sum[threadIdx.x >> 5][7 * c + k] = s;
-            }
+        __shared__ long long s_sum[kWarps][32];
+        s_sum[threadIdx.x >> 5][lane] = sum + bulk_reduce(acc, lane);
         __syncthreads();
         if (threadIdx.x < 21) {
-            unsigned long long s = 0;
+            long long s = 0;
 #pragma unroll
             for (int w = 0; w < kWarps; ++w) s += s_sum[w][threadIdx.x];
-            if (s) atomicAdd(&raw[threadIdx.x], s);
+            if (s) atomicAdd(&raw[threadIdx.x], (unsigned long long)s);
         }
     } else if (cur_graph != 0xffffffffu) {
-        flush_bulk(acc, raw, lane);
+        flush();
     }
 }
 

@@ -49,3 +49,22 @@ def test_packed_vertices(n, p):
         b = tc.tc_batch_create([h.handle for h in handles], options=opts)
         assert tc.tc_batch_census(b, len(handles)) == want
         tc.tc_batch_destroy(b)
+
+
+# The bulk sums of a lane are 32 bits wide for 2^31 / n rounds of 32 pairs: with 2^28 vertices, 7.  The
+# other vertices have no link, so the compact graph's counts change in the classes of one link only.
+@pytest.mark.parametrize("k", [300, 1399])
+def test_bulk_sums_of_many_vertices(k):
+    n = 1 << 28
+    c, s, d = hubs([k, 1399, 1000, 700], 5, 100)
+    want = oracle.census_bm(c, s, d)
+    pairs = set(zip(s.tolist(), d.tolist()))
+    mutual = sum((b, a) in pairs for a, b in pairs) // 2
+    want = list(want)
+    want[1] += (len(pairs) - 2 * mutual) * (n - c)
+    want[2] += mutual * (n - c)
+    want[0] = n * (n - 1) * (n - 2) // 6 - sum(want[1:])
+    at = np.sort(np.random.default_rng(k).choice(n, c, replace=False)).astype(np.uint32)
+    with tc.Graph.from_arcs(n, at[s], at[d]) as g:
+        for item_work in (0, 1 << 20):
+            assert list(g.census(options={"algo": tc.TC_ALGO_TRIANGLE, "item_work": item_work})) == want
