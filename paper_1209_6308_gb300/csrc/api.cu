@@ -127,6 +127,13 @@ void DevBuf::release() {
     owned = true;
 }
 
+bool captured(cudaStream_t st) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &cap) == cudaSuccess) return cap != cudaStreamCaptureStatusNone;
+    cudaGetLastError();
+    return true;
+}
+
 int sm_count() {
     int dev = 0, c = 0;
     cudaGetDevice(&dev);
@@ -199,7 +206,12 @@ tc_status staging_take(unsigned long long** out) {
             }
     StagingPage pg = {nullptr, 1u};
     TC_CUDA(cudaHostAlloc((void**)&pg.p, kStagingPage, cudaHostAllocPortable));
-    g_staging.push_back(pg);
+    try {
+        g_staging.push_back(pg);
+    } catch (...) {
+        cudaFreeHost(pg.p);
+        return fail(TC_ERR_OOM, "page-locked staging");
+    }
     *out = reinterpret_cast<unsigned long long*>(pg.p);
     return TC_OK;
 }
@@ -468,6 +480,12 @@ tc_status tc_census_async(tc_graph* g, void* stream, const tc_options* opt, uint
     if (!lk.owns_lock()) return fail(TC_ERR_BUSY, "graph is in use by another call");
     census_fit_chunk(g->s, o);
     Plan* p = nullptr;
+    // a captured census cannot make its plan: where the form is the library's to choose and has none,
+    // the one that the same options plan in the other calls
+    if (!opt && g->s.no_opts && !has_plan(g->s, o) && captured(st)) {
+        TC_TRY(resolve_opts(opt, &g->s.opts, &o));
+        census_fit_chunk(g->s, o);
+    }
     TC_TRY(get_plan(g->s, o, st, &p));
     return census_enqueue(g->s, o, *p, st, reinterpret_cast<unsigned long long*>(d_out16));
 }

@@ -1011,6 +1011,12 @@ __global__ void k_item_splits(const Item* __restrict__ items, uint32_t n, uint32
 }
 }  // namespace
 
+bool has_plan(const GraphStore& g, const Opts& o) {
+    for (auto& p : g.plans)
+        if (p.valid && p.key == o) return true;
+    return false;
+}
+
 tc_status get_plan(GraphStore& g, const Opts& o, cudaStream_t st, Plan** out) {
     for (auto& p : g.plans)
         if (p.valid && p.key == o) { *out = &p; return TC_OK; }

@@ -123,6 +123,7 @@ inline unsigned grid_for(uint64_t n, unsigned block, unsigned cap = 1u << 20) {
 }
 
 int sm_count();
+bool captured(cudaStream_t st);   // launches on st are being captured
 
 inline tc_u128 to_u128(unsigned __int128 x) {
     tc_u128 r;

@@ -626,8 +626,24 @@ tc_status triangle_census_enqueue(GraphStore& g, const Opts& o, const Plan& p, u
     // the range's part of each of the plan's splits
     const uint32_t split[2] = {std::min(std::max(p.split[0], item0) - item0, n_items),
                                std::min(std::max(p.split[1], item0) - item0, n_items)};
-    const bool walk16 = walk16_takes(g);
-    if (walk16 && !g.blk16.p) TC_TRY(lists16_build(g, st));
+    // The 16-bit lists are made at a graph's first such census.  A captured one without them (planned
+    // by another call) cannot wait for that, and one short of memory need not: the general kernel
+    // counts the same.
+    bool walk16 = walk16_takes(g) && !g.no_lists16;
+    if (walk16 && !g.blk16.p) {
+        if (captured(st)) {
+            walk16 = false;
+        } else {
+            const tc_status made = lists16_build(g, st);
+            if (made == TC_ERR_OOM) {
+                g.rec.release();
+                g.no_lists16 = true;
+                walk16 = false;
+            } else if (made != TC_OK) {
+                return made;
+            }
+        }
+    }
     const GraphDev gd = g.dev();
     const uint64_t units = (uint64_t)n_items + (warp_end - warp_begin + 31u) / 32u;
     if (units) {

@@ -28,3 +28,24 @@ def test_no_options_give_the_union_walks_counts(name):
         with tc.Stream(n, 10) as stream:
             stream.push(s, d, np.zeros(len(s), np.uint64))
             assert stream.census(0)[0] == want
+
+
+@pytest.mark.parametrize("census_first", [False, True])
+def test_captured_without_options(census_first):
+    """The captured call takes the form that has a plan: the library's after a census, else the one that
+    the same options planned."""
+    n, s, d = GRAPHS["rmat"]
+    with tc.Graph.from_arcs(n, s, d) as g, tc.Graph.from_arcs(n, s, d, options={"algo": tc.TC_ALGO_UNION}) as u:
+        want = u.census()
+        if census_first:
+            assert g.census() == want
+        else:
+            tc.tc_census_shard_bounds(g.handle, 1)
+        out = torch.zeros(16, dtype=torch.int64, device="cuda")
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            tc.tc_census_async(g.handle, out, stream=torch.cuda.current_stream().cuda_stream)
+        graph.replay()
+        torch.cuda.synchronize()
+        assert out.tolist()[1:] == want[1:]
+        assert g.census() == want
