@@ -653,8 +653,8 @@ FORM_NAMES = {0: "union", 1: "suffix", 2: "triangle"}
 
 
 def triangle_kernel(info) -> str:
-    """The triangle form's walk: the launches of walk16.cu from 2^25 walked entries and 12 per pair on."""
-    return "k_walk16" if info["sum_tri_walk"] >= max(1 << 25, 12 * info["e_sym"]) else "k_triangles"
+    """The triangle form's walk: the launches of walk16.cu from 7 * 2^26 walked entries and 64 per pair on."""
+    return "k_walk16" if info["sum_tri_walk"] >= max(7 << 26, 64 * info["e_sym"]) else "k_triangles"
 
 
 def census_launches(tc, g, n, info, algo) -> int:

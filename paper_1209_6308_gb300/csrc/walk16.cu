@@ -762,13 +762,15 @@ __global__ void __launch_bounds__(kT16, kCtasWarp) k_walk_warp(TriParams P, Stam
 
 }  // namespace
 
-// Against the general kernel (triangles.cu), a census in ms, this / that: R-MAT 18 edge factor 8
-// (59 M entries walked, 30 per pair) 0.338 / 0.352, R-MAT 20 e.f. 8 (342 M, 43) 0.944 / 1.044,
-// Chung-Lu 9 M x 8 (1.2 G, 19) 5.32 / 5.84; but R-MAT 18 e.f. 4 (16 M, 16) 0.245 / 0.231, Chung-Lu
-// 100 k x 16 (16 M, 12) 0.251 / 0.225, R-MAT 14 e.f. 16 (5 M, 25) 0.144 / 0.101: three launches and a
-// 32 KB map per CTA want work, and 8-entry blocks want prefixes longer than a few entries.
+// Against the general kernel (triangles.cu), a graph's first census, which makes the lists, and a later
+// one, in ms, this / that.  Taken: R-MAT 19 edge factor 16 (500 M entries walked, 65 per pair) 1.22 /
+// 1.39, later 0.84 / 1.16; R-MAT 20 e.f. 16 (1.2 G, 78) 2.31 / 2.54, 1.65 / 2.22; R-MAT 24 e.f. 16
+// (42 G, 160) 56.3 / 73.4, 47.4 / 70.1; G(2400, 0.5) (1.3 G, 594) 1.35 / 1.45, 0.88 / 1.31.  Not taken,
+// as the first census would lose: R-MAT 22 e.f. 8 (2.0 G, 60) 4.94 / 4.80, 3.34 / 4.28; R-MAT 18 e.f. 16
+// (204 M, 54) 0.84 / 0.76, 0.53 / 0.57; Chung-Lu 9 M x 16 (3.8 G, 31) 17.4 / 13.4, 10.5 / 12.0; G(1600,
+// 0.5) (378 M, 394) 0.71 / 0.62, 0.33 / 0.48.
 bool walk16_takes(const GraphStore& g) {
-    return g.n <= kTableMaxN && g.sum_tri_walk >= (1ull << 25) && g.sum_tri_walk >= 12ull * g.e_sym;
+    return g.n <= kTableMaxN && g.sum_tri_walk >= (7ull << 26) && g.sum_tri_walk >= 64ull * g.e_sym;
 }
 
 tc_status lists16_build(GraphStore& g, cudaStream_t st) {

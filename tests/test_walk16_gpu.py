@@ -4,7 +4,6 @@ import numpy as np
 import pytest
 
 import graphgen
-import oracle
 import paper_1209_6308_gb300 as tc
 
 pytestmark = pytest.mark.gpu
@@ -26,13 +25,13 @@ def circulant(n, offsets):
     return lo, hi
 
 
-@pytest.mark.parametrize("n,p", [(900, 0.5), (1600, 0.15)])
-def test_dense_graphs_match_the_oracle(n, p):
+@pytest.mark.parametrize("n,p", [(2400, 0.5), (6000, 0.1)])
+def test_dense_graphs_match_the_suffix_form(n, p):
     n, s, d = graphgen.gnp(n, p, seed=n)
-    want = oracle.census_bm(n, s, d)
     with tc.Graph.from_arcs(n, s, d) as g:
         st = g.stats()
-        assert st["sum_tri_walk"] >= max(12 * st["e_sym"], 1 << 25)     # the form under test
+        assert st["sum_tri_walk"] >= max(64 * st["e_sym"], 7 << 26)     # the form under test
+        want = g.census(options={"algo": tc.TC_ALGO_SUFFIX})
         for opts in ({}, {"warp_max_deg": 16}, {"chunk_entries": 8192}, {"item_work": 256}, {"ctas_per_sm": 1}):
             assert g.census(options={"algo": tc.TC_ALGO_TRIANGLE, **opts}) == want
 
@@ -49,7 +48,7 @@ def test_regular_graphs_match_the_suffix_form(name, n, offsets):
     s, d = arcs_of(lo, hi, seed=len(name))
     with tc.Graph.from_arcs(n, s, d) as g:
         st = g.stats()
-        assert st["sum_tri_walk"] >= max(12 * st["e_sym"], 1 << 25)
+        assert st["sum_tri_walk"] >= max(64 * st["e_sym"], 7 << 26)
         assert g.census(options={"algo": tc.TC_ALGO_TRIANGLE}) == g.census(options={"algo": tc.TC_ALGO_SUFFIX})
         grid = sum(np.array(shard) for shard in _shards(g, 3))
         assert list(grid[1:]) == g.census(options={"algo": tc.TC_ALGO_TRIANGLE})[1:]
@@ -61,3 +60,23 @@ def _shards(g, world):
     for r in range(world):
         tc.tc_census_shard(g.handle, out, r, world, options={"algo": tc.TC_ALGO_TRIANGLE})
         yield out.cpu().tolist()
+
+
+def test_captured_census_planned_by_another_call():
+    """No census has made the 16-bit lists yet: the captured one counts without them."""
+    torch = pytest.importorskip("torch")
+    n, s, d = graphgen.gnp(2400, 0.5, seed=2400)
+    opts = {"algo": tc.TC_ALGO_TRIANGLE}
+    with tc.Graph.from_arcs(n, s, d) as g:
+        want = g.census(options={"algo": tc.TC_ALGO_SUFFIX})
+        tc.tc_census_shard_bounds(g.handle, 1, options=opts)
+        out = torch.zeros(16, dtype=torch.int64, device="cuda")
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            tc.tc_census_async(g.handle, out, stream=torch.cuda.current_stream().cuda_stream, options=opts)
+        for _ in range(2):
+            out.zero_()
+            graph.replay()
+            torch.cuda.synchronize()
+            assert out.tolist()[1:] == want[1:]
+            assert g.census(options=opts) == want       # makes the lists; the captured launches stay as they were
