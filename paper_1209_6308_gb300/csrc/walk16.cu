@@ -16,7 +16,7 @@
 // places them in one flattened range of blocks, and the warps take rounds of 32 blocks of that
 // range, so long and short prefixes share the lanes evenly and only the range's end is ragged.
 //
-// Census of R-MAT scale 20 / 26 (edge factor 16): 2.20 -> 1.70 ms / 391.6 -> 276.6 ms against the walk
+// Census of R-MAT scale 20 / 26 (edge factor 16): 2.20 -> 1.60 ms / 391.6 -> 275.1 ms against the walk
 // of 32-bit entries alone.  At scale 20 k_walk16 keeps the shared-memory pipe 66% and the issue
 // slots 60% busy: 32 lookups at random ids cost 3.0 wavefronts (bank conflicts), which neither a
 // denser map (two bits per id: 2.6) nor a plain-shift map for window 0 (fewer instructions, same
