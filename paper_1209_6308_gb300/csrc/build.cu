@@ -122,14 +122,23 @@ __global__ void k_transpose_keys(const uint64_t* __restrict__ key, uint64_t E, i
         tkey[p] = ((key[p] >> 2) & mask) << 32 | p;
 }
 
-// start[x] = the first of the E > 0 sorted keys whose row (key >> shift) is >= x, for x in [0, n].
+// start[x] = the first of the E > 0 sorted keys whose row (key >> shift) is >= x, for x in [0, n]: a
+// search per vertex, whose neighbours in the warp take the same path but for its end; the rows before
+// the first key's and past the last one's (vertices without entries) need none.  Filling the rows
+// between two keys from the keys' side leaves a run of rows without keys to one thread: a build of
+// 10 M vertices in pairs (i, i + n/2), whose first half has no lower entry, took 24.1 ms so and takes
+// 2.9 (pairs anywhere 2.8 and 3.1; R-MAT 20, 15 pairs per vertex, 3.57 and 3.46).
 __global__ void k_row_starts(const uint64_t* __restrict__ key, uint64_t E, int shift, uint32_t n, uint64_t* __restrict__ start) {
-    const uint64_t t0 = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x, stride = (uint64_t)gridDim.x * blockDim.x;
-    for (uint64_t p = t0; p < E; p += stride) {
-        const uint64_t row = key[p] >> shift;
-        for (uint64_t x = p ? (key[p - 1] >> shift) + 1 : 0; x <= row; ++x) start[x] = p;
+    const uint64_t first = key[0] >> shift, last = key[E - 1] >> shift;
+    for (uint64_t x = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; x <= n; x += (uint64_t)gridDim.x * blockDim.x) {
+        uint64_t lo = x <= first ? 0ull : x > last ? E : 1ull, hi = x > first && x <= last ? E - 1ull : lo;
+        while (lo < hi) {   // key lo - 1 is of a row below x, key hi of none
+            const uint64_t mid = (lo + hi) >> 1;
+            if (key[mid] >> shift < x) lo = mid + 1;
+            else hi = mid;
+        }
+        start[x] = lo;
     }
-    for (uint64_t x = (key[E - 1] >> shift) + 1 + t0; x <= n; x += stride) start[x] = E;
 }
 
 // off and up from the starts of the upper pairs (ub) and of the lower entries (lb) of each vertex.
@@ -474,9 +483,10 @@ tc_status finish_graph(GraphStore& g, uint64_t E, int B, uint64_t* ukey, uint32_
         TC_LAUNCH("k_transpose_keys");
         TC_TRY(radix_sort_u64(&kp, &tp, E, 32, 32 + B, st));
         ts = kp;
-        k_row_starts<<<gridE, kB, 0, st>>>(ks, E, B + 2, n, ub);
+        const unsigned gridS = grid_for(n + 1ull, kB, 1u << 16);
+        k_row_starts<<<gridS, kB, 0, st>>>(ks, E, B + 2, n, ub);
         TC_LAUNCH("k_row_starts (upper)");
-        k_row_starts<<<gridE, kB, 0, st>>>(ts, E, 32, n, lb);
+        k_row_starts<<<gridS, kB, 0, st>>>(ts, E, 32, n, lb);
         TC_LAUNCH("k_row_starts (lower)");
     } else {
         TC_CUDA(cudaMemsetAsync(ub, 0, sizeof(uint64_t) * (n + 1ull), st));
