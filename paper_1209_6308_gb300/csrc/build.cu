@@ -502,8 +502,9 @@ tc_status finish_graph(GraphStore& g, uint64_t E, int B, uint64_t* ukey, uint32_
     TC_LAUNCH("k_graph_sums");
     if (E) {
         // the suffix counts of the per upper pair tables; the walk lengths go to stats[8..9]
-        k_pair_tables<<<gridN, kB, 0, st>>>(off, g.adj.as<uint32_t>(), g.up.as<uint32_t>(), ub, lb, n, d_stats + 12, ts,
-                                            g.vs.as<uint2>(), g.us.as<uint2>(), d_stats + 8);
+        // (at most 2E / 33 lists have more than 32 entries)
+        k_pair_tables<<<grid_lists(n, std::min<uint64_t>(n, 2ull * E / 33)), kB, 0, st>>>(off, g.adj.as<uint32_t>(), g.up.as<uint32_t>(), ub, lb, n,
+                                            d_stats + 12, ts, g.vs.as<uint2>(), g.us.as<uint2>(), d_stats + 8);
         TC_LAUNCH("k_pair_tables");
         // lists longer than kLongList: at most 2E / kLongList of them, the first ids
         const uint64_t n_long = std::min<uint64_t>(n, 2ull * E / kLongList + 1);

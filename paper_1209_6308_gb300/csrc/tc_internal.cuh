@@ -123,6 +123,14 @@ inline unsigned grid_for(uint64_t n, unsigned block, unsigned cap = 1u << 20) {
 }
 
 int sm_count();
+// CTAs of 256 threads for a kernel over n lists that gives each of at most `wide` longer ones a warp
+// and lets a warp's lanes share 32 shorter ones: a thread per list, and where that is few, a warp per
+// longer list up to eight CTAs per SM.  (A thread per list alone: a dense graph of 2400 vertices has its
+// 2400 lists walked by ten CTAs.)
+inline unsigned grid_lists(uint64_t n, uint64_t wide) {
+    const unsigned by_list = grid_for(n, 256, 1u << 16), by_warp = grid_for(32ull * wide, 256, 8u * (unsigned)sm_count());
+    return by_list > by_warp ? by_list : by_warp;
+}
 bool captured(cudaStream_t st);   // launches on st are being captured
 
 inline tc_u128 to_u128(unsigned __int128 x) {

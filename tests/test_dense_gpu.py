@@ -1,0 +1,45 @@
+"""Dense and small graphs, whose few long lists must not be left to a few CTAs: a step over the lists of
+a dense graph is compared with the same step over a sparse graph of as many entries."""
+import time
+
+import pytest
+import torch
+
+import paper_1209_6308_gb300 as tc
+
+pytestmark = pytest.mark.gpu
+
+
+def dense(n, degree):
+    """x -> x + 1 .. x + degree/2 (mod n): every list has `degree` entries."""
+    x = torch.arange(n, device="cuda", dtype=torch.int64).repeat_interleave(degree // 2)
+    return n, x.int(), ((x + 1 + torch.arange(degree // 2, device="cuda").repeat(n)) % n).int()
+
+
+def best_of(calls, reps=7):
+    """Best wall time in s of each call (name -> function), taken in turn."""
+    best = dict.fromkeys(calls, float("inf"))
+    for rep in range(reps):
+        for name, call in calls.items():
+            torch.cuda.synchronize()
+            t = time.perf_counter()
+            call()
+            torch.cuda.synchronize()
+            if rep:
+                best[name] = min(best[name], time.perf_counter() - t)
+    return best
+
+
+def test_build_of_a_dense_graph():
+    """8 M pairs in 4099 lists of 4094 entries or in 2^18 of 64: the same bytes through the sorts and tables,
+    so not slower by more than half (the clock's noise and the coarser tail)."""
+    graphs = {"dense": dense(4099, 4094), "sparse": dense(1 << 18, 64)}
+    best = best_of({k: lambda g=g: tc.Graph.from_arcs(*g).close() for k, g in graphs.items()})
+    assert best["dense"] <= 1.5 * best["sparse"], best
+
+
+@pytest.mark.parametrize("n,degree", [(33, 32), (35, 34), (70, 64), (300, 254), (4099, 4094), (4101, 4098)])
+def test_counts_of_dense_graphs(n, degree):
+    with tc.Graph.from_arcs(*dense(n, degree)) as g:
+        forms = [g.census(options={"algo": k}) for k in (0, 1, 2)]
+        assert forms[0] == forms[1] == forms[2]
