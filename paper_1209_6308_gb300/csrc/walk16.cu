@@ -790,7 +790,7 @@ tc_status lists16_build(GraphStore& g, cudaStream_t st) {
     TC_CUDA(cudaStreamSynchronize(st));
     DevBuf blk;
     TC_TRY(blk.alloc_persistent(sizeof(uint4) * (n_blocks ? n_blocks : 1u)));
-    k_lists16<<<grid_for(n, 256, 1u << 16), 256, 0, st>>>(gd, n, g.n_wide, first.as<uint32_t>(), g.rec.as<uint4>(),
+    k_lists16<<<grid_lists(n, g.n_wide), 256, 0, st>>>(gd, n, g.n_wide, first.as<uint32_t>(), g.rec.as<uint4>(),
                                                           g.rec.as<uint4>() + n, blk.as<uint16_t>());
     TC_LAUNCH("k_lists16");
     TC_CUDA(cudaStreamSynchronize(st));   // later censuses may come on other streams
