@@ -62,3 +62,13 @@ def test_first_census_of_a_dense_graph():
             later = min(later, best_of({"census": lambda: h.census(options=opts)}, 4)["census"])
     build = best_of({"build": lambda: tc.Graph.from_arcs(*g).close()})["build"]
     assert first - later <= build / 3, (first, later, build)
+
+
+def test_64_states_of_rows_below_and_above_the_cta_limit():
+    """Rows of 254 entries go a warp each, rows of 258 a CTA each: the fewer entries take no longer, with
+    15% for the clock's noise."""
+    graphs = {d: tc.Graph.from_arcs(*dense(1025, d)) for d in (254, 258)}
+    best = best_of({d: g.census64 for d, g in graphs.items()}, 40)
+    for g in graphs.values():
+        g.close()
+    assert best[254] <= 1.15 * best[258], best
