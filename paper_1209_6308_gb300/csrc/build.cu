@@ -424,10 +424,16 @@ __global__ void k_upper_counts(const uint64_t* off, const uint32_t* adj, uint32_
 }
 
 
+// Below this many vertices and pairs a build takes its graph's memory first, while the stream is idle:
+// a later allocation that outlives the stream waits for the sorts.
+constexpr uint64_t kStoreFirst = 1ull << 22;
+
 // Steps shared by both inputs: E unique pairs (ukey = lo<<B | hi, udir relative to lo) and
-// degrees -> relabel, CSR, up[], stats.
-tc_status finish_graph(GraphStore& g, uint64_t E, int B, uint64_t* ukey, uint32_t* udir, uint32_t* deg,
-                       DevBuf& stats, cudaStream_t st) {
+// degrees -> relabel, CSR, up[], stats.  Each input is released after its last use, and a large
+// graph's own memory is taken after the sorts, in place of the buffer they leave over: 44 B per pair and
+// 32 B per vertex at most (up front, with the inputs kept, it was 64 B per pair).
+tc_status finish_graph(GraphStore& g, uint64_t E, int B, DevBuf& ukey, DevBuf& udir, DevBuf& deg, DevBuf& stats,
+                       cudaStream_t st) {
     const uint32_t n = g.n;
     const unsigned gridE = grid_for(E, kB, 1u << 16), gridN = grid_for(n, kB, 1u << 16);
     // relabel by descending degree
@@ -435,23 +441,29 @@ tc_status finish_graph(GraphStore& g, uint64_t E, int B, uint64_t* ukey, uint32_
     TC_TRY(rk.alloc(sizeof(uint64_t) * n, st));
     TC_TRY(rtmp.alloc(sizeof(uint64_t) * n, st));
     // the graph's buffers, carved from one (an allocation that outlives its stream is synchronised)
-    {
+    const bool store_first = n + E < kStoreFirst;
+    auto make_store = [&]() -> tc_status {
         struct { DevBuf* b; size_t bytes; } parts[] = {
             {&g.off, sizeof(uint64_t) * (n + 1ull)}, {&g.ub, sizeof(uint64_t) * (n + 1ull)},
             {&g.adj, sizeof(uint32_t) * (2 * E + 4)},   // read in aligned blocks of four
-            {&g.up, sizeof(uint32_t) * n}, {&g.new_of_old, sizeof(uint32_t) * n}, {&g.rp, sizeof(uint32_t) * E},
-            {&g.vs, sizeof(uint2) * E}, {&g.us, sizeof(uint2) * E}};
+            {&g.up, sizeof(uint32_t) * n}, {&g.rp, sizeof(uint32_t) * E},
+            {&g.vs, sizeof(uint2) * E}, {&g.us, sizeof(uint2) * E},
+            {&g.new_of_old, store_first ? sizeof(uint32_t) * n : 0u}};   // last: else it has memory of its own
         size_t total = 0;
         for (const auto& q : parts) total += (q.bytes + 255u) & ~(size_t)255u;
         TC_TRY(g.store.alloc_persistent(total));
         size_t at = 0;
         for (const auto& q : parts) {
-            q.b->carve(g.store, at, q.bytes);
+            if (q.b != &g.new_of_old || store_first) q.b->carve(g.store, at, q.bytes);
             at += (q.bytes + 255u) & ~(size_t)255u;
         }
-    }
-    k_relabel_keys<<<gridN, kB, 0, st>>>(deg, n, B, rk.as<uint64_t>());
+        return TC_OK;
+    };
+    if (store_first) TC_TRY(make_store());
+    else TC_TRY(g.new_of_old.alloc_persistent(sizeof(uint32_t) * n));
+    k_relabel_keys<<<gridN, kB, 0, st>>>(deg.as<uint32_t>(), n, B, rk.as<uint64_t>());
     TC_LAUNCH("k_relabel_keys");
+    deg.release();
     uint64_t* kp = rk.as<uint64_t>();
     uint64_t* tp = rtmp.as<uint64_t>();
     TC_TRY(radix_sort_u64(&kp, &tp, n, B, 2 * B, st));   // stable: ties stay in id order
@@ -459,21 +471,21 @@ tc_status finish_graph(GraphStore& g, uint64_t E, int B, uint64_t* ukey, uint32_
     TC_LAUNCH("k_perm");
     rk.release();
     rtmp.release();
-    uint64_t *off = g.off.as<uint64_t>(), *ub = g.ub.as<uint64_t>();
     unsigned long long* d_stats = stats.as<unsigned long long>();
     // the pairs in the new ids, sorted by (lo, hi): the upper lists in order, a pair's place its table
     // index; and their transpose, sorted by hi: the lower lists in order
     DevBuf key, tmp, tkey, lbuf;
-    TC_TRY(lbuf.alloc(sizeof(uint64_t) * (n + 1ull), st));
-    uint64_t* lb = lbuf.as<uint64_t>();
     const uint64_t* ks = nullptr;
     const uint64_t* ts = nullptr;
     if (E) {
         TC_TRY(key.alloc(sizeof(uint64_t) * E, st));
+        k_upper_keys<<<gridE, kB, 0, st>>>(ukey.as<uint64_t>(), udir.as<uint32_t>(), E, B, g.new_of_old.as<uint32_t>(),
+                                           key.as<uint64_t>());
+        TC_LAUNCH("k_upper_keys");
+        ukey.release();
+        udir.release();
         TC_TRY(tmp.alloc(sizeof(uint64_t) * E, st));
         TC_TRY(tkey.alloc(sizeof(uint64_t) * E, st));
-        k_upper_keys<<<gridE, kB, 0, st>>>(ukey, udir, E, B, g.new_of_old.as<uint32_t>(), key.as<uint64_t>());
-        TC_LAUNCH("k_upper_keys");
         kp = key.as<uint64_t>();
         tp = tmp.as<uint64_t>();
         TC_TRY(radix_sort_u64(&kp, &tp, E, 2, 2 * B + 2, st));
@@ -483,6 +495,13 @@ tc_status finish_graph(GraphStore& g, uint64_t E, int B, uint64_t* ukey, uint32_
         TC_LAUNCH("k_transpose_keys");
         TC_TRY(radix_sort_u64(&kp, &tp, E, 32, 32 + B, st));
         ts = kp;
+        for (DevBuf* b : {&key, &tmp, &tkey})
+            if (b->p != ks && b->p != ts) b->release();
+    }
+    if (!store_first) TC_TRY(make_store());
+    TC_TRY(lbuf.alloc(sizeof(uint64_t) * (n + 1ull), st));
+    uint64_t *off = g.off.as<uint64_t>(), *ub = g.ub.as<uint64_t>(), *lb = lbuf.as<uint64_t>();
+    if (E) {
         const unsigned gridS = grid_for(n + 1ull, kB, 1u << 16);
         k_row_starts<<<gridS, kB, 0, st>>>(ks, E, B + 2, n, ub);
         TC_LAUNCH("k_row_starts (upper)");
@@ -581,7 +600,7 @@ tc_status graph_from_pairs(GraphStore& g, int B, uint32_t E, DevBuf& ukey, DevBu
                                                              deg.as<uint32_t>(), stats.as<unsigned long long>());
         TC_LAUNCH("k_degrees");
     }
-    return finish_graph(g, E, B, ukey.as<uint64_t>(), udir.as<uint32_t>(), deg.as<uint32_t>(), stats, st);
+    return finish_graph(g, E, B, ukey, udir, deg, stats, st);
 }
 
 }  // namespace
@@ -664,7 +683,9 @@ tc_status build_from_csr(GraphStore& g, const uint64_t* d_off, const uint32_t* d
     k_csr_pairs<<<gridN, kB, 0, st>>>(d_off, d_adj, n, B, upos.as<uint32_t>(), ukey.as<uint64_t>(),
                                       udir.as<uint32_t>(), deg.as<uint32_t>(), stats.as<unsigned long long>());
     TC_LAUNCH("k_csr_pairs");
-    TC_TRY(finish_graph(g, E, B, ukey.as<uint64_t>(), udir.as<uint32_t>(), deg.as<uint32_t>(), stats, st));
+    cnt.release();
+    upos.release();
+    TC_TRY(finish_graph(g, E, B, ukey, udir, deg, stats, st));
     g.dups = 0;
     g.loops = 0;
     return TC_OK;
