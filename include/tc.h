@@ -117,7 +117,8 @@ typedef struct {
  * pair's share of the staged lower lists); 4 B per entry walked; the 96 counters and the fold. */
 
 /* Build a graph from an arc list (Sec. 6, Fig. 7).  src[i] -> dst[i] for i < m; self-loops
- * and repeated arcs are dropped and counted.  Ids >= n give TC_ERR_RANGE.  src/dst are
+ * and repeated arcs are dropped and counted.  Ids >= n give TC_ERR_RANGE, as do 2^32 arcs or more
+ * and, after cleaning, 2^31 connected pairs or more.  src/dst are
  * device pointers if ptr_is_device, else host pointers: page-locked host arrays (cudaHostAlloc,
  * cudaHostRegister) are read once by the build's first kernel directly over the host link,
  * pageable ones are copied to the device on `stream` first.
@@ -130,7 +131,8 @@ tc_status tc_graph_create_arcs(uint32_t n, uint64_t m, const uint32_t* src, cons
  * adj_flagged[off[n]] where each entry is (id << 2) | dir, dir 1 = owner->id, 2 = id->owner,
  * 3 = both.  Every list must be strictly ascending by id, loop-free, with dir != 0, and the
  * lists must be symmetric (x in N[y] iff y in N[x], with mirrored dir bits); otherwise
- * TC_ERR_ARG.  Pointers are device or host as for tc_graph_create_arcs. */
+ * TC_ERR_ARG.  2^32 entries or more give TC_ERR_RANGE.  Pointers are device or host as for
+ * tc_graph_create_arcs. */
 tc_status tc_graph_create_csr(uint32_t n, const uint64_t* off, const uint32_t* adj_flagged,
                               int ptr_is_device, void* stream, const tc_options* opt, tc_graph** out);
 

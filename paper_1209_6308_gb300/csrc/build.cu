@@ -435,6 +435,8 @@ constexpr uint64_t kStoreFirst = 1ull << 22;
 tc_status finish_graph(GraphStore& g, uint64_t E, int B, DevBuf& ukey, DevBuf& udir, DevBuf& deg, DevBuf& stats,
                        cudaStream_t st) {
     const uint32_t n = g.n;
+    // the lists hold 2E entries, and the 64-state census sorts them all: 32-bit counts
+    if (E >= (1ull << 31)) return fail(TC_ERR_RANGE, "more than 2^31-1 connected pairs");
     const unsigned gridE = grid_for(E, kB, 1u << 16), gridN = grid_for(n, kB, 1u << 16);
     // relabel by descending degree
     DevBuf rk, rtmp;
