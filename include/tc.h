@@ -148,8 +148,11 @@ tc_status tc_census_opts(tc_graph* g, void* stream, const tc_options* opt, tc_u1
 
 /* Asynchronous census: enqueues the kernels on `stream` and writes, when they finish,
  * counts of classes 1..15 to d_out16[1..15] (device memory, uint64) and 0 to d_out16[0].
- * The null count needs 128-bit arithmetic: obtain it with tc_null_count.  Does not
- * synchronise; d_out16 must stay valid until the stream reaches the end of the census. */
+ * The null count needs 128-bit arithmetic: obtain it with tc_null_count.  d_out16 must stay valid
+ * until the stream reaches the end of the census.  The first call of a graph with given options makes
+ * their plan, and a large graph's first plan of TC_ALGO_TRIANGLE also its 16-bit lists (52 B per vertex
+ * with a neighbour and about 4 B per pair, kept with the graph): it allocates and synchronises `stream`.
+ * Later calls only launch, and can be captured.  (A graph keeps the last four plans.) */
 tc_status tc_census_async(tc_graph* g, void* stream, const tc_options* opt, uint64_t* d_out16);
 
 /* Instrumented census, for scheduling and for training the learned cost model: the same
@@ -159,7 +162,7 @@ tc_status tc_census_async(tc_graph* g, void* stream, const tc_options* opt, uint
  * may be NULL) receives, for each of the tc_census_grid() CTAs, the global timer in ns at
  * its start, at the end of its CTA work items and at its end (in the TC_ALGO_TRIANGLE form,
  * those of the triangle walk; where that takes launches of fewer CTAs, a CTA's times fill the
- * entries of several).  Does not synchronise. */
+ * entries of several).  Synchronises only where tc_census_async does. */
 tc_status tc_census_profile(tc_graph* g, void* stream, const tc_options* opt, uint64_t* d_out16,
                             uint64_t* d_vcost, uint64_t* d_phase);
 
@@ -172,7 +175,7 @@ tc_status tc_census_profile(tc_graph* g, void* stream, const tc_options* opt, ui
  * this shard's counts of classes 1..15 (index 0 = 0), as tc_census_async does; summing the
  * world shards' outputs (an all-reduce of 16 uint64) gives the census's classes 1..15, and
  * tc_null_count of that sum gives the null count.  The first call for a plan and a world
- * computes the shards and synchronises `stream`; later calls only enqueue.  TC_ERR_BUSY if the
+ * computes the shards and synchronises `stream` (as may the plan: tc_census_async); later calls only enqueue.  TC_ERR_BUSY if the
  * graph is in use by another call; TC_ERR_RANGE if world > 2^20. */
 tc_status tc_census_shard(tc_graph* g, void* stream, const tc_options* opt, uint32_t rank, uint32_t world,
                           uint64_t* d_out16);

@@ -486,7 +486,7 @@ tc_status tc_census_async(tc_graph* g, void* stream, const tc_options* opt, uint
         TC_TRY(resolve_opts(opt, &g->s.opts, &o));
         census_fit_chunk(g->s, o);
     }
-    TC_TRY(get_plan(g->s, o, st, &p));
+    TC_TRY(census_plan(g->s, o, st, &p));
     return census_enqueue(g->s, o, *p, st, reinterpret_cast<unsigned long long*>(d_out16));
 }
 
@@ -500,7 +500,7 @@ tc_status tc_census_profile(tc_graph* g, void* stream, const tc_options* opt, ui
     if (!lk.owns_lock()) return fail(TC_ERR_BUSY, "graph is in use by another call");
     census_fit_chunk(g->s, o);
     Plan* p = nullptr;
-    TC_TRY(get_plan(g->s, o, st, &p));
+    TC_TRY(census_plan(g->s, o, st, &p));
     return census_enqueue(g->s, o, *p, st, reinterpret_cast<unsigned long long*>(d_out16),
                           reinterpret_cast<unsigned long long*>(d_vcost), reinterpret_cast<unsigned long long*>(d_phase));
 }
@@ -517,7 +517,7 @@ tc_status tc_census_shard(tc_graph* g, void* stream, const tc_options* opt, uint
     if (!lk.owns_lock()) return fail(TC_ERR_BUSY, "graph is in use by another call");
     census_fit_chunk(g->s, o);
     Plan* p = nullptr;
-    TC_TRY(get_plan(g->s, o, st, &p));
+    TC_TRY(census_plan(g->s, o, st, &p));
     TC_TRY(plan_shards(g->s, o, *p, world, st));
     const uint32_t* b = p->shard_bounds.data();
     const uint32_t i0 = b[2 * rank], i1 = b[2 * rank + 2];
@@ -537,7 +537,7 @@ tc_status tc_census_shard_bounds(tc_graph* g, void* stream, const tc_options* op
     if (!lk.owns_lock()) return fail(TC_ERR_BUSY, "graph is in use by another call");
     census_fit_chunk(g->s, o);
     Plan* p = nullptr;
-    TC_TRY(get_plan(g->s, o, st, &p));
+    TC_TRY(census_plan(g->s, o, st, &p));
     TC_TRY(plan_shards(g->s, o, *p, world, st));
     for (uint32_t r = 0; r <= world; ++r) {
         bounds[2 * r] = p->shard_bounds[2 * r];
@@ -561,7 +561,7 @@ tc_status tc_census_opts(tc_graph* g, void* stream, const tc_options* opt, tc_u1
     if (!lk.owns_lock()) return fail(TC_ERR_BUSY, "graph is in use by another call");
     census_fit_chunk(g->s, o);
     Plan* p = nullptr;
-    TC_TRY(get_plan(g->s, o, st, &p));
+    TC_TRY(census_plan(g->s, o, st, &p));
     TC_TRY(census_enqueue(g->s, o, *p, st, g->s.acc.as<unsigned long long>()));
     TC_CUDA(cudaMemcpyAsync(g->s.h_counts, g->s.acc.p, sizeof(unsigned long long) * 16, cudaMemcpyDeviceToHost, st));
     TC_CUDA(cudaStreamSynchronize(st));

@@ -69,7 +69,7 @@ struct GraphStore {
     DevBuf off, adj, up, new_of_old;
     DevBuf ub, rp, vs, us;   // per upper pair tables (see GraphDev)
     DevBuf rec, blk16;   // 16-bit lower lists (see GraphDev): rec holds rec, rec2 and n16 of the active vertices
-    bool no_lists16 = false;   // the device had no room for them
+    bool no_lists16 = false;   // the device had no room for them since the last plan was made
     DevBuf ctr;        // census work counters (uint32 x 4)
     DevBuf acc;        // census accumulators (uint64 x 16)
     DevBuf cost;       // optional per-vertex predicted cost (float x n) for the learned schedule
@@ -135,10 +135,12 @@ int bits_for(uint32_t n);
 tc_status graph_create_sorted(uint32_t n, const uint64_t* d_keys, uint64_t m, cudaStream_t st, const tc_options* opt,
                               tc_graph** out);
 
-// Enqueue one census on `st`; counts of classes 1..15 go to d_out16, index 0 is 0.  No host synchronisation, no allocation once
-// the plan for `o` exists (get_plan allocates it on first use).
+// Enqueue one census on `st`; counts of classes 1..15 go to d_out16, index 0 is 0.  No host synchronisation and
+// no allocation: census_plan, called first, does both where the plan or the lists are not there yet.
 bool has_plan(const GraphStore& g, const Opts& o);
 tc_status get_plan(GraphStore& g, const Opts& o, cudaStream_t st, Plan** out);
+// The plan and, for the triangle form of a large graph, its 16-bit lists: before census_enqueue.
+tc_status census_plan(GraphStore& g, const Opts& o, cudaStream_t st, Plan** out);
 // The single-graph census's form (map or not) and, for an automatic chunk, its size: call
 // before get_plan, whose items depend on the chunk.
 bool census_map(const GraphStore& g, const Opts& o);

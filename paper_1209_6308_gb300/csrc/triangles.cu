@@ -608,6 +608,21 @@ tc_status triangles_launch(const GraphDev& gd, const Opts& o, const Item* items,
     return TC_OK;
 }
 
+// The 16-bit lists are made with a graph's first plan of this form, so that a census that has its plan only
+// launches.  One that is captured cannot make them (its plan may be another call's: the 64-state census
+// and the server read no such lists), and a device without room for them need not: the general kernel
+// counts the same.  The next plan tries again.
+tc_status census_plan(GraphStore& g, const Opts& o, cudaStream_t st, Plan** out) {
+    if (!has_plan(g, o)) g.no_lists16 = false;
+    TC_TRY(get_plan(g, o, st, out));
+    if (o.algo != TC_ALGO_TRIANGLE || g.blk16.p || g.no_lists16 || !walk16_takes(g) || captured(st)) return TC_OK;
+    const tc_status made = lists16_build(g, st);
+    if (made != TC_ERR_OOM) return made;
+    g.rec.release();
+    g.no_lists16 = true;
+    return TC_OK;
+}
+
 tc_status triangle_census_enqueue(GraphStore& g, const Opts& o, const Plan& p, uint32_t item0, uint32_t n_items,
                                   uint32_t warp_begin, uint32_t warp_end, cudaStream_t st, unsigned long long* d_out16,
                                   unsigned long long* d_vcost, unsigned long long* d_phase) {
@@ -626,24 +641,8 @@ tc_status triangle_census_enqueue(GraphStore& g, const Opts& o, const Plan& p, u
     // the range's part of each of the plan's splits
     const uint32_t split[2] = {std::min(std::max(p.split[0], item0) - item0, n_items),
                                std::min(std::max(p.split[1], item0) - item0, n_items)};
-    // The 16-bit lists are made at a graph's first such census.  A captured one without them (planned
-    // by another call) cannot wait for that, and one short of memory need not: the general kernel
-    // counts the same.
-    bool walk16 = walk16_takes(g) && !g.no_lists16;
-    if (walk16 && !g.blk16.p) {
-        if (captured(st)) {
-            walk16 = false;
-        } else {
-            const tc_status made = lists16_build(g, st);
-            if (made == TC_ERR_OOM) {
-                g.rec.release();
-                g.no_lists16 = true;
-                walk16 = false;
-            } else if (made != TC_OK) {
-                return made;
-            }
-        }
-    }
+    // without the lists (census_plan) the general kernel counts the same
+    const bool walk16 = walk16_takes(g) && g.blk16.p;
     const GraphDev gd = g.dev();
     const uint64_t units = (uint64_t)n_items + (warp_end - warp_begin + 31u) / 32u;
     if (units) {
