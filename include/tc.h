@@ -162,7 +162,10 @@ tc_status tc_census_async(tc_graph* g, void* stream, const tc_options* opt, uint
  * may be NULL) receives, for each of the tc_census_grid() CTAs, the global timer in ns at
  * its start, at the end of its CTA work items and at its end (in the TC_ALGO_TRIANGLE form,
  * those of the triangle walk; where that takes launches of fewer CTAs, a CTA's times fill the
- * entries of several).  Synchronises only where tc_census_async does. */
+ * entries of several).  opt NULL on a graph made with NULL is TC_ALGO_UNION here, as an algo of 0 is, so
+ * that what is measured fits tc_costmodel_samples, tc_census_grid(NULL) and the learned schedule of the
+ * same options: to profile the form tc_census(NULL) runs, ask for TC_ALGO_TRIANGLE in both calls.
+ * Synchronises only where tc_census_async does. */
 tc_status tc_census_profile(tc_graph* g, void* stream, const tc_options* opt, uint64_t* d_out16,
                             uint64_t* d_vcost, uint64_t* d_phase);
 
@@ -171,7 +174,7 @@ tc_status tc_census_profile(tc_graph* g, void* stream, const tc_options* opt, ui
  * census).  The census's work - the plan's CTA work items in order, then the vertices handled
  * one warp each, in id order - is cut into `world` contiguous shards of about equal work
  * (the plan's exact per-pair work units), and this call runs shard `rank` (0 <= rank < world,
- * else TC_ERR_ARG).  Every rank holds the same graph.  d_out16 (device, 16 uint64) receives
+ * else TC_ERR_ARG).  opt as for tc_census_opts.  Every rank holds the same graph.  d_out16 (device, 16 uint64) receives
  * this shard's counts of classes 1..15 (index 0 = 0), as tc_census_async does; summing the
  * world shards' outputs (an all-reduce of 16 uint64) gives the census's classes 1..15, and
  * tc_null_count of that sum gives the null count.  The first call for a plan and a world
@@ -182,7 +185,8 @@ tc_status tc_census_shard(tc_graph* g, void* stream, const tc_options* opt, uint
 
 /* Where the shards of tc_census_shard start: bounds[2r] = the first CTA work item and
  * bounds[2r+1] = the first one-warp-per-vertex id of shard r, for r = 0..world (r = world: the
- * item count and the end of that tier's id range).  Host array of 2 (world + 1) uint32.
+ * item count and the end of that tier's id range).  opt as for tc_census_opts.  Host array of
+ * 2 (world + 1) uint32.
  * Synchronises `stream` when the shards are not yet computed. */
 tc_status tc_census_shard_bounds(tc_graph* g, void* stream, const tc_options* opt, uint32_t world, uint32_t* bounds);
 
@@ -226,7 +230,7 @@ tc_status tc_census_batch(tc_graph* const* gs, uint32_t k, void* stream, uint64_
 /* A reusable batch: one combined work plan for the k graphs (largest graph first; CTA items of
  * every graph, then one-warp-per-vertex blocks of every graph, drawn by one persistent launch
  * from two device work counters) and that launch captured in a CUDA graph.  The graphs must
- * outlive the batch.  opt may be NULL (the defaults of tc_options).  Synchronises `stream`. */
+ * outlive the batch.  opt may be NULL (the defaults of tc_options, so TC_ALGO_UNION).  Synchronises `stream`. */
 typedef struct tc_batch tc_batch;
 tc_status tc_batch_create(tc_graph* const* gs, uint32_t k, const tc_options* opt, void* stream, tc_batch** out);
 

@@ -245,6 +245,20 @@ tc_status resolve_census_opts(const GraphStore& g, const tc_options* opt, Opts* 
     return resolve_opts(&t, nullptr, out);
 }
 
+// The options and the plan of a census of g, whole or in `world` shards (0: whole).  A captured one cannot
+// make its plan (or its shards): where the form is the library's to choose and has none, an earlier call
+// whose options' algo is 0, the union walk, may have.
+tc_status prepare_census(GraphStore& g, const tc_options* opt, uint32_t world, cudaStream_t st, Opts* o, Plan** p) {
+    TC_TRY(resolve_census_opts(g, opt, o));
+    census_fit_chunk(g, *o);
+    if (!opt && g.no_opts && !has_plan(g, *o, world) && captured(st)) {
+        TC_TRY(resolve_opts(opt, &g.opts, o));
+        census_fit_chunk(g, *o);
+    }
+    TC_TRY(census_plan(g, *o, st, p));
+    return world ? plan_shards(g, *o, **p, world, st) : TC_OK;
+}
+
 tc_status init_graph(tc_graph* g, uint32_t n, const tc_options* opt) {
     g->s.n = n;
     Opts check;
@@ -474,19 +488,11 @@ tc_u128 tc_null_count(uint32_t n, const uint64_t counts16[16]) {
 tc_status tc_census_async(tc_graph* g, void* stream, const tc_options* opt, uint64_t* d_out16) {
     if (!g || !d_out16) return fail(TC_ERR_ARG, "null argument");
     cudaStream_t st = (cudaStream_t)stream;
-    Opts o;
-    TC_TRY(resolve_census_opts(g->s, opt, &o));
     std::unique_lock<std::mutex> lk(g->s.busy, std::try_to_lock);
     if (!lk.owns_lock()) return fail(TC_ERR_BUSY, "graph is in use by another call");
-    census_fit_chunk(g->s, o);
+    Opts o;
     Plan* p = nullptr;
-    // a captured census cannot make its plan: where the form is the library's to choose and has none,
-    // the one that the same options plan in the other calls
-    if (!opt && g->s.no_opts && !has_plan(g->s, o) && captured(st)) {
-        TC_TRY(resolve_opts(opt, &g->s.opts, &o));
-        census_fit_chunk(g->s, o);
-    }
-    TC_TRY(census_plan(g->s, o, st, &p));
+    TC_TRY(prepare_census(g->s, opt, 0, st, &o, &p));
     return census_enqueue(g->s, o, *p, st, reinterpret_cast<unsigned long long*>(d_out16));
 }
 
@@ -511,14 +517,11 @@ tc_status tc_census_shard(tc_graph* g, void* stream, const tc_options* opt, uint
     if (world == 0 || rank >= world) return fail(TC_ERR_ARG, "tc_census_shard: need 0 <= rank < world");
     if (world > (1u << 20)) return fail(TC_ERR_RANGE, "tc_census_shard: world above 2^20");
     cudaStream_t st = (cudaStream_t)stream;
-    Opts o;
-    TC_TRY(resolve_opts(opt, &g->s.opts, &o));
     std::unique_lock<std::mutex> lk(g->s.busy, std::try_to_lock);
     if (!lk.owns_lock()) return fail(TC_ERR_BUSY, "graph is in use by another call");
-    census_fit_chunk(g->s, o);
+    Opts o;
     Plan* p = nullptr;
-    TC_TRY(census_plan(g->s, o, st, &p));
-    TC_TRY(plan_shards(g->s, o, *p, world, st));
+    TC_TRY(prepare_census(g->s, opt, world, st, &o, &p));
     const uint32_t* b = p->shard_bounds.data();
     const uint32_t i0 = b[2 * rank], i1 = b[2 * rank + 2];
     const uint32_t v0 = b[2 * rank + 1], v1 = b[2 * rank + 3];
@@ -531,14 +534,11 @@ tc_status tc_census_shard_bounds(tc_graph* g, void* stream, const tc_options* op
     if (world == 0) return fail(TC_ERR_ARG, "tc_census_shard_bounds: world must be >= 1");
     if (world > (1u << 20)) return fail(TC_ERR_RANGE, "tc_census_shard_bounds: world above 2^20");
     cudaStream_t st = (cudaStream_t)stream;
-    Opts o;
-    TC_TRY(resolve_opts(opt, &g->s.opts, &o));
     std::unique_lock<std::mutex> lk(g->s.busy, std::try_to_lock);
     if (!lk.owns_lock()) return fail(TC_ERR_BUSY, "graph is in use by another call");
-    census_fit_chunk(g->s, o);
+    Opts o;
     Plan* p = nullptr;
-    TC_TRY(census_plan(g->s, o, st, &p));
-    TC_TRY(plan_shards(g->s, o, *p, world, st));
+    TC_TRY(prepare_census(g->s, opt, world, st, &o, &p));
     for (uint32_t r = 0; r <= world; ++r) {
         bounds[2 * r] = p->shard_bounds[2 * r];
         bounds[2 * r + 1] = p->warp_begin + p->shard_bounds[2 * r + 1];
@@ -555,13 +555,11 @@ uint32_t tc_census_grid(const tc_options* opt) {
 tc_status tc_census_opts(tc_graph* g, void* stream, const tc_options* opt, tc_u128 out[16]) {
     if (!g || !out) return fail(TC_ERR_ARG, "null argument");
     cudaStream_t st = (cudaStream_t)stream;
-    Opts o;
-    TC_TRY(resolve_census_opts(g->s, opt, &o));
     std::unique_lock<std::mutex> lk(g->s.busy, std::try_to_lock);
     if (!lk.owns_lock()) return fail(TC_ERR_BUSY, "graph is in use by another call");
-    census_fit_chunk(g->s, o);
+    Opts o;
     Plan* p = nullptr;
-    TC_TRY(census_plan(g->s, o, st, &p));
+    TC_TRY(prepare_census(g->s, opt, 0, st, &o, &p));
     TC_TRY(census_enqueue(g->s, o, *p, st, g->s.acc.as<unsigned long long>()));
     TC_CUDA(cudaMemcpyAsync(g->s.h_counts, g->s.acc.p, sizeof(unsigned long long) * 16, cudaMemcpyDeviceToHost, st));
     TC_CUDA(cudaStreamSynchronize(st));

@@ -1011,9 +1011,9 @@ __global__ void k_item_splits(const Item* __restrict__ items, uint32_t n, uint32
 }
 }  // namespace
 
-bool has_plan(const GraphStore& g, const Opts& o) {
+bool has_plan(const GraphStore& g, const Opts& o, uint32_t world) {
     for (auto& p : g.plans)
-        if (p.valid && p.key == o) return true;
+        if (p.valid && p.key == o && (!world || p.shard_world == world)) return true;
     return false;
 }
 

@@ -137,7 +137,7 @@ tc_status graph_create_sorted(uint32_t n, const uint64_t* d_keys, uint64_t m, cu
 
 // Enqueue one census on `st`; counts of classes 1..15 go to d_out16, index 0 is 0.  No host synchronisation and
 // no allocation: census_plan, called first, does both where the plan or the lists are not there yet.
-bool has_plan(const GraphStore& g, const Opts& o);
+bool has_plan(const GraphStore& g, const Opts& o, uint32_t world = 0);   // world: and its shards
 tc_status get_plan(GraphStore& g, const Opts& o, cudaStream_t st, Plan** out);
 // The plan and, for the triangle form of a large graph, its 16-bit lists: before census_enqueue.
 tc_status census_plan(GraphStore& g, const Opts& o, cudaStream_t st, Plan** out);
