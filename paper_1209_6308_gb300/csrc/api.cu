@@ -161,8 +161,8 @@ tc_status resolve_opts(const tc_options* in, const Opts* base, Opts* out) {
     if (o.schedule > TC_SCHED_LEARNED) return fail(TC_ERR_ARG, "unknown schedule");
     // the suffix form's hash takes 4 slots per entry, the union walk's 2 plus the sorted copy:
     // both fill about 70 KB of shared memory, three CTAs per SM
-    // the triangle form's CTAs hold a small hash (2 slots per staged entry) and few registers:
-    // eight per SM keep the most loads in flight
+    // the triangle form's CTAs hold a small hash (2 slots per staged entry) and few registers: eight per SM,
+    // as k_walk_warp's are (a kernel of fewer resident CTAs launches those: triangles.cu, walk16.cu)
     if (!o.chunk) {
         o.chunk = o.algo == TC_ALGO_UNION ? 4096u : 2048u;
         o.chunk_auto = true;

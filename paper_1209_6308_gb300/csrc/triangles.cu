@@ -49,11 +49,15 @@ __device__ __forceinline__ void load_graph(GraphDev& to, const GraphDev* from, i
     __syncwarp();
 }
 
+// Resident CTAs per SM; a single graph's launch has no more.  (CTAs beyond them start when others end and
+// find the counters run out, so their times say nothing of the walk's balance.)
+constexpr int kCtasTri = 6, kCtasOld = 5;
+
 template <bool OLD, int MODE>
 // 1024 batched graphs at 8 / 6 / 5 resident CTAs: 4.67 / 4.53 / 4.66 ms (8 spill 500 bytes).  The
 // 64-state census of scale 20 with 4 CTAs and 2048-entry chunks / 5 and 1024 / 8 and 512: 5.94 / 5.49 /
 // 5.46 ms (at the 32 registers of 8 CTAs, 4 resident: 6.32).
-__global__ void __launch_bounds__(kThreads, OLD ? 5 : 6) k_triangles(TriParams P) {
+__global__ void __launch_bounds__(kThreads, OLD ? kCtasOld : kCtasTri) k_triangles(TriParams P) {
     extern __shared__ __align__(16) unsigned char smem[];
     const uint32_t slots = 2u * P.chunk;
     uint32_t* sH = reinterpret_cast<uint32_t*>(smem);                 // [slots] CTA hash of L(b)
@@ -71,7 +75,7 @@ __global__ void __launch_bounds__(kThreads, OLD ? 5 : 6) k_triangles(TriParams P
     // prefixes: the path would only cost the kernel registers); the one-warp tier's prefixes
     // are below its degree bound, never long
     constexpr bool kLongWalk = MODE != kTriBatch;
-    if (P.phase && tid == 0) P.phase[3 * blockIdx.x] = tri_clock_ns();
+    if (P.phase) tri_stamp(P, 0, tri_clock_ns());
     for (int k = tid; k < kWarps * 64; k += kThreads) sHist[k] = 0u;
     if (OLD)
         for (int k = tid; k < 9 * 64; k += kThreads) sPerm[k] = P.perm_state[k];
@@ -168,7 +172,7 @@ __global__ void __launch_bounds__(kThreads, OLD ? 5 : 6) k_triangles(TriParams P
         __syncthreads();   // every thread has read s_item before thread 0 takes the next item
     }
 
-    if (P.phase && tid == 0) P.phase[3 * blockIdx.x + 1] = tri_clock_ns();
+    if (P.phase) tri_stamp(P, 1, tri_clock_ns());
 
     // ---------------------------------------------------------------- one warp per vertex
     uint32_t* wH = sWH + warp * kWarpSlots;
@@ -238,7 +242,7 @@ __global__ void __launch_bounds__(kThreads, OLD ? 5 : 6) k_triangles(TriParams P
     if (MODE == kTriSingle || cur_graph != 0xffffffffu) flush_warp_hist(myHist, ghist, lane);
     if (P.phase) {   // uniform over the CTA
         __syncthreads();
-        if (tid == 0) P.phase[3 * blockIdx.x + 2] = tri_clock_ns();
+        tri_stamp(P, 2, tri_clock_ns());
     }
 }
 
@@ -598,10 +602,12 @@ tc_status triangles_launch(const GraphDev& gd, const Opts& o, const Item* items,
     P.hist = d_hist64;
     P.vcost = d_vcost;
     P.phase = d_phase;
-    const unsigned grid = (unsigned)census_grid(o);
+    unsigned grid = (unsigned)census_grid(o);
+    P.stamps = grid;
     if (split && !is_old) return walk16_launch(P, split, grid, ctr + 4, st);
     const size_t smem = tri_smem(o.chunk, is_old);
     TC_TRY(tri_prepare(is_old ? 1 : 0, smem));
+    grid = std::min(grid, (unsigned)(sm_count() * (is_old ? kCtasOld : kCtasTri)));
     if (is_old) k_triangles<true, kTriSingle><<<grid, kThreads, smem, st>>>(P);
     else k_triangles<false, kTriSingle><<<grid, kThreads, smem, st>>>(P);
     TC_LAUNCH("k_triangles");

@@ -19,7 +19,8 @@ struct TriParams {
     unsigned long long* hist;     // 64 bins (triangle tricodes, or states with OLD); batched: graph g's at
                                   // hist + kBatchStride g
     unsigned long long* vcost;    // optional [n]: SM cycles per CTA-tier vertex b
-    unsigned long long* phase;    // optional [3 * gridDim]: globaltimer at start, end of items, end
+    unsigned long long* phase;    // optional [3 * stamps]: globaltimer at start, end of items, end per CTA of
+    uint32_t stamps;              // the option's grid; a smaller launch's CTAs fill several entries
     // batched launch: item.pad is the graph index, warp-tier blocks are (u0, u1, graph)
     const GraphDev* graphs;
     const uint4* wblocks;
@@ -46,6 +47,11 @@ __device__ __forceinline__ unsigned long long tri_clock_ns() {
     unsigned long long t;
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
     return t;
+}
+
+// Per-CTA times (tc_census_profile): slot 0, 1 or 2 of this CTA's entries.
+__device__ __forceinline__ void tri_stamp(const TriParams& P, uint32_t slot, unsigned long long t) {
+    for (uint32_t k = blockIdx.x + gridDim.x * threadIdx.x; k < P.stamps; k += gridDim.x * blockDim.x) P.phase[3 * k + slot] = t;
 }
 
 __device__ __forceinline__ uint32_t tri_hash(uint32_t x, int hb) { return (x * 2654435761u) >> (32 - hb); }

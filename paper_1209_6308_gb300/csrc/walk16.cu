@@ -434,16 +434,11 @@ struct Runner {
         __syncthreads();
         for (uint32_t k = tid; k < dirty; k += kT16) sH[k] = ~0u;
     }
-    // Per-CTA times (tc_census_profile): slot 0, 1 or 2 of every CTA of the option's grid, which may be
-    // larger than this launch's.
-    __device__ static void stamp(const TriParams& P, uint32_t slot, uint32_t grid, unsigned long long t) {
-        for (uint32_t k = blockIdx.x + gridDim.x * threadIdx.x; k < grid; k += gridDim.x * blockDim.x) P.phase[3 * k + slot] = t;
-    }
 };
 
-// Launch marks for tc_census_profile: the option's grid, and which of its times this launch writes.
+// Which of tc_census_profile's times this launch writes.
 struct Stamps {
-    uint32_t grid, start, items;
+    uint32_t start, items;
 };
 
 // The map's byte holds, for each of the four windows, two bits of the id there: dir(b, a) - 1, or 3
@@ -452,7 +447,7 @@ __global__ void __launch_bounds__(kT16, kCtas16) k_walk16(TriParams P, Stamps T)
     extern __shared__ __align__(16) unsigned char smem[];
     Shared16& S = *reinterpret_cast<Shared16*>(smem);
     const GraphDev& G = P.g;
-    if (P.phase && T.start) Runner::stamp(P, 0, T.grid, tri_clock_ns());
+    if (P.phase && T.start) tri_stamp(P, 0, tri_clock_ns());
     Flat& F = S.f;
     Runner R(P, F);
     const int tid = R.tid, warp = R.warp, lane = R.lane;
@@ -562,7 +557,7 @@ __global__ void __launch_bounds__(kT16, kCtas16) k_walk16(TriParams P, Stamps T)
         R.next_item(lb != 0u);
     }
     R.flush_all();
-    if (P.phase && T.items) Runner::stamp(P, 1, T.grid, tri_clock_ns());
+    if (P.phase && T.items) tri_stamp(P, 1, tri_clock_ns());
 }
 
 // The table walk: the pairs' whole prefixes as stored, 32-bit entries in aligned blocks of four,
@@ -573,7 +568,7 @@ __global__ void __launch_bounds__(kT16, kCtas16) k_walk_table(TriParams P, Stamp
     extern __shared__ __align__(16) unsigned char smem[];
     SharedTable& S = *reinterpret_cast<SharedTable*>(smem);
     const GraphDev& G = P.g;
-    if (P.phase && T.start) Runner::stamp(P, 0, T.grid, tri_clock_ns());
+    if (P.phase && T.start) tri_stamp(P, 0, tri_clock_ns());
     Flat& F = S.f;
     Runner R(P, F);
     const int tid = R.tid, warp = R.warp, lane = R.lane;
@@ -688,7 +683,7 @@ __global__ void __launch_bounds__(kT16, kCtas16) k_walk_table(TriParams P, Stamp
         R.next_item(lb != 0u);
     }
     R.flush_all();
-    if (P.phase && T.items) Runner::stamp(P, 1, T.grid, tri_clock_ns());
+    if (P.phase && T.items) tri_stamp(P, 1, tri_clock_ns());
 }
 
 // The small vertices' items and the one-warp vertices, a warp each.
@@ -697,7 +692,7 @@ __global__ void __launch_bounds__(kT16, kCtasWarp) k_walk_warp(TriParams P, Stam
     __shared__ uint8_t s_at[kW16][32];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const GraphDev& G = P.g;
-    if (P.phase && T.start) Runner::stamp(P, 0, T.grid, tri_clock_ns());
+    if (P.phase && T.start) tri_stamp(P, 0, tri_clock_ns());
     for (int k = lane; k < 64; k += 32) s_hist[warp][k] = 0u;
     __syncwarp();
     uint32_t* wH = s_hash[warp];
@@ -739,7 +734,7 @@ __global__ void __launch_bounds__(kT16, kCtasWarp) k_walk_warp(TriParams P, Stam
     }
     if (P.phase && T.items) {
         __syncthreads();
-        Runner::stamp(P, 1, T.grid, tri_clock_ns());
+        tri_stamp(P, 1, tri_clock_ns());
     }
     for (;;) {
         uint32_t vb = 0;
@@ -756,7 +751,7 @@ __global__ void __launch_bounds__(kT16, kCtasWarp) k_walk_warp(TriParams P, Stam
     flush_warp_hist(s_hist[warp], P.hist, lane);
     if (P.phase) {
         __syncthreads();
-        Runner::stamp(P, 2, T.grid, tri_clock_ns());
+        tri_stamp(P, 2, tri_clock_ns());
     }
 }
 
@@ -805,7 +800,7 @@ tc_status walk16_launch(const TriParams& P0, const uint32_t split[2], uint32_t g
     const unsigned sms = (unsigned)sm_count();
     const unsigned ctas = grid < sms * kCtas16 ? grid : sms * kCtas16;
     const uint32_t s1 = split[0], s2 = split[1];
-    Stamps T = {grid, 1u, s2 == s1};
+    Stamps T = {1u, s2 == s1};
     TriParams P = P0;
     if (s1) {
         P.ctr = ctr;
