@@ -150,7 +150,7 @@ tc_status tc_census_opts(tc_graph* g, void* stream, const tc_options* opt, tc_u1
  * counts of classes 1..15 to d_out16[1..15] (device memory, uint64) and 0 to d_out16[0].
  * The null count needs 128-bit arithmetic: obtain it with tc_null_count.  d_out16 must stay valid
  * until the stream reaches the end of the census.  The first call of a graph with given options makes
- * their plan, and a large graph's first plan of TC_ALGO_TRIANGLE also its 16-bit lists (52 B per vertex
+ * their plan, and a large graph's first plan of TC_ALGO_TRIANGLE also its 16-bit lists (48 B per vertex
  * with a neighbour and about 4 B per pair, kept with the graph): it allocates and synchronises `stream`.
  * Later calls only launch, and can be captured.  (A graph keeps the last four plans.) */
 tc_status tc_census_async(tc_graph* g, void* stream, const tc_options* opt, uint64_t* d_out16);

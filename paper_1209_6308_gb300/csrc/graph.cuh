@@ -68,7 +68,7 @@ struct GraphStore {
     DevBuf store, scratch;       // what the buffers below are carved from (not rec, blk16, cost)
     DevBuf off, adj, up, new_of_old;
     DevBuf ub, rp, vs, us;   // per upper pair tables (see GraphDev)
-    DevBuf rec, blk16;   // 16-bit lower lists (see GraphDev): rec holds rec, rec2 and n16 of the active vertices
+    DevBuf rec, blk16;   // 16-bit lower lists (see GraphDev): rec holds rec and rec2 of the active vertices
     bool no_lists16 = false;   // the device had no room for them since the last plan was made
     DevBuf ctr;        // census work counters (uint32 x 4)
     DevBuf acc;        // census accumulators (uint64 x 16)
@@ -96,7 +96,6 @@ struct GraphStore {
         d.rec = rec.as<uint4>();
         d.blk16 = blk16.as<uint4>();
         d.rec2 = rec.p ? d.rec + n_active : nullptr;
-        d.n16 = rec.p ? reinterpret_cast<const uint32_t*>(d.rec + 3ull * n_active) : nullptr;
         return d;
     }
 };

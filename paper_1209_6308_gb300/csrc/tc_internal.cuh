@@ -80,11 +80,10 @@ struct GraphDev {
     // of eight, the last block padded with kPad16; the segments' blocks follow each other.
     // rec[x] = (first block, the lengths of window 0's class 1 and 2 as 16-bit halves, the class-1
     // and class-2 entries of all of N[x]); rec2[2x], rec2[2x + 1] (x >= kWin16 only) = the 16-bit
-    // lengths of the segments from window 0's class 3 on.  n16[x] = entries in all segments.
-    const uint4* rec;       // [n_active], set where n16 is not 0
+    // lengths of the segments from window 0's class 3 on.
+    const uint4* rec;       // [n_active], set where the list is not empty
     const uint4* rec2;      // [2 n_active]
     const uint4* blk16;
-    const uint32_t* n16;    // [n_active]
 };
 constexpr uint32_t kWin16 = 1u << 15, kIds16 = 4u * kWin16, kPad16 = kWin16;
 

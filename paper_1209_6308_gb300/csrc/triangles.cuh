@@ -102,8 +102,7 @@ __device__ __forceinline__ uint32_t nth_set(uint32_t mask, bool mine, volatile u
 // a < b is in its range); else a hash.  One warp: a batch's pairs with long prefixes are walked
 // one after another by all lanes, and the lanes share the flattened (pair, position) range of
 // the others.  Returns the entries walked (warp-uniform).
-// REST: only the entries past c's 16-bit list (walk16.cu counted the others).
-template <bool OLD, bool MAP, bool LONGW, bool REST = false>
+template <bool OLD, bool MAP, bool LONGW>
 __device__ __forceinline__ uint32_t walk_pairs(const TriParams& P, const GraphDev& G, uint64_t bbase, uint64_t pb,
                                                uint32_t j0, uint32_t j1, const uint32_t* sH, const uint32_t* sO,
                                                int hb, uint32_t hmask, uint32_t ob, const uint8_t* sPerm,
@@ -148,11 +147,6 @@ __device__ __forceinline__ uint32_t walk_pairs(const TriParams& P, const GraphDe
         const uint32_t c = e_bc >> 2;
         uint64_t cb = ok ? off[c] : 0ull;
         uint32_t len = ok ? rp[pb + j] : 0u;
-        if (REST && ok) {
-            const uint32_t h = G.n16[c];
-            cb += h;
-            len -= h;
-        }
         uint32_t oc = (OLD && ok) ? P.old[c] : 0u;
         if (LONGW) {
             // pairs with long prefixes, one at a time over the whole warp: consecutive entries,

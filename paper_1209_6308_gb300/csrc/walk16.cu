@@ -55,8 +55,8 @@ struct Flat {
     uint8_t lanes[kW16][32];                    // walk_pairs' scratch
     uint32_t nblk[kW16], nseg[kW16];
     Item item;                                  // the next item and its vertex's list: offset, table index,
-    uint64_t base, table;                       // lower entries, entries in the 16-bit list
-    uint32_t lower, held, next;
+    uint64_t base, table;                       // lower entries
+    uint32_t lower, next;
 };
 
 struct Shared16 {
@@ -99,8 +99,8 @@ __global__ void k_count16(const uint64_t* __restrict__ off, const uint32_t* __re
 // one that counts the classes and one (from the caches) that places each entry behind the earlier
 // ones of its class; for the others a warp takes 32 vertices (rows.cuh) whose lists share its lanes,
 // an entry's place counted by one ballot per segment (one with entries past the windows goes alone).
-__global__ void __launch_bounds__(256) k_lists16(GraphDev g, uint32_t n, uint32_t n_wide, const uint32_t* __restrict__ first, uint4* rec,
-                                                 uint4* rec2, uint16_t* ids) {
+__global__ void __launch_bounds__(256) k_lists16(GraphDev g, uint32_t n, uint32_t n_wide, const uint32_t* __restrict__ n16,
+                                                 const uint32_t* __restrict__ first, uint4* rec, uint4* rec2, uint16_t* ids) {
     __shared__ uint8_t s_at[8][32];
     const uint32_t lane = threadIdx.x & 31, lt = (1u << lane) - 1u;
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
@@ -183,7 +183,7 @@ __global__ void __launch_bounds__(256) k_lists16(GraphDev g, uint32_t n, uint32_
     };
     for (uint64_t x = (blockIdx.x * (uint64_t)blockDim.x + threadIdx.x) >> 5; x < n_wide; x += stride >> 5) {
         const uint64_t base = g.off[x];
-        const uint32_t h = g.n16[x], low = g.up[x];
+        const uint32_t h = n16[x], low = g.up[x];
         if (!h) continue;
         const uint2 v = upper(x, base, low, (uint32_t)(g.off[x + 1] - base));
         long_list(x, base, h, first[x], low, v.x, v.y);
@@ -192,7 +192,7 @@ __global__ void __launch_bounds__(256) k_lists16(GraphDev g, uint32_t n, uint32_
         const bool ok = x0 + lane < n;
         const uint64_t vbase = ok ? g.off[x0 + lane] : 0ull;
         const uint32_t vdeg = ok ? (uint32_t)(g.off[x0 + lane + 1] - vbase) : 0u, vlow = ok ? g.up[x0 + lane] : 0u;
-        const uint32_t vh = ok ? g.n16[x0 + lane] : 0u, vf = ok ? first[x0 + lane] : 0u;
+        const uint32_t vh = ok ? n16[x0 + lane] : 0u, vf = ok ? first[x0 + lane] : 0u;
         const uint2 vu = vh ? upper(x0 + lane, vbase, vlow, vdeg) : make_uint2(0u, 0u);
         const uint32_t v1 = vu.x, v2 = vu.y;
         for_rows(vlow != vh ? 33u : vh, s_at[threadIdx.x >> 5],
@@ -281,7 +281,7 @@ struct Runner {
     Item ahead1, ahead2;               // thread 0 runs ahead: the next item, the one after it,
     uint32_t ahead3;                   // and the index of a third, so no item waits for that chain
     uint64_t nbase = 0, ntable = 0;
-    uint32_t nlower = 0, nheld = 0;
+    uint32_t nlower = 0;
     static constexpr uint32_t kNone = 0xffffffffu;
 
     __device__ Runner(const TriParams& p, Flat& f)
@@ -304,14 +304,12 @@ struct Runner {
         if (ahead1.u == kNone) return;
         nbase = P.g.off[ahead1.u];
         nlower = P.g.up[ahead1.u];
-        nheld = P.g.n16[ahead1.u];
         ntable = P.g.ub[ahead1.u];
     }
     __device__ void publish() {   // thread 0
         F.item = ahead1;
         F.base = nbase;
         F.lower = nlower;
-        F.held = nheld;
         F.table = ntable - nlower;
     }
     __device__ void run_ahead() {
@@ -397,9 +395,7 @@ struct Runner {
         for (uint32_t k = tid; k < n_rounds; k += kT16) F.start[k] = 0u;
     }
     // The general walk of an item's pairs [j0, j1): L(b)[c0, c1) in a hash, at most `room` bytes of it
-    // per pass, in the place of a map or table whose idle state is all ones.  REST: only the pairs'
-    // entries past their 16-bit lists.
-    template <bool REST>
+    // per pass, in the place of a table whose idle state is all ones.
     __device__ void hash_walk(void* at, uint32_t room, uint64_t bbase, uint64_t pb, uint32_t j0, uint32_t j1, uint32_t c0,
                               uint32_t c1) {
         uint32_t dirty = 0;
@@ -425,7 +421,7 @@ struct Runner {
                 uint32_t jb, g;
                 grab_pairs(&F.next, j1, lane, jb, g);
                 if (jb >= j1) break;
-                walked += walk_pairs<false, false, true, REST>(P, P.g, bbase, pb, jb, min(jb + g, j1), sH, nullptr, hb,
+                walked += walk_pairs<false, false, true>(P, P.g, bbase, pb, jb, min(jb + g, j1), sH, nullptr, hb,
                                                                hmask, 0u, nullptr, F.hist[warp], F.lanes[warp], lane);
                 if (walked >= kFlushElems) flush_all();
             }
@@ -442,7 +438,8 @@ struct Stamps {
 };
 
 // The map's byte holds, for each of the four windows, two bits of the id there: dir(b, a) - 1, or 3
-// for an id that is not in L(b).
+// for an id that is not in L(b).  All of L(b) is in the lists' id range:
+static_assert(kTableFrom <= kIds16, "k_walk16's vertices have their lower neighbours in the 16-bit lists");
 __global__ void __launch_bounds__(kT16, kCtas16) k_walk16(TriParams P, Stamps T) {
     extern __shared__ __align__(16) unsigned char smem[];
     Shared16& S = *reinterpret_cast<Shared16*>(smem);
@@ -460,18 +457,18 @@ __global__ void __launch_bounds__(kT16, kCtas16) k_walk16(TriParams P, Stamps T)
         const long long t0 = clock64();
         const uint32_t b = w.u;
         const uint64_t bbase = F.base, pb = F.table;   // table index of the pair (b, N[b][j]) is pb + j
-        const uint32_t lb = F.lower, held = F.held;
+        const uint32_t lb = F.lower;
         R.run_ahead();
-        for (uint32_t k = tid; k < held; k += kT16) {
+        for (uint32_t k = tid; k < lb; k += kT16) {
             const uint32_t e = G.adj[bbase + k], a = (e >> 2) & (kWin16 - 1u);
             // 3 -> dir - 1 in the two bits of the id's window
             const uint32_t clear = (4u - (e & 3u)) << (8u * (a & 3u) + 2u * (e >> 17));
             atomicAnd(reinterpret_cast<uint32_t*>(S.map) + (a >> 2), ~clear);
         }
         // threads per pair: one for each window of 16-bit ids below b (1, 2 or 4)
-        const uint32_t wb = min(b >> 15, 4u);
+        const uint32_t wb = b >> 15;
         const uint32_t ws = wb == 0u ? 0u : wb == 1u ? 1u : 2u;
-        for (uint32_t jb = w.j0; held && jb < w.j1; jb += kT16 >> ws) {
+        for (uint32_t jb = w.j0; lb && jb < w.j1; jb += kT16 >> ws) {
             // this thread's segments (its pair's in its window): their lengths and first blocks
             const uint32_t j = jb + (tid >> ws), win = tid & ((1u << ws) - 1u);
             uint32_t m1 = 0, m2 = 0, m3 = 0, f1 = 0, f2 = 0, f3 = 0, tag = 0;
@@ -550,9 +547,7 @@ __global__ void __launch_bounds__(kT16, kCtas16) k_walk16(TriParams P, Stamps T)
                     });
             }
         }
-        for (uint32_t k = tid; k < held; k += kT16) S.map[(G.adj[bbase + k] >> 2) & (kWin16 - 1u)] = 0xffu;
-        // L(b) past the map against the pairs' entries past their 16-bit lists
-        R.hash_walk<true>(S.map, kWin16, bbase, pb, w.j0, w.j1, held, lb);
+        for (uint32_t k = tid; k < lb; k += kT16) S.map[(G.adj[bbase + k] >> 2) & (kWin16 - 1u)] = 0xffu;
         if (P.vcost && tid == 0) atomicAdd(&P.vcost[b], (unsigned long long)(clock64() - t0));
         R.next_item(lb != 0u);
     }
@@ -676,7 +671,7 @@ __global__ void __launch_bounds__(kT16, kCtas16) k_walk_table(TriParams P, Stamp
                 }
             }
             for (uint32_t k = c0 + tid; k < c1; k += kT16) *slot(G.adj[bbase + k]) = 0xffffu;
-            if (!fits) R.hash_walk<false>(S.tab, sizeof(S.tab), bbase, pb, w.j0, w.j1, c0, c1);
+            if (!fits) R.hash_walk(S.tab, sizeof(S.tab), bbase, pb, w.j0, w.j1, c0, c1);
             __syncthreads();
         }
         if (P.vcost && tid == 0) atomicAdd(&P.vcost[b], (unsigned long long)(clock64() - t0));
@@ -769,14 +764,15 @@ bool walk16_takes(const GraphStore& g) {
 }
 
 tc_status lists16_build(GraphStore& g, cudaStream_t st) {
-    DevBuf blocks, first, total;
+    DevBuf n16, blocks, first, total;
     const uint32_t n = g.n_active;   // the others have no list
-    TC_TRY(g.rec.alloc_persistent((3ull * sizeof(uint4) + sizeof(uint32_t)) * n));   // rec, rec2 and n16
+    TC_TRY(g.rec.alloc_persistent(3ull * sizeof(uint4) * n));   // rec and rec2
+    TC_TRY(n16.alloc(sizeof(uint32_t) * n, st));
     TC_TRY(blocks.alloc(sizeof(uint32_t) * n, st));
     TC_TRY(first.alloc(sizeof(uint32_t) * n, st));
     const GraphDev gd = g.dev();
     TC_TRY(total.alloc(sizeof(uint32_t), st));
-    k_count16<<<grid_for(n, 256, 1u << 16), 256, 0, st>>>(gd.off, gd.adj, gd.up, n, const_cast<uint32_t*>(gd.n16),
+    k_count16<<<grid_for(n, 256, 1u << 16), 256, 0, st>>>(gd.off, gd.adj, gd.up, n, n16.as<uint32_t>(),
                                                           blocks.as<uint32_t>());
     TC_LAUNCH("k_count16");
     TC_TRY(scan_u32(blocks.as<uint32_t>(), first.as<uint32_t>(), n, total.as<uint32_t>(), st));
@@ -785,7 +781,7 @@ tc_status lists16_build(GraphStore& g, cudaStream_t st) {
     TC_CUDA(cudaStreamSynchronize(st));
     DevBuf blk;
     TC_TRY(blk.alloc_persistent(sizeof(uint4) * (n_blocks ? n_blocks : 1u)));
-    k_lists16<<<grid_lists(n, g.n_wide), 256, 0, st>>>(gd, n, g.n_wide, first.as<uint32_t>(), g.rec.as<uint4>(),
+    k_lists16<<<grid_lists(n, g.n_wide), 256, 0, st>>>(gd, n, g.n_wide, n16.as<uint32_t>(), first.as<uint32_t>(), g.rec.as<uint4>(),
                                                           g.rec.as<uint4>() + n, blk.as<uint16_t>());
     TC_LAUNCH("k_lists16");
     TC_CUDA(cudaStreamSynchronize(st));   // later censuses may come on other streams
