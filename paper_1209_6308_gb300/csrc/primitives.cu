@@ -30,7 +30,10 @@ constexpr int kSortWarps = kSortThreads / 32;
 constexpr int kSortPer = 16;
 constexpr int kSortTile = kSortThreads * kSortPer;
 constexpr int kPasses = 8;                      // of 8 bits
-constexpr uint32_t kPatience = 1u << 16;
+#ifndef TC_LOOKS   // a test build sets 1, so that tiles do give up
+#define TC_LOOKS (1u << 16)
+#endif
+constexpr uint32_t kPatience = TC_LOOKS;
 constexpr int kLook = 4;   // predecessors a sort tile looks at together
 
 // A tile's published sums: the value, and in the top bits which one it is.
