@@ -70,7 +70,7 @@ struct GraphStore {
     DevBuf ub, rp, vs, us;   // per upper pair tables (see GraphDev)
     DevBuf rec, blk16;   // 16-bit lower lists (see GraphDev): rec holds rec and rec2 of the active vertices
     bool no_lists16 = false;   // the device had no room for them since the last plan was made
-    DevBuf ctr;        // census work counters (uint32 x 4)
+    DevBuf ctr;        // work counters of the per-pair walks (uint32 x 4); the triangle form's are in tri
     DevBuf acc;        // census accumulators (uint64 x 16)
     DevBuf cost;       // optional per-vertex predicted cost (float x n) for the learned schedule
     DevBuf tri;        // triangle form: bulk sums and triangle tricode histogram (uint64 x 96), counters (uint32 x 8)
@@ -118,7 +118,7 @@ struct WaveReq {
     unsigned long long* out;
     uint32_t n_items, item_pre, warp_begin, warp_end, block_pre, pad;
 };
-// slices per wave launch; 32 descriptors (2.3 KB of static shared memory) keep three CTAs
+// slices per wave launch; 32 descriptors (4 KB of static shared memory) keep three CTAs
 // per SM at the default chunk
 constexpr uint32_t kMaxWave = 32;
 

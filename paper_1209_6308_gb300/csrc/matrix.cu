@@ -201,8 +201,8 @@ struct MaskedProduct {
 // way by TMA, a warp issues the products (tcgen05.mma, 128 x 256 x 32 each, accumulated in 256
 // columns of tensor memory), and four warps read the tile back, a row per lane, and add the
 // entries their masks select.  At n = 16384 a whole product takes 3.1 ms, 2.8 PFLOP/s; the triangle
-// of 003 at n = 16001 0.47 ms, half the L2's rate: the stages' 48 KB for 590 clocks of products come
-// from the L2.  (16-bit products would double both; 1-bit ones the tensor cores don't have.)  Every
+// of 003 at n = 16001 0.47 ms with the tensor pipe 65% busy and the L2 half: the stages' 48 KB for 590
+// clocks of products come from the L2.  (16-bit products would double both; 1-bit ones the tensor cores don't have.)  Every
 // wait is bounded; one that runs out sets *error and the
 // CTA ends without the sums.
 __global__ void __launch_bounds__(kThreadsM, 1) k_masked_product(const __grid_constant__ MaskedProduct P) {

@@ -17,10 +17,12 @@
 // range, so long and short prefixes share the lanes evenly and only the range's end is ragged.
 //
 // Census of R-MAT scale 20 / 26 (edge factor 16): 2.20 -> 1.60 ms / 391.6 -> 275.1 ms against the walk
-// of 32-bit entries alone.  At scale 20 k_walk16 keeps the shared-memory pipe 66% and the issue
-// slots 60% busy: 32 lookups at random ids cost 3.0 wavefronts (bank conflicts), which neither a
-// denser map (two bits per id: 2.6) nor a plain-shift map for window 0 (fewer instructions, same
-// time) turned into time.  CTAs of 128 or 512 threads, maps of 2^14 and 2^16 ids and 4 to 6 rounds in
+// of 32-bit entries alone.  At scale 20 no unit is full under k_walk16 (1.12 ms): the load/store data
+// pipe is 74% busy, 57% with shared memory (32 lookups at random ids cost 3.0 wavefronts), the issue slots
+// 53%, the L2 15%; per issue 4.2 warps wait for the L2 or DRAM, 3.3 for shared memory, 2.2 at a barrier, of
+// eight per scheduler, which registers and shared memory both limit.  A denser map (two bits per
+// id: 2.6 wavefronts) and a plain-shift map for window 0 (fewer instructions) each left the time as it
+// was: latency at this occupancy more than any pipe.  CTAs of 128 or 512 threads, maps of 2^14 and 2^16 ids and 4 to 6 rounds in
 // flight (spills) were slower.
 #include <cstring>
 
@@ -753,10 +755,11 @@ __global__ void __launch_bounds__(kT16, kCtasWarp) k_walk_warp(TriParams P, Stam
 }  // namespace
 
 // Against the general kernel (triangles.cu), a graph's first census, which makes the lists, and a later
-// one, in ms, this / that.  Taken: R-MAT 19 edge factor 16 (500 M entries walked, 65 per pair) 1.22 /
-// 1.39, later 0.84 / 1.16; R-MAT 20 e.f. 16 (1.2 G, 78) 2.31 / 2.54, 1.65 / 2.22; R-MAT 24 e.f. 16
-// (42 G, 160) 56.3 / 73.4, 47.4 / 70.1; G(2400, 0.5) (1.3 G, 594) 1.35 / 1.45, 0.88 / 1.31.  Not taken,
-// as the first census would lose: R-MAT 22 e.f. 8 (2.0 G, 60) 4.94 / 4.80, 3.34 / 4.28; R-MAT 18 e.f. 16
+// one, in ms, this / that.  Taken: R-MAT 19 edge factor 16 (500 M entries walked, 65 per pair) 1.18 /
+// 1.39, later 0.80 / 1.16; R-MAT 20 e.f. 16 (1.2 G, 78) 2.29 / 2.54, 1.62 / 2.22; R-MAT 24 e.f. 16
+// (42 G, 160) 56.5 / 73.4, 47.5 / 70.1; G(2400, 0.5) (1.3 G, 594) 1.11 / 1.45, 0.87 / 1.31.  Not taken,
+// as the first census would lose (this side with k_lists16 on fewer warps than long lists, so G(1600, 0.5)
+// may have come to gain since): R-MAT 22 e.f. 8 (2.0 G, 60) 4.94 / 4.80, 3.34 / 4.28; R-MAT 18 e.f. 16
 // (204 M, 54) 0.84 / 0.76, 0.53 / 0.57; Chung-Lu 9 M x 16 (3.8 G, 31) 17.4 / 13.4, 10.5 / 12.0; G(1600,
 // 0.5) (378 M, 394) 0.71 / 0.62, 0.33 / 0.48.
 bool walk16_takes(const GraphStore& g) {
