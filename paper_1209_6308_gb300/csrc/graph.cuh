@@ -96,6 +96,7 @@ struct GraphStore {
         d.rec = rec.as<uint4>();
         d.blk16 = blk16.as<uint4>();
         d.rec2 = rec.p ? d.rec + n_active : nullptr;
+        d.unused = 0;
         return d;
     }
 };

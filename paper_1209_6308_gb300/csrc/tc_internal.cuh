@@ -84,6 +84,7 @@ struct GraphDev {
     const uint4* rec;       // [n_active], set where the list is not empty
     const uint4* rec2;      // [2 n_active]
     const uint4* blk16;
+    uint64_t unused;        // 96 bytes: the records of a batch start on 32-byte sectors
 };
 constexpr uint32_t kWin16 = 1u << 15, kIds16 = 4u * kWin16, kPad16 = kWin16;
 
