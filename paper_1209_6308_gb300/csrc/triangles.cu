@@ -50,14 +50,21 @@ __device__ __forceinline__ void load_graph(GraphDev& to, const GraphDev* from, i
 }
 
 // Resident CTAs per SM; a single graph's launch has no more.  (CTAs beyond them start when others end and
-// find the counters run out, so their times say nothing of the walk's balance.)
-constexpr int kCtasTri = 6, kCtasOld = 5;
+// find the counters run out, so their times say nothing of the walk's balance.)  The packed one-warp
+// vertices need the registers of six; the items alone run at eight (32 registers, no spills), which hide
+// more of the latency of short lists, but are a launch more.  A graph takes the two from kItemsApart items
+// on, where that pays; one launch / two, ms: random graphs, 2^16 vertices of degree 60 (18 k items)
+// 0.276 / 0.282, 2^15 of 80 (31 k) 0.247 / 0.247, 2^16 of 100 (65 k) 0.532 / 0.510, 2^18 of 100 (258 k) 2.79 /
+// 2.45, 2^20 of 128 (1 M) 16.3 / 13.9; R-MAT 18 e.f. 16 (21 k) 0.537 / 0.533, R-MAT 20 e.f. 8 (52 k) 0.993 /
+// 0.950, R-MAT 22 e.f. 8 (131 k) 4.24 / 3.96; Chung-Lu 1 M x 16 (54 k) 1.079 / 1.034.
+constexpr int kCtasTri = 6, kCtasOld = 5, kCtasItems = 8;
+constexpr uint32_t kItemsApart = 1u << 15;
 
 template <bool OLD, int MODE>
 // 1024 batched graphs at 8 / 6 / 5 resident CTAs: 4.67 / 4.53 / 4.66 ms (8 spill 500 bytes).  The
 // 64-state census of scale 20 with 4 CTAs and 2048-entry chunks / 5 and 1024 / 8 and 512: 5.94 / 5.49 /
 // 5.46 ms (at the 32 registers of 8 CTAs, 4 resident: 6.32).
-__global__ void __launch_bounds__(kThreads, OLD ? kCtasOld : kCtasTri) k_triangles(TriParams P) {
+__global__ void __launch_bounds__(kThreads, OLD ? kCtasOld : MODE == kTriItems ? kCtasItems : kCtasTri) k_triangles(TriParams P) {
     extern __shared__ __align__(16) unsigned char smem[];
     const uint32_t slots = 2u * P.chunk;
     uint32_t* sH = reinterpret_cast<uint32_t*>(smem);                 // [slots] CTA hash of L(b)
@@ -68,20 +75,21 @@ __global__ void __launch_bounds__(kThreads, OLD ? kCtasOld : kCtasTri) k_triangl
     uint8_t* sPerm = reinterpret_cast<uint8_t*>(sHist + kWarps * 64);  // [9][64] OLD
     __shared__ uint32_t s_item, s_next;
     __shared__ uint8_t s_at[kWarps][32];   // walk_pairs' scratch
-    __shared__ GraphDev s_g[MODE == kTriSingle ? 1 : kWarps];
+    constexpr bool kOne = MODE == kTriSingle || MODE == kTriItems;
+    __shared__ GraphDev s_g[kOne ? 1 : kWarps];
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     // the whole-warp walk of long prefixes, except in a batch of graphs (small graphs, short
     // prefixes: the path would only cost the kernel registers); the one-warp tier's prefixes
     // are below its degree bound, never long
     constexpr bool kLongWalk = MODE != kTriBatch;
-    if (P.phase) tri_stamp(P, 0, tri_clock_ns());
+    if (P.marks & 1u) tri_stamp(P, 0, tri_clock_ns());
     for (int k = tid; k < kWarps * 64; k += kThreads) sHist[k] = 0u;
     if (OLD)
         for (int k = tid; k < 9 * 64; k += kThreads) sPerm[k] = P.perm_state[k];
     __syncthreads();
     uint32_t* myHist = sHist + warp * 64;
-    const GraphDev& G = MODE == kTriSingle ? P.g : s_g[warp];   // several graphs: the warp's
+    const GraphDev& G = kOne ? P.g : s_g[warp];   // several graphs: the warp's
     unsigned long long* ghist = P.hist;
     uint32_t cur_graph = 0xffffffffu;   // batched: the graph whose counts the warp's bins hold
     // batched: move to graph gi, flushing this warp's bins to the graph they belong to
@@ -172,7 +180,11 @@ __global__ void __launch_bounds__(kThreads, OLD ? kCtasOld : kCtasTri) k_triangl
         __syncthreads();   // every thread has read s_item before thread 0 takes the next item
     }
 
-    if (P.phase) tri_stamp(P, 1, tri_clock_ns());
+    if (P.marks & 2u) tri_stamp(P, 1, tri_clock_ns());
+    if (MODE == kTriItems) {
+        flush_warp_hist(myHist, ghist, lane);
+        return;
+    }
 
     // ---------------------------------------------------------------- one warp per vertex
     uint32_t* wH = sWH + warp * kWarpSlots;
@@ -240,7 +252,7 @@ __global__ void __launch_bounds__(kThreads, OLD ? kCtasOld : kCtasTri) k_triangl
         }
     }
     if (MODE == kTriSingle || cur_graph != 0xffffffffu) flush_warp_hist(myHist, ghist, lane);
-    if (P.phase) {   // uniform over the CTA
+    if (P.marks & 4u) {   // uniform over the CTA
         __syncthreads();
         tri_stamp(P, 2, tri_clock_ns());
     }
@@ -544,7 +556,7 @@ __global__ void k_tri_collect(TriCollect a, Table64 T) {
     for (uint32_t k = t; k < kBatchStride; k += blockDim.x) sc[k] = 0ull;
 }
 
-std::atomic<int> g_tri_limit[4][64] = {};   // dynamic shared memory the form's kernel was set to, per device
+std::atomic<int> g_tri_limit[5][64] = {};   // dynamic shared memory the form's kernel was set to, per device
 
 size_t tri_smem(uint32_t chunk, bool old) {
     const size_t slots = 2ull * chunk;
@@ -552,15 +564,16 @@ size_t tri_smem(uint32_t chunk, bool old) {
            (old ? 9 * 64 : 0);
 }
 
-// form: 0 single graph, 1 caller-id states (64-state census), 2 batched, 3 serving wave
+// form: 0 single graph, 1 caller-id states (64-state census), 2 batched, 3 serving wave, 4 a single graph's items
 tc_status tri_prepare(int form, size_t smem) {
     int dev = 0;
     TC_CUDA(cudaGetDevice(&dev));
     std::atomic<int>& limit = g_tri_limit[form][dev & 63];
     int lim = limit.load();
     if (!lim) {
-        const void* fns[4] = {(const void*)k_triangles<false, kTriSingle>, (const void*)k_triangles<true, kTriSingle>,
-                              (const void*)k_triangles<false, kTriBatch>, (const void*)k_triangles<false, kTriWave>};
+        const void* fns[5] = {(const void*)k_triangles<false, kTriSingle>, (const void*)k_triangles<true, kTriSingle>,
+                              (const void*)k_triangles<false, kTriBatch>, (const void*)k_triangles<false, kTriWave>,
+                              (const void*)k_triangles<false, kTriItems>};
         int optin = 0;
         TC_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
         cudaFuncAttributes fa;
@@ -604,8 +617,17 @@ tc_status triangles_launch(const GraphDev& gd, const Opts& o, const Item* items,
     P.phase = d_phase;
     unsigned grid = (unsigned)census_grid(o);
     P.stamps = grid;
+    P.marks = d_phase ? 7u : 0u;
     if (split && !is_old) return walk16_launch(P, split, grid, ctr + 4, st);
     const size_t smem = tri_smem(o.chunk, is_old);
+    if (!is_old && n_items >= kItemsApart) {
+        TC_TRY(tri_prepare(4, smem));
+        P.marks = d_phase ? 3u : 0u;
+        k_triangles<false, kTriItems><<<std::min(grid, (unsigned)(sm_count() * kCtasItems)), kThreads, smem, st>>>(P);
+        TC_LAUNCH("k_triangles (items)");
+        P.marks = d_phase ? 4u : 0u;
+        P.n_items = 0;
+    }
     TC_TRY(tri_prepare(is_old ? 1 : 0, smem));
     grid = std::min(grid, (unsigned)(sm_count() * (is_old ? kCtasOld : kCtasTri)));
     if (is_old) k_triangles<true, kTriSingle><<<grid, kThreads, smem, st>>>(P);

@@ -21,6 +21,7 @@ struct TriParams {
     unsigned long long* vcost;    // optional [n]: SM cycles per CTA-tier vertex b
     unsigned long long* phase;    // optional [3 * stamps]: globaltimer at start, end of items, end per CTA of
     uint32_t stamps;              // the option's grid; a smaller launch's CTAs fill several entries
+    uint32_t marks;               // k_triangles: which of the times this launch writes (bits 0, 1, 2)
     // batched launch: item.pad is the graph index, warp-tier blocks are (u0, u1, graph)
     const GraphDev* graphs;
     const uint4* wblocks;
@@ -72,7 +73,8 @@ constexpr uint32_t kBatchStride = 96;
 
 // launch modes: one graph; a batch of graphs (items tagged with the graph, blocks (u0, u1, g));
 // a serving wave (slices of several requests, descriptors in global memory)
-enum { kTriSingle = 0, kTriBatch = 1, kTriWave = 2 };
+// (kTriItems: one graph's CTA items alone)
+enum { kTriSingle = 0, kTriBatch = 1, kTriWave = 2, kTriItems = 3 };
 
 // index r of the last request whose prefix is <= i (prefixes ascend from 0)
 template <typename F>
