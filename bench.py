@@ -113,6 +113,47 @@ def bytes_alg_8d(n: int, info: dict) -> int:
     return 8 * (n + 1) + 8 * info["e_sym"] + 4 * info["sum_dv_upper"] + 16 * info["e_sym"] + 128
 
 
+def bytes_census64(n: int, info: dict) -> int:
+    """Bytes the 64-state census's kernels read and write: per list entry 16 B to key it (its word, the
+    neighbour's caller id, the key), 16 B per pass of the sort by two caller ids, 8 B to count its digits and
+    8 B for the wedges; the triangle walk's tables, and 4 B per entry it walks."""
+    bits = max(1, (n - 1).bit_length())
+    passes = (2 * bits + 7) // 8
+    return 2 * info["e_sym"] * (16 + 16 * passes + 8 + 8) + 32 * (n + 1) + 20 * info["e_sym"] + 4 * info["sum_tri_walk"]
+
+
+def entries_in_16_bits(tc, torch, g) -> int:
+    """Of the entries the triangle form walks, those the 16-bit walk reads as 16-bit ids: for each vertex c
+    with h lower neighbours below id b* = min(2^17, the vertices of degree above 256), h (h - 1) / 2."""
+    off_p, adj_p, _ = tc.tc_graph_device_csr(g.handle)
+    e2 = 2 * g.stats()["e_sym"]
+
+    class Words:
+        def __init__(self, ptr, count, kind):
+            self.__cuda_array_interface__ = {"data": (ptr, False), "shape": (count,), "typestr": kind, "version": 3}
+
+    off = torch.as_tensor(Words(off_p, g.n + 1, "<i8"), device="cuda")
+    limit = min(1 << 17, int(((off[1:] - off[:-1]) > 256).sum()))
+    total, row, chunk = 0, 0, 1 << 27
+    host = off.cpu()
+    adj = torch.as_tensor(Words(adj_p, e2, "<i4"), device="cuda")
+    while row < g.n:
+        last = int(torch.searchsorted(host, host[row] + chunk, right=True)) - 1     # rows [row, last): at most a chunk
+        last = min(max(last, row + 1), g.n)
+        b, e = int(host[row]), int(host[last])
+        if e > b:
+            deg = off[row + 1:last + 1] - off[row:last]
+            ids = (adj[b:e].to(torch.int64) & 0xFFFFFFFF) >> 2
+            own = torch.repeat_interleave(torch.arange(row, last, device="cuda"), deg)
+            seen = torch.zeros(e - b + 1, dtype=torch.int64, device="cuda")
+            torch.cumsum((ids < own.clamp(max=limit)).to(torch.int64), 0, out=seen[1:])
+            h = seen[off[row + 1:last + 1] - b] - seen[off[row:last] - b]
+            total += int((h * (h - 1) // 2).sum())
+            del ids, own, seen, h, deg
+        row = last
+    return total
+
+
 def dist_env():
     return int(os.environ.get("RANK", 0)), int(os.environ.get("WORLD_SIZE", 1)), int(os.environ.get("LOCAL_RANK", 0))
 
@@ -365,7 +406,7 @@ def batched_comparison(tc, torch, sh, st, trials):
     return res
 
 
-def learned_comparison(tc, g, stream, model, info, reps, algo):
+def learned_comparison(tc, g, stream, model, info, reps, algo, in16):
     """Cost model trained on R-MAT scales 18-22 (seeds 18-22) from cycles the plain census of the
     same kernel form measures, attached to the bench graph: census time with the plain and the
     learned schedule (identical counts required), each arm's roofline, and the held-out
@@ -382,8 +423,8 @@ def learned_comparison(tc, g, stream, model, info, reps, algo):
             "speedup": plain_ms / learned_ms, "counts_identical": plain_c == learned_c,
             "balance_plain": bal_plain, "balance_learned": bal_learned,
             "plain_arcs_per_s": None, "learned_arcs_per_s": None,
-            "roofline_plain": form_roofline(tc, g.n, g.stats(), algo, plain_ms),
-            "roofline_learned": form_roofline(tc, g.n, g.stats(), algo, learned_ms),
+            "roofline_plain": form_roofline(tc, g.n, g.stats(), algo, plain_ms, in16),
+            "roofline_learned": form_roofline(tc, g.n, g.stats(), algo, learned_ms, in16),
             "heldout_rms_log_cycle_error": {"model": q["rms_log_err_model"], "degree": q["rms_log_err_degree"],
                                             "vertices": q["vertices"]}}
 
@@ -611,9 +652,9 @@ def census64_comparison(tc, torch, sh, scale, steps=3):
     ms = statistics.median(times)
     return {"workload": f"rmat{scale}_ef16_r20_seed{scale}", "n": n, "arcs": len(s), "ms": ms,
             "arcs_per_s": len(s) / (ms * 1e-3), "fold_equals_census16": fold == c16,
-            "roofline": dict(roofline_hbm(bytes_alg_8d(n, info), ms, "census64 (sort, wedges, triangle walk)", None,
-                                          "issue"),
-                             note="bytes: the scope formula of the 16-class census (each pair streams its v list)")}
+            "roofline": dict(roofline_hbm(bytes_census64(n, info), ms, "census64 (sort, wedges, triangle walk)", None,
+                                          "latency"),
+                             note="bytes its kernels read and write: keys, sort passes, wedges, 4 B per entry walked")}
 
 
 def matrix_comparison(tc, torch, sh, steps=3):
@@ -671,17 +712,17 @@ def census_launches(tc, g, n, info, algo) -> int:
     return 4 + table
 
 
-def form_roofline(tc, n, info, algo, ms):
+def form_roofline(tc, n, info, algo, ms, in16=0):
     """Roofline of one census.  `bytes_alg_per_launch` is what the kernel form itself must read
-    (tc_graph_info: the triangle form's or the suffix form's count; the scope contract's count
-    for the union walk, which reads what it describes), so `frac` compares the form with
-    streaming its own data at copy speed.  The scope contract's count (every pair streams its
+    (tc_graph_info: the triangle form's or the suffix form's count, less 2 B for each of the `in16`
+    entries that the walk reads as 16-bit ids; the scope contract's count for the union walk, which reads
+    what it describes), so `frac` compares the form with streaming its own data at copy speed.  The scope contract's count (every pair streams its
     v list, the paper's walk) is given beside it as `contract_*`: a form that skips most of
     that reading can exceed 1 there."""
     kernel = {tc.TC_ALGO_TRIANGLE: triangle_kernel(info), tc.TC_ALGO_SUFFIX: "k_census (suffix)"}.get(algo, "k_census (union)")
     b8d = bytes_alg_8d(n, info)
     own = {tc.TC_ALGO_TRIANGLE: info["bytes_alg_tri"], tc.TC_ALGO_SUFFIX: info["bytes_alg"]}.get(algo, b8d)
-    r = roofline_hbm(own, ms, kernel, None, "issue")
+    r = roofline_hbm(own - 2 * in16, ms, kernel, None, "latency" if kernel == "k_walk16" else "issue")
     r["contract_bytes_per_launch"] = b8d
     r["contract_achieved"] = b8d / (ms * 1e-3) / 1e9
     r["contract_frac"] = r["contract_achieved"] / r["peak"]
@@ -703,8 +744,9 @@ def medium_section(tc, torch, stream, steps=5):
         for algo in (tc.TC_ALGO_TRIANGLE, tc.TC_ALGO_SUFFIX, tc.TC_ALGO_UNION):
             ms, c = learned.census_ms(g, {"algo": algo}, stream, reps=steps if algo else 3)
             counts[algo] = c
+            in16 = entries_in_16_bits(tc, torch, g) if algo == tc.TC_ALGO_TRIANGLE and triangle_kernel(info) == "k_walk16" else 0
             out[FORM_NAMES[algo]] = {"ms": ms, "arcs_per_s": len(s) / (ms * 1e-3),
-                                     "roofline": form_roofline(tc, n, info, algo, ms)}
+                                     "roofline": form_roofline(tc, n, info, algo, ms, in16)}
     c = counts[tc.TC_ALGO_TRIANGLE]
     out["forms_agree"] = all(v == c for v in counts.values())
     c[0] = tc.tc_null_count(n, c)
@@ -813,13 +855,16 @@ def run_gpu(args):
             dist.destroy_process_group()
         return 0
 
+    in16 = 0
+    if algo == tc.TC_ALGO_TRIANGLE and triangle_kernel(info) == "k_walk16":
+        in16 = entries_in_16_bits(tc, torch, g)
     learned_line, model = None, None
     if not args.no_learned:
         from paper_1209_6308_gb300 import learned
         log("training the cost model")
         model, minfo = learned.train_cost_model(scales=(18, 19, 20, 21, 22), steps=800, stream=sh, options=opts)
         log(f"cost model trained: {minfo}")
-        learned_line = learned_comparison(tc, g, stream, model, minfo, args.learned_reps, algo)
+        learned_line = learned_comparison(tc, g, stream, model, minfo, args.learned_reps, algo, in16)
         learned_line["kernel_form"] = args.algo
         learned_line["plain_arcs_per_s"] = arcs / (learned_line["plain_ms"] * 1e-3)
         learned_line["learned_arcs_per_s"] = arcs / (learned_line["learned_ms"] * 1e-3)
@@ -870,13 +915,13 @@ def run_gpu(args):
 
     kernel = triangle_kernel(info) if algo == tc.TC_ALGO_TRIANGLE else "k_census"
     traffic = stored_traffic(WORKLOAD["name"], kernel)
-    roof = form_roofline(tc, n, info, algo, ms)
+    roof = form_roofline(tc, n, info, algo, ms, in16)
     roof["traffic"] = traffic
-    roof["note"] = ("bytes_alg_per_launch = what this kernel form reads (tc_graph_info bytes_alg_tri: "
-                    "32(n+1) + 60 E + 4 sum_tri_walk + 1280); contract_* = the scope formula 8(n+1) + 8 E + "
-                    "sum over upper pairs (4 d_v + 16) + 128 (each pair streams N[v], the paper's walk), which "
-                    "this form does not read; the walk of 16-bit lists reads half of the 4 B per walked entry; it is "
-                    "bound by shared-memory lookups (bank conflicts) and instruction issue (ncu)")
+    roof["note"] = ("bytes_alg_per_launch = what this kernel form reads (32(n+1) + 60 E + 4 B per entry walked + 1280, "
+                    "but 2 B for the entries_16bit the walk reads as 16-bit ids); contract_* = the scope formula "
+                    "8(n+1) + 8 E + sum over upper pairs (4 d_v + 16) + 128 (each pair streams N[v], the paper's walk), "
+                    "which this form does not read; no unit is full: latency at 32 warps per SM (ncu, scale 20)")
+    roof["entries_walked"], roof["entries_16bit"] = info["sum_tri_walk"], in16
     line = {
         "metric": METRIC, "value": job_value(arcs, ms),
         "unit": "arcs/s", "n_gpus": world, "steps": args.steps, "warmup": args.warmup, "ms_per_step": ms,
