@@ -699,12 +699,13 @@ def triangle_kernel(info) -> str:
 
 
 def census_launches(tc, g, n, info, algo) -> int:
-    """Kernels of one census: k_census, or k_pair_bulk, the walk and k_tri_fold; the 16-bit walk is
+    """Kernels of one census: k_census, or k_pair_bulk, the walk and k_tri_fold; the general walk is one
+    launch, or two from 2^15 CTA items on; the 16-bit walk is
     k_walk16, k_walk_table (only if vertices past id 2^17 have more than 256 neighbours) and k_walk_warp."""
     if algo != tc.TC_ALGO_TRIANGLE:
         return 1
     if triangle_kernel(info) == "k_triangles":
-        return 3
+        return 3 + (int(tc.tc_census_shard_bounds(g, 1, options={"algo": algo})[1][0]) >= 1 << 15)
     import numpy as np
     off = np.zeros(n + 1, np.uint64)
     tc.load().tc_graph_export_csr(g, off.ctypes.data, None, None)
