@@ -30,3 +30,20 @@ def test_entries_read_as_16_bit_ids(name):
     assert got == int(position[lower & (b < limit)].sum()) > 0
     whole = bench.form_roofline(tc, n, info, tc.TC_ALGO_TRIANGLE, 1.0)["bytes_alg_per_launch"]
     assert bench.form_roofline(tc, n, info, tc.TC_ALGO_TRIANGLE, 1.0, got)["bytes_alg_per_launch"] == whole - 2 * got
+
+
+@pytest.mark.parametrize("name,launches", [("small", 3), ("items", 4), ("dense", 4)])
+def test_launches_of_a_census(name, launches):
+    """One walk, a walk whose 2^15 items and more have a launch of their own, and the 16-bit walk without a
+    vertex past its table's first id."""
+    def random(n, degree):
+        rng = np.random.default_rng(n)
+        return n, *(rng.integers(0, n, n * degree // 2).astype(np.uint32) for _ in range(2))
+
+    n, s, d = {"small": lambda: random(1 << 12, 32), "items": lambda: random(60_000, 100),
+               "dense": lambda: graphgen.gnp(2400, 0.5, seed=2400)}[name]()
+    with tc.Graph.from_arcs(n, s, d) as g:
+        info = g.stats()
+        assert (bench.triangle_kernel(info) == "k_walk16") == (name == "dense")
+        assert bench.census_launches(tc, g.handle, n, info, tc.TC_ALGO_TRIANGLE) == launches
+        assert bench.census_launches(tc, g.handle, n, info, tc.TC_ALGO_SUFFIX) == 1
