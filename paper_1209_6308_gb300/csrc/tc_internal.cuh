@@ -126,7 +126,8 @@ int sm_count();
 // CTAs of 256 threads for a kernel over n lists that gives each of at most `wide` longer ones a warp
 // and lets a warp's lanes share 32 shorter ones: a thread per list, and where that is few, a warp per
 // longer list up to eight CTAs per SM.  (A thread per list alone: a dense graph of 2400 vertices has its
-// 2400 lists walked by ten CTAs.)
+// 2400 lists walked by ten CTAs.  Builds of G(2400, 0.5) / G(4096, 0.9) / G(16384, 0.1) 1.49 / 4.86 / 6.20 ms
+// so, with this 0.65 / 1.78 / 4.01; R-MAT 20, whose grid is by lists either way, 3.45.)
 inline unsigned grid_lists(uint64_t n, uint64_t wide) {
     const unsigned by_list = grid_for(n, 256, 1u << 16), by_warp = grid_for(32ull * wide, 256, 8u * (unsigned)sm_count());
     return by_list > by_warp ? by_list : by_warp;
